@@ -274,14 +274,14 @@ static void inner_edge(double ci, double co, double &offset, double &slope, doub
     length = 2.0 / std::fabs(ci);
 }
 
-template <typename T>
-static AdjProj<T> adj_proj(const ProjGeom &g)
+AdjConst adj_const(const ProjGeom &g)
 {
-    double jc[4] = {g.jc0, 0, 0, 0}, kc[4] = {g.kc0, 0, 0, 0}, bu[4] = {g.u0, 0, 0, 0}, bv[4] = {g.v0, 0, 0, 0};
-    jc[1 + g.m] += g.jP; jc[1 + g.u] += g.jU; jc[1 + g.v] += g.jV;
-    kc[1 + g.m] += g.kP; kc[1 + g.u] += g.kU; kc[1 + g.v] += g.kV;
-    bu[1 + g.m] += g.up; bu[1 + g.u] -= 1.0;
-    bv[1 + g.m] += g.vp; bv[1 + g.v] -= 1.0;
+    AdjConst c = {};
+    c.jc[0] = g.jc0; c.kc[0] = g.kc0; c.bu[0] = g.u0; c.bv[0] = g.v0;
+    c.jc[1 + g.m] += g.jP; c.jc[1 + g.u] += g.jU; c.jc[1 + g.v] += g.jV;
+    c.kc[1 + g.m] += g.kP; c.kc[1 + g.u] += g.kU; c.kc[1 + g.v] += g.kV;
+    c.bu[1 + g.m] += g.up; c.bu[1 + g.u] -= 1.0;
+    c.bv[1 + g.m] += g.vp; c.bv[1 + g.v] -= 1.0;
     // the two enumeration orders: outer k / inner j, and outer j / inner k
     double au[2], lu[2], av[2], lv[2];
     int no[2], ni[2];
@@ -297,21 +297,37 @@ static AdjProj<T> adj_proj(const ProjGeom &g)
         ni[t] = points_in(std::min(std::min(Lu, Lv), 2.0 * hi));
     }
     const int t = (no[1] * ni[1] < no[0] * ni[0]) ? 1 : 0;
-    const bool outer_j = t == 1;
+    c.outer_j = t == 1;
+    for (int i = 0; i < 4; ++i) {
+        c.oc[i] = c.outer_j ? c.jc[i] : c.kc[i];
+        c.ic[i] = c.outer_j ? c.kc[i] : c.jc[i];
+    }
+    c.uo = c.outer_j ? g.uj : g.uk; c.ui = c.outer_j ? g.uk : g.uj;
+    c.vo = c.outer_j ? g.vj : g.vk; c.vi = c.outer_j ? g.vk : g.vj;
+    c.ho = c.outer_j ? g.hj : g.hk;
+    c.au = au[t]; c.lu = lu[t]; c.av = av[t]; c.lv = lv[t];
+    c.no = no[t]; c.ni = ni[t];
+    return c;
+}
+
+template <typename T>
+static AdjProj<T> adj_proj(const ProjGeom &g)
+{
+    const AdjConst c = adj_const(g);
     AdjProj<T> a;
     for (int i = 0; i < 4; ++i) {
-        a.oc[i] = (T)(outer_j ? jc[i] : kc[i]);
-        a.ic[i] = (T)(outer_j ? kc[i] : jc[i]);
-        a.bu[i] = (T)bu[i];
-        a.bv[i] = (T)bv[i];
+        a.oc[i] = (T)c.oc[i];
+        a.ic[i] = (T)c.ic[i];
+        a.bu[i] = (T)c.bu[i];
+        a.bv[i] = (T)c.bv[i];
     }
-    a.uo = (T)(outer_j ? g.uj : g.uk); a.ui = (T)(outer_j ? g.uk : g.uj);
-    a.vo = (T)(outer_j ? g.vj : g.vk); a.vi = (T)(outer_j ? g.vk : g.vj);
-    a.ho = (T)(outer_j ? g.hj : g.hk);
-    a.au = (T)au[t]; a.lu = (T)lu[t]; a.av = (T)av[t]; a.lv = (T)lv[t];
+    a.uo = (T)c.uo; a.ui = (T)c.ui;
+    a.vo = (T)c.vo; a.vi = (T)c.vi;
+    a.ho = (T)c.ho;
+    a.au = (T)c.au; a.lu = (T)c.lu; a.av = (T)c.av; a.lv = (T)c.lv;
     a.step = (T)g.step;
-    a.shape = (no[t] <= 3 && ni[t] <= 3) ? 16 * no[t] + ni[t] : 0;
-    a.order = no[t] | (ni[t] << 8) | ((outer_j ? 1 : 0) << 16);
+    a.shape = (c.no <= 3 && c.ni <= 3) ? 16 * c.no + c.ni : 0;
+    a.order = c.no | (c.ni << 8) | ((c.outer_j ? 1 : 0) << 16);
     return a;
 }
 
@@ -407,7 +423,7 @@ static void free_handle(tt_handle *h)
 {
     if (!h) return;
     cudaFree(h->geo); cudaFree(h->tmaps); cudaFree(h->B64); cudaFree(h->Bp); cudaFree(h->cpad); cudaFree(h->gpad);
-    cudaFree(h->G); cudaFree(h->partials); cudaFree(h->loss_dev); cudaFree(h->red);
+    cudaFree(h->G); cudaFree(h->Qm); cudaFree(h->F64); cudaFree(h->FB); cudaFree(h->mode_org); cudaFree(h->FM); cudaFree(h->order); cudaFree(h->slots); cudaFree(h->partials); cudaFree(h->loss_dev); cudaFree(h->red);
     cudaFree(h->hc); cudaFree(h->hI); cudaFree(h->hW); cudaFree(h->hg);
     for (cudaEvent_t e : h->chunk_ready) cudaEventDestroy(e);
     if (h->copy_stream) cudaStreamDestroy(h->copy_stream);
@@ -502,7 +518,7 @@ static void plan_forward(tt_handle *h)
         fits = fits && g.st_rv <= kStMaxRv && g.st_ru <= 256;
         cap = std::max(cap, (long long)((g.st_ru * g.st_rv + 1) & ~1));
     }
-    const long long bytes = (long long)kStRing * cap * 16 * 4 + (long long)h->CP * 16 * 4 + 128;
+    const long long bytes = (long long)kStRing * cap * 16 * 4 + (long long)h->CP * (16 + 16) * 4 + 128;
     if (!fits || bytes > kStMaxSmem) return;
     h->tmaps_host.resize(h->S);
     for (int s = 0; s < h->S; ++s)
@@ -549,6 +565,14 @@ template <typename T>
 static tt_status adjoint_impl(tt_handle *h, const T *R, T *g)
 {
     if (bad_ptr(R) || bad_ptr(g)) return invalid("tt_adjoint: device pointers must be non-null and 16-byte aligned");
+    if constexpr (std::is_same<T, float>::value) {
+        // the modes are the segments and R already has their row layout:
+        // nothing to contract
+        if (h->R && h->q_identity && h->R == 4 * h->R4) {
+            TT_CUDA(launch_adjoint_modes(h, R, g, false), "adjoint");
+            return TT_OK;
+        }
+    }
     return with_storage<T>(h, [&]<typename S>() -> tt_status {
         TT_CUDA((launch_backcontract<T, S>(h, R)), "backcontract");
         TT_CUDA((launch_adjoint<T, S>(h, g)), "adjoint");
@@ -570,7 +594,7 @@ struct ZeroVolume {
     {
         if (on) {
             h->zero_volume = true;
-            h->n_fwd_ctas = forward_ctas(h, false);
+            if (!h->fwd_modes) h->n_fwd_ctas = forward_ctas(h, false);
         }
     }
     ~ZeroVolume()
@@ -773,10 +797,24 @@ tt_status tt_create(const tt_problem *P, tt_precision prec, void *stream, tt_han
     }
     ALLOC(h->gpad, es * h->nvox() * h->KP);
     ALLOC(h->G, es * h->npix() * h->KP);
+    plan_modes(h);
+    if (h->R) {
+        ALLOC(h->Qm, sizeof(float) * h->CP * kModeQ);
+        if (!h->q_identity) ALLOC(h->F64, sizeof(double) * h->S * h->R * h->K);
+        ALLOC(h->FB, sizeof(float) * mode_operand_floats(h));
+        ALLOC(h->mode_org, sizeof(ModeOrigin) * h->S);
+        plan_mode_forward(h);
+        if (h->slot_floats) {
+            ALLOC(h->FM, sizeof(float) * 2 * h->S * modes_m(h->R) * h->KP);
+            ALLOC(h->order, sizeof(int) * h->S);
+            ALLOC(h->slots, sizeof(float) * (h->chunk * h->slot_floats + h->slots1));
+        }
+        h->fwd_modes = h->slots != nullptr;
+    }
     plan_forward(h);
     h->fwd_staged = false;   // the tap-pair march is the faster one on every measured workload
-    h->n_fwd_ctas = forward_ctas(h, h->fwd_staged);
-    h->n_partials = std::max(forward_ctas(h, false), forward_ctas(h, true));
+    h->n_fwd_ctas = h->fwd_modes ? mode_forward_ctas(h) : forward_ctas(h, h->fwd_staged);
+    h->n_partials = std::max(std::max(forward_ctas(h, false), forward_ctas(h, true)), mode_forward_ctas(h));
     ALLOC(h->partials, sizeof(double) * h->n_partials);
     ALLOC(h->loss_dev, sizeof(double) * 4);
     ALLOC(h->red, sizeof(double) * dot_blocks(h));
@@ -809,6 +847,7 @@ tt_status tt_create(const tt_problem *P, tt_precision prec, void *stream, tt_han
         e = cudaMemcpyAsync(h->geo, h->geo_host.data(), sizeof(ProjGeom) * h->S, cudaMemcpyHostToDevice, h->stream);
     if (e == cudaSuccess) e = launch_basis(h, dstage, dstage + kQuadNodes);
     if (e == cudaSuccess) e = (prec != TT_F64) ? launch_cast_basis<float>(h) : launch_cast_basis<double>(h);
+    if (e == cudaSuccess) e = setup_modes(h, dstage + 2 * kQuadNodes);
     if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
     cudaFree(dstage);
     if (e != cudaSuccess) {
@@ -851,7 +890,8 @@ tt_status tt_set_forward_kernel(tt_handle *h, int kind)
         return TT_UNSUPPORTED;
     }
     h->fwd_staged = kind == kFwdStaged;
-    h->n_fwd_ctas = forward_ctas(h, h->fwd_staged);
+    h->fwd_modes = kind == kFwdAuto && h->slots != nullptr;
+    h->n_fwd_ctas = h->fwd_modes ? mode_forward_ctas(h) : forward_ctas(h, h->fwd_staged);
     return TT_OK;
 }
 
@@ -979,8 +1019,8 @@ tt_status tt_gradient_residual_host(tt_handle *h, const float *c_host, const flo
         cudaError_t e = cudaSuccess;
         for (int q = 0; q < Q && e == cudaSuccess; ++q) {
             const int s0 = (int)((long long)h->S * q / Q), s1 = (int)((long long)h->S * (q + 1) / Q);
-            e = cudaStreamWaitEvent(h->side[q & 1], h->chunk_ready[q], 0);
-            h->stream = h->side[q & 1];          // the launcher enqueues on h->stream
+            e = cudaStreamWaitEvent(h->side[h->fwd_modes ? 0 : q & 1], h->chunk_ready[q], 0);
+            h->stream = h->side[h->fwd_modes ? 0 : q & 1];   // the launcher enqueues on h->stream
             if (e == cudaSuccess) e = launch_forward<float, S>(h, nullptr, I, W, true, s0, s1);
             h->stream = main_stream;
         }

@@ -120,6 +120,84 @@ struct AdjParams {
     AdjProj<T> p[kMax];
 };
 
+// Where a gradient-mode forward writes the back-contracted residual when the
+// handle works in detector modes (tt_modes.cuh): rows of `row` floats at the
+// kernel's G argument and, with G1, one more value per ray; Q [CP][kModeQ],
+// zero padded.
+constexpr int kModeQ = 12;          // padded mode count of Q (at most 9 modes)
+constexpr int kMaxModes = 9;
+struct ModeOut {
+    const float *Q = nullptr;
+    float *G1 = nullptr;
+    int row = 0, nk1 = 0;             // nk1: row pitch of G1 (the detector's nk rounded up to 4)
+};
+
+// Layout of the R modes of a ray or voxel: rows of 4 * R4 floats and, with R1,
+// one more value in a separate plane behind all rows (R = 5 and 9 would waste
+// three floats of padding otherwise).
+__host__ __device__ constexpr int modes_r4(int R) { return R <= 5 ? 1 : 2; }
+__host__ __device__ constexpr int modes_r1(int R) { return (R == 5 || R == 9) ? 1 : 0; }
+
+// Mode adjoint (k_adjoint_modes): M = 4 * R4 + R1 stored modes; projections of
+// a hand-off unit, its tensor-core operand columns (2 M per projection, to a
+// multiple of 8) and channels (to a multiple of 16).
+__host__ __device__ constexpr int modes_m(int R) { return 4 * modes_r4(R) + modes_r1(R); }
+__host__ __device__ constexpr int modes_up(int M) { return M == 9 ? 1 : 2; }
+__host__ __device__ constexpr int modes_ku(int M) { return (2 * M * modes_up(M) + 7) / 8 * 8; }
+__host__ __device__ constexpr int modes_n(int K) { return (K + 15) / 16 * 16; }
+constexpr int kModeVox = 256;                  // voxels of a CTA: 8 (x) x 4 (y) x 8 (z), two tiles of 128
+// A mapped volume (slot): innermost axis first, rows of slot_pitch(n) voxels
+// -- kSlotLead zeros, the n voxels, zeros up to the pitch -- and kSlotBorder
+// zero rows and planes around them.  The taps of a ray's planes reach three
+// voxels beyond the volume (behind a row, into the next row's lead).  The rows
+// start on whole sectors, and the pitch modulo a 128-byte line (2 of 8 voxels
+// of four values, 16 of 32 single values) keeps neighbouring rays that have
+// stepped into the next row off each other's banks.
+constexpr int kSlotBorder = 3, kSlotLead = 8;
+__host__ __device__ constexpr int slot_pitch4(int n) { return (n + kSlotLead + 7) / 8 * 8 + 2; }
+__host__ __device__ constexpr int slot_pitch1(int n) { return (n + kSlotLead + 15) / 32 * 32 + 16; }
+constexpr long long kSlotBytes = 4LL << 30;    // slots of either copy
+constexpr uint32_t kMapCols = 256;             // tensor-memory columns of a map CTA
+constexpr int kModeStages = 3;                 // units in flight
+constexpr uint32_t kModeWaitTries = 1u << 20;
+constexpr long long kModeMaxSmem = 110 * 1024; // two CTAs per SM
+constexpr int kModeThreads = kModeVox / 2 + 32;   // two voxels per thread, and the warp that feeds the tensor cores
+// Resident CTAs per SM: the accumulators (2 N registers) and the tensor memory
+// (256 columns for N > 16) allow two, N = 16 four.
+__host__ __device__ constexpr int mode_ctas(int N) { return N == 16 ? 4 : 2; }
+__host__ __device__ constexpr uint32_t mode_align(uint32_t b) { return (b + 127) & ~127u; }
+
+// Per-projection constants of the mode adjoint, detector coordinates relative
+// to the CTA's box (o: outer, i: inner enumeration axis, see AdjProj): slopes
+// along the voxel axes, taps' slopes, oh = 1/2 - ho, the lower edge's au, av
+// with 1/2 added, index strides in the box, k0 = -kRoundBits (so + si), the
+// largest row index a column may start at.
+struct alignas(16) ModeProj {
+    float o[3], oh;
+    float i[3], pad;
+    float uo, vo, ui, vi;
+    float au, av, lu, lv;
+    int so, si, k0, lim;
+    int shape, order, pad2[2];
+};
+struct ModeParams {
+    static constexpr int kMax = 256;
+    ModeProj p[kMax];
+};
+// Detector coordinates of the voxel (x, y, z) = j[0] + j[1] x + ..., and the
+// lowest one of a block's candidate rays relative to its corner's.
+struct ModeOrigin {
+    double j[4], k[4], jlo, klo;
+    int outer_j;
+};
+// The adjoint's enumeration constants of a projection in FP64 (see AdjProj).
+struct AdjConst {
+    double oc[4], ic[4], bu[4], bv[4], jc[4], kc[4];
+    double uo, ui, vo, vi, ho, hi, au, lu, av, lv;
+    int no, ni;
+    bool outer_j;
+};
+
 struct LossSlot {
     double value;
     unsigned long long seq;
@@ -176,6 +254,29 @@ struct tt_handle {
     long long cpadx_origin = 0;          // voxel offset of (0,0,0) in the x-innermost copy (from its start)
     void *gpad = nullptr;                // device [nvox][KP]
     void *G = nullptr;                   // device [S][nj][nk][KP]
+    // Detector modes (tt_modes.cuh; 0: the handle works in channels): G holds
+    // rows of 4 * R4 mode values, then (R1) one more per ray.
+    int R = 0, R4 = 0, R1 = 0;
+    bool q_identity = false;             // the modes are the segments (Q = 1)
+    float *Qm = nullptr;                 // device [CP][kModeQ], zero padded
+    double *F64 = nullptr;               // device [S][R][K]: F_s
+    float *FB = nullptr;                 // device: F_s as the adjoint's tensor-core operand
+    tt::ModeOrigin *mode_org = nullptr;  // device [S]
+    int box_j = 0, box_k = 0;            // the adjoint's detector box (pixels)
+    int nk1 = 0;                         // row pitch of the single values' plane (R1)
+    std::vector<tt::ModeParams> mode_params;   // one block per launch
+    // Mode forward (tt_modes_fwd.cu): F rows for the map, the projections
+    // reading copy 0, then copy 1 of the packed volume, and the slots of
+    // mapped volumes: chunk slots for either copy, zero border.
+    void *FM = nullptr;
+    int *order = nullptr;                // device [S]
+    std::vector<int> order_host;
+    int order_begin[2] = {0, 0};
+    float *slots = nullptr;
+    long long slot_floats = 0, slot_vox = 0;   // floats of a slot, voxels of its four-value planes
+    long long slots1 = 0;                // where copy 1's slots start
+    int chunk = 0;                       // slots, the projections of a chunk
+    bool fwd_modes = false;              // the forward maps and marches modes
     double *partials = nullptr;          // device, per-CTA loss partials
     long long n_partials = 0;            // allocated entries
     long long n_fwd_ctas = 0;            // entries the forward kernel writes
@@ -338,6 +439,42 @@ cudaError_t launch_backcontract(tt_handle *h, const T *R);
 // reduction launch.
 template <typename T, typename S>
 cudaError_t launch_adjoint(tt_handle *h, T *g, bool reduce_loss = false);
+// The adjoint of K-channel G rows (h->G as [S][nj][nk][KP], filled by the
+// caller), whatever the handle's own layout.
+template <typename T, typename S>
+cudaError_t launch_adjoint_channels(tt_handle *h, T *g);
+// Detector modes: set-up (F_s, Q and the operand; enqueued on the handle's
+// stream, nodes as for launch_basis), the adjoint and the back-contraction.
+AdjConst adj_const(const ProjGeom &g);
+inline long long mode_operand_floats(const tt_handle *h)
+{
+    const int M = modes_m(h->R), UP = modes_up(M);
+    return (long long)((h->S + UP - 1) / UP) * 2 * modes_ku(M) * modes_n(h->K);
+}
+// Sets R and the boxes of a handle that can work in detector modes, else R = 0.
+void plan_modes(tt_handle *h);
+cudaError_t setup_modes(tt_handle *h, const double *frames);
+// The forward in modes (tt_modes_fwd.cu): ray tiles (loss partials), sizes
+// (slot_floats 0: the handle does not use it), set-up and launch.
+void plan_mode_forward(tt_handle *h);
+long long mode_forward_ctas(const tt_handle *h);
+cudaError_t setup_mode_forward(tt_handle *h, const double *F);
+template <typename S>
+cudaError_t launch_forward_modes(tt_handle *h, float *Iout, const float *I, const float *W, bool grad, int s0, int s1);
+// rows: the mode rows [S][nj][nk][4 R4] (h->G, or a caller's array).
+cudaError_t launch_adjoint_modes(tt_handle *h, const float *rows, float *g, bool reduce_loss);
+cudaError_t launch_backcontract_modes(tt_handle *h, const float *R);
+inline ModeOut mode_out(const tt_handle *h)
+{
+    ModeOut m;
+    if (h->R) {
+        m.Q = h->Qm;
+        m.row = 4 * h->R4;
+        m.nk1 = h->nk1;
+        m.G1 = h->R1 ? (float *)h->G + h->npix() * m.row : nullptr;
+    }
+    return m;
+}
 cudaError_t launch_reduce(tt_handle *h, const double *partials, long long n, double *out,
                           const double *add, double mul);
 cudaError_t launch_basis(tt_handle *h, const double *nodes, const double *weights);
@@ -363,7 +500,7 @@ inline int dot_blocks(const tt_handle *h) { return 4 * h->n_sm; }
 // bytes of slack to align the ring.
 inline size_t staged_forward_smem(const tt_handle *h)
 {
-    return (size_t)kStRing * h->stage_cap * 16 * sizeof(float) + (size_t)h->CP * 16 * sizeof(float) + 128;
+    return (size_t)kStRing * h->stage_cap * 16 * sizeof(float) + (size_t)h->CP * (16 + 16) * sizeof(float) + 128;   // (B_s and Q, 16 floats a segment each)
 }
 
 }  // namespace tt

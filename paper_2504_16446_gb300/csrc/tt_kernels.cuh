@@ -17,6 +17,7 @@
 
 #include <algorithm>
 #include <climits>
+#include <cmath>
 #include <type_traits>
 #include <vector>
 
@@ -232,15 +233,13 @@ __device__ __forceinline__ double block_sum(double v, double *red)
     return t;
 }
 
-// Sum of p[0..n) in a fixed order, for a block of kThreads threads: thread t
-// keeps eight running sums over t + kThreads i (i = 0, 1, ... taken round
-// robin), adds them pairwise, then block_sum.  The eight independent load
-// chains keep a single-CTA reduction short.  The result is valid on thread 0.
-__device__ __forceinline__ double sum_fixed_order(const double *__restrict__ p, long long n, double *red)
+// Thread t's share of a fixed-order sum by kThreads threads: eight running
+// sums over t + kThreads i (i = 0, 1, ... taken round robin), added pairwise.
+// The eight independent load chains keep a single-CTA reduction short.
+__device__ __forceinline__ double strided_sum(const double *__restrict__ p, long long n, long long t)
 {
     constexpr long long B = kThreads;
     double v8[8] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-    long long t = threadIdx.x;
     for (; t + 7 * B < n; t += 8 * B) {
 #pragma unroll
         for (int i = 0; i < 8; ++i) v8[i] += __ldg(p + t + i * B);
@@ -248,8 +247,61 @@ __device__ __forceinline__ double sum_fixed_order(const double *__restrict__ p, 
 #pragma unroll
     for (int i = 0; i < 7; ++i)
         if (t + i * B < n) v8[i] += __ldg(p + t + i * B);
-    const double v = ((v8[0] + v8[1]) + (v8[2] + v8[3])) + ((v8[4] + v8[5]) + (v8[6] + v8[7]));
-    return block_sum(v, red);
+    return ((v8[0] + v8[1]) + (v8[2] + v8[3])) + ((v8[4] + v8[5]) + (v8[6] + v8[7]));
+}
+
+// Sum of p[0..n) in a fixed order, for a block of kThreads threads
+// (strided_sum, then block_sum).  The result is valid on thread 0.
+__device__ __forceinline__ double sum_fixed_order(const double *__restrict__ p, long long n, double *red)
+{
+    return block_sum(strided_sum(p, n, threadIdx.x), red);
+}
+
+// Even-l real SH at a direction (need not be normalised), written to
+// out[i*stride].  Cartesian recurrences: with r = |q|, (x + i y)^m gives
+// sin^m(theta) cos(m phi) and sin^m(theta) sin(m phi); the associated
+// Legendre factor without its sin^m(theta) is the polynomial
+//   Q_m^m = (2m-1)!!,  Q_{m+1}^m = (2m+1) z Q_m^m,
+//   (l-m) Q_l^m = (2l-1) z Q_{l-1}^m - (l+m-1) Q_{l-2}^m
+// and Y_lm = sqrt(2) N_lm Q_l^m Re/Im (x+iy)^m (m != 0), Y_l0 = N_l0 Q_l^0 with
+// N_lm = sqrt((2l+1)/(4 pi) (l-m)!/(l+m)!) -- orthonormal, no Condon-Shortley
+// phase, polar axis +z (Section "Basis sets", SH).
+template <typename T>
+__device__ void sh_even(int L, T x, T y, T z, T *out, int stride)
+{
+    const T rn = T(1) / sqrt(x * x + y * y + z * z);
+    x *= rn; y *= rn; z *= rn;
+    T cr = T(1), ci = T(0);                 // (x + i y)^m
+    T qmm = T(1);                           // Q_m^m
+    for (int m = 0; m <= L; ++m) {
+        if (m > 0) {
+            const T ncr = cr * x - ci * y, nci = cr * y + ci * x;
+            cr = ncr; ci = nci;
+            qmm *= T(2 * m - 1);
+        }
+        T q_lm2 = T(0), q_lm1 = qmm;        // Q_{l-2}^m, Q_{l-1}^m as l advances
+        for (int l = m; l <= L; ++l) {
+            T qlm;
+            if (l == m) qlm = qmm;
+            else if (l == m + 1) qlm = T(2 * m + 1) * z * qmm;
+            else qlm = (T(2 * l - 1) * z * q_lm1 - T(l + m - 1) * q_lm2) / T(l - m);
+            if (l > m) { q_lm2 = q_lm1; q_lm1 = qlm; }
+            if ((l & 1) == 0) {
+                // (l-m)!/(l+m)!
+                T ratio = T(1);
+                for (int t = l - m + 1; t <= l + m; ++t) ratio /= T(t);
+                const T nlm = sqrt(T(2 * l + 1) / T(4.0 * M_PI) * ratio);
+                const int base = l * (l - 1) / 2 + l;   // index of (l, m = 0)
+                if (m == 0) {
+                    out[base * stride] = nlm * qlm;
+                } else {
+                    const T f = T(M_SQRT2) * nlm * qlm;
+                    out[(base + m) * stride] = f * cr;
+                    out[(base - m) * stride] = f * ci;
+                }
+            }
+        }
+    }
 }
 
 // Transverse coordinates of ray (j, k) on plane 0, u0 + j uj + k uk and
@@ -279,7 +331,26 @@ __device__ __forceinline__ void clip_planes(T w0, T dw, int N, T &lo, T &hi)
     hi = fmin(hi, fmax(p1, p2));
 }
 
-// SH contraction of a marched ray and, in GRAD mode, the residual, its
+// kGradModes keeps Q in shared memory as the lanes of a group read it: lane q
+// sums modes q, q + LG, ... and finds their entries of a segment side by side,
+// padded to a multiple of four.
+__host__ __device__ constexpr int mode_lane(int LG) { return ((kMaxModes + LG - 1) / LG + 3) / 4 * 4; }
+template <int LG, int THREADS>
+__device__ __forceinline__ void stage_modes(float *Qs, const float *Q, int CP)
+{
+    constexpr int NL = mode_lane(LG);
+    for (int t = threadIdx.x; t < CP * LG * NL; t += THREADS) {
+        const int i = t % NL, q = t / NL % LG, c = t / (NL * LG), m = q + i * LG;
+        Qs[t] = m < kModeQ ? Q[c * kModeQ + m] : 0.f;
+    }
+}
+
+// What a forward kernel does with a marched ray: PROJECT writes the segment
+// intensities; GRAD forms the residual, its square and its back-contraction
+// into the K channels, GRAD_MODES into the detector modes (tt_modes.cuh).
+enum { kProject = 0, kGrad = 1, kGradModes = 2 };
+
+// SH contraction of a marched ray and, in the gradient modes, the residual, its
 // weighted square and the back-contraction (Eq. forward_model, Eq. residual).
 // The contraction runs four segments at a time: partial dot products over the
 // lane's CPL channels (chunk `chunk` of the row), a butterfly across the LG
@@ -287,16 +358,21 @@ __device__ __forceinline__ void clip_planes(T w0, T dw, int N, T &lo, T &hi)
 // channels.  Lanes with
 // writer == false (duplicate halves) compute but do not store.  Returns the
 // ray's sum of W r^2 on every lane.
-template <typename T, typename S, int CPL, int KP, int LG, bool GRAD>
+template <typename T, typename S, int CPL, int KP, int LG, int MODE>
 __device__ __forceinline__ T forward_epilogue(const T (&acc)[CPL], int q, int chunk, bool valid, bool writer,
                                               long long pix,
                                               const T *__restrict__ Bs, int C, int CP, T *__restrict__ Iout,
                                               const T *__restrict__ Id, const T *__restrict__ Wd,
-                                              T *__restrict__ G)
+                                              T *__restrict__ G, const float *__restrict__ Qs, const ModeOut &mo, long long pix1)
 {
-    T gacc[CPL];
+    constexpr bool GRAD = MODE != kProject;
+    // kGradModes: lane q of the group sums modes q, q + LG, ...
+    constexpr int NM = MODE == kGradModes ? (kMaxModes + LG - 1) / LG : 1;
+    T gacc[CPL], gm[NM];
 #pragma unroll
     for (int i = 0; i < CPL; ++i) gacc[i] = T(0);
+#pragma unroll
+    for (int i = 0; i < NM; ++i) gm[i] = T(0);
     T lossr = T(0);
     const int boff = chunk * CPL;
     const bool vec4 = (C % 4) == 0;
@@ -357,14 +433,36 @@ __device__ __forceinline__ T forward_epilogue(const T (&acc)[CPL], int q, int ch
                 const T rr = live ? ih[t] - dI[t] : T(0);
                 const T wr = live ? dW[t] * rr : T(0);
                 lossr = fma(wr, rr, lossr);
-                const T *brow = Bs + (c0 + t) * KP + boff;
+                if constexpr (MODE == kGradModes) {
+                    const float4 *qrow = reinterpret_cast<const float4 *>(Qs) + ((c0 + t) * LG + q) * (mode_lane(LG) / 4);
 #pragma unroll
-                for (int i = 0; i < CPL; ++i) gacc[i] = fma(brow[i], wr, gacc[i]);
+                    for (int i = 0; i < NM; i += 4) {
+                        const float4 f = qrow[i / 4];
+                        const float fq[4] = {f.x, f.y, f.z, f.w};
+#pragma unroll
+                        for (int k = 0; k < 4; ++k)
+                            if (i + k < NM) gm[i + k] = fma(T(fq[k]), wr, gm[i + k]);
+                    }
+                } else {
+                    const T *brow = Bs + (c0 + t) * KP + boff;
+#pragma unroll
+                    for (int i = 0; i < CPL; ++i) gacc[i] = fma(brow[i], wr, gacc[i]);
+                }
             }
         }
     }
-    if constexpr (GRAD) {
+    if constexpr (MODE == kGrad) {
         if (valid && writer) store_row<T, CPL>(G + pix * KP + chunk * CPL, gacc, T(2));
+    }
+    if constexpr (MODE == kGradModes) {
+        if (valid && writer) {
+#pragma unroll
+            for (int i = 0; i < NM; ++i) {
+                const int m = q + i * LG;
+                if (m < mo.row) G[pix * mo.row + m] = T(2) * gm[i];
+                else if (m == mo.row && mo.G1) mo.G1[pix1] = 2.f * (float)gm[i];
+            }
+        }
     }
     return lossr;
 }
@@ -379,19 +477,40 @@ __device__ __forceinline__ T forward_epilogue(const T (&acc)[CPL], int q, int ch
 // The SH contraction runs four segments at a time: partial dot products over
 // the lane's channels, a butterfly across the lane group, then each lane
 // back-contracts into its own channels.
-template <typename T, typename S, int KP, int LG, bool GRAD>
-__global__ void __launch_bounds__(kFwdThreads)
+// Resident CTAs asked of the compiler (0: none).  What it trades is registers,
+// hence planes in flight, against CTAs; measured in whole calls (us), project /
+// evaluation:
+//   FP32, 16 channels: five when the long gradient epilogue follows, four else
+//     (64^3: project 307 / 328 with four / five, evaluation 578 / 575; 128^3,
+//     l_max 4: 4780 / 5206, 8380 / 7896)
+//   2-byte, 16 channels: 64^3 project 286 / 275 with none / four, 128^3
+//     evaluation 7229 / 7258
+//   2-byte, 8 channels (56^3, 240 projections): 200 / 562 with none, 192 / 562
+//     with four; wider rows (28^3, l_max 6): 41.6 / 104.4 none, 37.0 / 101.5 three
+//   FP32, 8 channels (56^3, 240 projections): 281 / 626 with none, 243 / 606 with
+//     one; wider rows (20^3, l_max 8): 46.9 / 112.5, 37.3 / 102.2
+__host__ __device__ constexpr int fwd_ctas(int KP, int bytes, int mode)
+{
+    if (bytes == 8) return 0;
+    if (bytes == 4) return KP == 16 ? (mode == kProject ? 4 : 5) : 1;
+    return KP == 16 ? (mode == kProject ? 4 : 0) : (KP <= 8 ? 4 : 3);
+}
+
+template <typename T, typename S, int KP, int LG, int MODE>
+__global__ void __launch_bounds__(kFwdThreads, fwd_ctas(KP, sizeof(S), MODE))
 k_forward(const ProjGeom *__restrict__ geo, const S *__restrict__ cpad /* interior origin */,
           const S *__restrict__ cpadx /* interior origin of the x-innermost copy, or NULL */, const T *__restrict__ Bp,
           int nj, int nk, int C, int CP, int tiles_k, int slab_order, int s_base,
           T *__restrict__ Iout, const T *__restrict__ Id, const T *__restrict__ Wd,
-          T *__restrict__ G, double *__restrict__ partials)
+          T *__restrict__ G, double *__restrict__ partials, ModeOut mo)
 {
+    constexpr bool GRAD = MODE != kProject;
     constexpr int CPL = KP / LG;
     constexpr int TK = fwd_tk(LG);
     constexpr int TJ = fwd_tj(LG);
     extern __shared__ __align__(16) unsigned char smem_raw[];
     T *Bs = reinterpret_cast<T *>(smem_raw);   // [CP][KP]
+    float *Qs = reinterpret_cast<float *>(Bs + (size_t)CP * KP);   // kGradModes: [CP][LG][mode_lane]
     __shared__ double red[kFwdThreads / 32];
 
     // CTA order.  slab_order == 0: all tiles of one projection, projection by
@@ -411,6 +530,7 @@ k_forward(const ProjGeom *__restrict__ geo, const S *__restrict__ cpad /* interi
 
     const T *Bsrc = Bp + (size_t)s * CP * KP;
     for (int t = threadIdx.x; t < CP * KP; t += kFwdThreads) Bs[t] = Bsrc[t];
+    if constexpr (MODE == kGradModes) stage_modes<LG, kFwdThreads>(Qs, mo.Q, CP);
 
     const ProjGeom &P = geo[s];
     // Ray base in FP64 (one rounding to T), per-plane stepping in T.
@@ -459,29 +579,41 @@ k_forward(const ProjGeom *__restrict__ geo, const S *__restrict__ cpad /* interi
     // bfloat16 0.313 -> 0.277 ms); FP32 rows of 16 channels hold 16 words
     // per plane already, and unrolling them was measured slower.
     constexpr int kUnroll = KP == 32 ? 2 : ((sizeof(S) == 2 && KP <= 16) ? 4 : 1);
-#pragma unroll kUnroll
-    for (int p = plo; p <= phi; ++p) {
+    struct Plane {
+        unsigned x0[NW], x1[NW];
+        T wu, wv;
+    };
+    auto fetch = [&](Plane &q, int p) {
         const T u = fma((T)p, up, ur), v = fma((T)p, vp, vr);
         const T fu = floor(u), fv = floor(v);
         const int iu = min(max((int)fu, -2), Nu), iv = min(max((int)fv, -2), Nv);
-        const T wu = u - fu, wv = v - fv;
+        q.wu = u - fu;
+        q.wv = v - fv;
         const S *t0 = cq + ((long long)p * sm + (long long)iu * su + iv) * KP;
-        unsigned x0[NW], x1[NW];
         // any p in [plo - 1, phi + 1] and the clamped iu, iv address the padded
         // volume (two-voxel border), so the loads may run speculatively
-        ldg_words<PIECEB, ALIGN, true>(t0, x0);
-        ldg_words<PIECEB, ALIGN, true>(t0 + sub, x1);
+        ldg_words<PIECEB, ALIGN, true>(t0, q.x0);
+        ldg_words<PIECEB, ALIGN, true>(t0 + sub, q.x1);
+    };
+    auto add = [&](const Plane &q) {
+        const T wu = q.wu, wv = q.wv;
         if constexpr (LG >= 2) {
             const T wvh = h ? wv : T(1) - wv;
-            fma_words<T, S, ACH, 0>(acc, (T(1) - wu) * wvh, x0);
-            fma_words<T, S, ACH, 0>(acc, wu * wvh, x1);
+            fma_words<T, S, ACH, 0>(acc, (T(1) - wu) * wvh, q.x0);
+            fma_words<T, S, ACH, 0>(acc, wu * wvh, q.x1);
         } else {
             const T a0 = T(1) - wu, b0 = T(1) - wv;
-            fma_words<T, S, ACH, 0>(acc, a0 * b0, x0);
-            fma_words<T, S, ACH, KP>(acc, a0 * wv, x0);
-            fma_words<T, S, ACH, 0>(acc, wu * b0, x1);
-            fma_words<T, S, ACH, KP>(acc, wu * wv, x1);
+            fma_words<T, S, ACH, 0>(acc, a0 * b0, q.x0);
+            fma_words<T, S, ACH, KP>(acc, a0 * wv, q.x0);
+            fma_words<T, S, ACH, 0>(acc, wu * b0, q.x1);
+            fma_words<T, S, ACH, KP>(acc, wu * wv, q.x1);
         }
+    };
+#pragma unroll kUnroll
+    for (int p = plo; p <= phi; ++p) {
+        Plane a;
+        fetch(a, p);
+        add(a);
     }
     // Both rows' sums in every lane of a pair, then lane q keeps channel
     // chunk `chunk` (CPL channels) for the epilogue.
@@ -504,8 +636,8 @@ k_forward(const ProjGeom *__restrict__ geo, const S *__restrict__ cpad /* interi
     __syncthreads();   // Bs staged
 
     const long long pix = ((long long)s * nj + j) * nk + k;
-    const T lossr = forward_epilogue<T, S, CPL, KP, LG, GRAD>(accq, q, chunk, valid, true, pix, Bs, C, CP, Iout, Id,
-                                                              Wd, G);
+    const T lossr = forward_epilogue<T, S, CPL, KP, LG, MODE>(accq, q, chunk, valid, true, pix, Bs, C, CP, Iout, Id,
+                                                              Wd, G, Qs, mo, ((long long)s * nj + j) * mo.nk1 + k);
     if constexpr (GRAD) {
         double tot;
         if constexpr (std::is_same<T, float>::value)
@@ -561,13 +693,14 @@ __device__ __forceinline__ int stage_lo(float cmin, int N)
     return min(max((int)floorf(cmin - kStEps), -2), N);
 }
 
-template <bool GRAD>
+template <int MODE>
 __global__ void __launch_bounds__(kStThreads, 2)
 k_forward_staged(const ProjGeom *__restrict__ geo, const TmaDesc *__restrict__ tmaps, const float *__restrict__ Bp,
                  int nj, int nk, int C, int CP, int tiles_k, int slab_order, int s_base, int cap,
                  float *__restrict__ Iout, const float *__restrict__ Id, const float *__restrict__ Wd,
-                 float *__restrict__ G, double *__restrict__ partials)
+                 float *__restrict__ G, double *__restrict__ partials, ModeOut mo)
 {
+    constexpr bool GRAD = MODE != kProject;
     constexpr int KP = 16, LG = 4, CPL = 4, NR = 2;
     // The tensor copies write 128-byte aligned stages: the dynamic shared
     // memory holds 128 bytes of slack and the ring starts at its first
@@ -576,6 +709,7 @@ k_forward_staged(const ProjGeom *__restrict__ geo, const TmaDesc *__restrict__ t
     unsigned char *ring = st_smem + ((128u - (umma::smem_u32(st_smem) & 127u)) & 127u);
     float *stages = reinterpret_cast<float *>(ring);           // kStRing * cap voxels of KP floats
     float *Bs = stages + (size_t)kStRing * cap * KP;           // [CP][KP]
+    float *Qs = Bs + (size_t)CP * KP;                          // [CP][LG][mode_lane]
     __shared__ __align__(8) uint64_t full[kStMaxDepth], empty[kStMaxDepth];
     __shared__ StageHdr hdr[kStMaxDepth];
     __shared__ int prange[2];
@@ -589,6 +723,7 @@ k_forward_staged(const ProjGeom *__restrict__ geo, const TmaDesc *__restrict__ t
 
     const float *Bsrc = Bp + (size_t)s * CP * KP;
     for (int t = threadIdx.x; t < CP * KP; t += kStThreads) Bs[t] = Bsrc[t];
+    if constexpr (MODE == kGradModes) stage_modes<LG, kStThreads>(Qs, mo.Q, CP);
     if (threadIdx.x == 0) {
         for (int i = 0; i < kStMaxDepth; ++i) {
             umma::mbar_init(&full[i], 1);
@@ -744,8 +879,9 @@ k_forward_staged(const ProjGeom *__restrict__ geo, const TmaDesc *__restrict__ t
 #pragma unroll
             for (int i = 0; i < CPL; ++i) accq[i] = ok ? ((q >> 1) ? acc[r][CPL + i] : acc[r][i]) * step : bad;
             const long long pix = ((long long)s * nj + (j0 + 4 * r)) * nk + k;
-            const float lr = forward_epilogue<float, float, CPL, KP, LG, GRAD>(accq, q, chunk, valid[r], true, pix, Bs,
-                                                                           C, CP, Iout, Id, Wd, G);
+            const float lr = forward_epilogue<float, float, CPL, KP, LG, MODE>(accq, q, chunk, valid[r], true, pix, Bs,
+                                                                           C, CP, Iout, Id, Wd, G, Qs, mo,
+                                                                           ((long long)s * nj + (j0 + 4 * r)) * mo.nk1 + k);
             if (q == 0 && valid[r]) dot2_add1(lossr, lr);
         }
     }
@@ -1089,6 +1225,8 @@ template <typename T, typename S, int L>
 cudaError_t launch_forward_L(tt_handle *h, T *Iout, const T *I, const T *W, bool grad, int s0, int s1)
 {
     if (s1 < 0) s1 = h->S;
+    if constexpr (std::is_same<T, float>::value)
+        if (h->fwd_modes) return launch_forward_modes<S>(h, Iout, I, W, grad, s0, s1);
     const int ns = s1 - s0;
     constexpr int K = num_coeffs(L), KP = padded_k(K), LG = lane_group(K);
     // slab order once the padded volume would take more than half of L2
@@ -1107,17 +1245,17 @@ cudaError_t launch_forward_L(tt_handle *h, T *Iout, const T *I, const T *W, bool
             const size_t smem = staged_forward_smem(h);
             prof_begin(h, TT_KSLOT_FORWARD, &ev);
             if (grad) {
-                auto kern = k_forward_staged<true>;
+                auto kern = h->R ? k_forward_staged<kGradModes> : k_forward_staged<kGrad>;
                 cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
                 kern<<<grid, kStThreads, smem, h->stream>>>(h->geo, h->tmaps, Bp, h->nj, h->nk, h->C, h->CP, tiles_k,
                                                             slab, s0, h->stage_cap, nullptr, I, W, (T *)h->G,
-                                                            h->partials);
+                                                            h->partials, mode_out(h));
             } else {
-                auto kern = k_forward_staged<false>;
+                auto kern = k_forward_staged<kProject>;
                 cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
                 kern<<<grid, kStThreads, smem, h->stream>>>(h->geo, h->tmaps, Bp, h->nj, h->nk, h->C, h->CP, tiles_k,
                                                             slab, s0, h->stage_cap, Iout, nullptr, nullptr, nullptr,
-                                                            nullptr);
+                                                            nullptr, ModeOut{});
             }
             cudaError_t e = cudaGetLastError();
             prof_end(h, TT_KSLOT_FORWARD, ev);
@@ -1127,18 +1265,27 @@ cudaError_t launch_forward_L(tt_handle *h, T *Iout, const T *I, const T *W, bool
     constexpr int TK = fwd_tk(LG), TJ = fwd_tj(LG);
     const int tiles_k = (h->nk + TK - 1) / TK, tiles_j = (h->nj + TJ - 1) / TJ;
     const dim3 grid = slab ? dim3(tiles_k * ns, tiles_j) : dim3(tiles_k * tiles_j, ns);
-    const size_t smem = (size_t)h->CP * KP * sizeof(T);
+    const size_t smem = (size_t)h->CP * (KP * sizeof(T) + LG * mode_lane(LG) * sizeof(float));
     prof_begin(h, TT_KSLOT_FORWARD, &ev);
-    if (grad) {
-        auto kern = k_forward<T, S, KP, LG, true>;
+    auto run = [&](auto kern) {
         if (smem > 48 * 1024) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        kern<<<grid, kFwdThreads, smem, h->stream>>>(h->geo, cpad, cpadx, Bp, h->nj, h->nk, h->C, h->CP, tiles_k, slab, s0,
-                                                 nullptr, I, W, (T *)h->G, h->partials);
+        if (grad)
+            kern<<<grid, kFwdThreads, smem, h->stream>>>(h->geo, cpad, cpadx, Bp, h->nj, h->nk, h->C, h->CP, tiles_k,
+                                                         slab, s0, nullptr, I, W, (T *)h->G, h->partials, mode_out(h));
+        else
+            kern<<<grid, kFwdThreads, smem, h->stream>>>(h->geo, cpad, cpadx, Bp, h->nj, h->nk, h->C, h->CP, tiles_k,
+                                                         slab, s0, Iout, nullptr, nullptr, nullptr, nullptr,
+                                                         ModeOut{});
+    };
+    if (!grad) {
+        run(k_forward<T, S, KP, LG, kProject>);
     } else {
-        auto kern = k_forward<T, S, KP, LG, false>;
-        if (smem > 48 * 1024) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        kern<<<grid, kFwdThreads, smem, h->stream>>>(h->geo, cpad, cpadx, Bp, h->nj, h->nk, h->C, h->CP, tiles_k, slab, s0,
-                                                 Iout, nullptr, nullptr, nullptr, nullptr);
+        bool modes = false;
+        if constexpr (std::is_same<T, float>::value && L >= 2 && L <= 8) {
+            modes = h->R > 0;
+            if (modes) run(k_forward<T, S, KP, LG, kGradModes>);
+        }
+        if (!modes) run(k_forward<T, S, KP, LG, kGrad>);
     }
     cudaError_t e = cudaGetLastError();
     prof_end(h, TT_KSLOT_FORWARD, ev);
@@ -1193,6 +1340,21 @@ cudaError_t launch_adjoint_L(tt_handle *h, T *g, bool reduce_loss)
     return e;
 }
 
+template <typename T, typename S>
+cudaError_t adjoint_channels(tt_handle *h, T *g, bool rl)
+{
+    switch (h->L) {
+    case 0: return launch_adjoint_L<T, S, 0>(h, g, rl);
+    case 2: return launch_adjoint_L<T, S, 2>(h, g, rl);
+    case 4: return launch_adjoint_L<T, S, 4>(h, g, rl);
+    case 6: return launch_adjoint_L<T, S, 6>(h, g, rl);
+    case 8: return launch_adjoint_L<T, S, 8>(h, g, rl);
+    case 10: return launch_adjoint_L<T, S, 10>(h, g, rl);
+    case 12: return launch_adjoint_L<T, S, 12>(h, g, rl);
+    default: return cudaErrorInvalidValue;
+    }
+}
+
 // Instantiates the three launchers of one (T, S) pair for every band limit.
 #define TT_INSTANTIATE_PROJECTORS(T, S)                                                        \
     template <>                                                                                \
@@ -1213,6 +1375,8 @@ cudaError_t launch_adjoint_L(tt_handle *h, T *g, bool reduce_loss)
     template <>                                                                                \
     cudaError_t launch_backcontract<T, S>(tt_handle * h, const T *R)                           \
     {                                                                                          \
+        if constexpr (std::is_same<T, float>::value)                                           \
+            if (h->R) return launch_backcontract_modes(h, (const float *)R);                     \
         switch (h->L) {                                                                        \
         case 0: return launch_backcontract_L<T, S, 0>(h, R);                                   \
         case 2: return launch_backcontract_L<T, S, 2>(h, R);                                   \
@@ -1225,18 +1389,13 @@ cudaError_t launch_adjoint_L(tt_handle *h, T *g, bool reduce_loss)
         }                                                                                      \
     }                                                                                          \
     template <>                                                                                \
+    cudaError_t launch_adjoint_channels<T, S>(tt_handle * h, T * g) { return adjoint_channels<T, S>(h, g, false); } \
+    template <>                                                                                \
     cudaError_t launch_adjoint<T, S>(tt_handle * h, T * g, bool rl)                            \
     {                                                                                          \
-        switch (h->L) {                                                                        \
-        case 0: return launch_adjoint_L<T, S, 0>(h, g, rl);                                    \
-        case 2: return launch_adjoint_L<T, S, 2>(h, g, rl);                                    \
-        case 4: return launch_adjoint_L<T, S, 4>(h, g, rl);                                    \
-        case 6: return launch_adjoint_L<T, S, 6>(h, g, rl);                                    \
-        case 8: return launch_adjoint_L<T, S, 8>(h, g, rl);                                    \
-        case 10: return launch_adjoint_L<T, S, 10>(h, g, rl);                                  \
-        case 12: return launch_adjoint_L<T, S, 12>(h, g, rl);                                  \
-        default: return cudaErrorInvalidValue;                                                 \
-        }                                                                                      \
+        if constexpr (std::is_same<T, float>::value)                                           \
+            if (h->R) return launch_adjoint_modes(h, (const float *)h->G, (float *)g, rl);     \
+        return adjoint_channels<T, S>(h, g, rl);                                               \
     }
 
 }  // namespace tt

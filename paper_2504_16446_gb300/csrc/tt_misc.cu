@@ -226,53 +226,6 @@ template cudaError_t vec_sub<double>(tt_handle *, double *, const double *, cons
 
 // ------------------------------------------------------------- real SH
 
-// Even-l real SH at a direction (need not be normalised), written to
-// out[i*stride].  Cartesian recurrences: with r = |q|, (x + i y)^m gives
-// sin^m(theta) cos(m phi) and sin^m(theta) sin(m phi); the associated
-// Legendre factor without its sin^m(theta) is the polynomial
-//   Q_m^m = (2m-1)!!,  Q_{m+1}^m = (2m+1) z Q_m^m,
-//   (l-m) Q_l^m = (2l-1) z Q_{l-1}^m - (l+m-1) Q_{l-2}^m
-// and Y_lm = sqrt(2) N_lm Q_l^m Re/Im (x+iy)^m (m != 0), Y_l0 = N_l0 Q_l^0 with
-// N_lm = sqrt((2l+1)/(4 pi) (l-m)!/(l+m)!) -- orthonormal, no Condon-Shortley
-// phase, polar axis +z (Section "Basis sets", SH).
-template <typename T>
-__device__ void sh_even(int L, T x, T y, T z, T *out, int stride)
-{
-    const T rn = T(1) / sqrt(x * x + y * y + z * z);
-    x *= rn; y *= rn; z *= rn;
-    T cr = T(1), ci = T(0);                 // (x + i y)^m
-    T qmm = T(1);                           // Q_m^m
-    for (int m = 0; m <= L; ++m) {
-        if (m > 0) {
-            const T ncr = cr * x - ci * y, nci = cr * y + ci * x;
-            cr = ncr; ci = nci;
-            qmm *= T(2 * m - 1);
-        }
-        T q_lm2 = T(0), q_lm1 = qmm;        // Q_{l-2}^m, Q_{l-1}^m as l advances
-        for (int l = m; l <= L; ++l) {
-            T qlm;
-            if (l == m) qlm = qmm;
-            else if (l == m + 1) qlm = T(2 * m + 1) * z * qmm;
-            else qlm = (T(2 * l - 1) * z * q_lm1 - T(l + m - 1) * q_lm2) / T(l - m);
-            if (l > m) { q_lm2 = q_lm1; q_lm1 = qlm; }
-            if ((l & 1) == 0) {
-                // (l-m)!/(l+m)!
-                T ratio = T(1);
-                for (int t = l - m + 1; t <= l + m; ++t) ratio /= T(t);
-                const T nlm = sqrt(T(2 * l + 1) / T(4.0 * M_PI) * ratio);
-                const int base = l * (l - 1) / 2 + l;   // index of (l, m = 0)
-                if (m == 0) {
-                    out[base * stride] = nlm * qlm;
-                } else {
-                    const T f = T(M_SQRT2) * nlm * qlm;
-                    out[(base + m) * stride] = f * cr;
-                    out[(base - m) * stride] = f * ci;
-                }
-            }
-        }
-    }
-}
-
 // B[s][c][i] = 0.5 * sum_n w_n Y_i(R_s^T q(phi_n)), phi_n = mid + half x_n
 // (Gauss-Legendre on the segment; 1/dphi * half = 0.5), Eq. (projection_matrix).
 // One CTA per (c, s), one thread per quadrature node.

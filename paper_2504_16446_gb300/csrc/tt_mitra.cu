@@ -167,7 +167,7 @@ tt_status sirt_weights_impl(tt_handle *h, const T *W, T *R, T *D)
         e = cudaGetLastError();
         prof_end(h, TT_KSLOT_VECTOR, ev);
     }
-    if (e == cudaSuccess) e = launch_adjoint<T, S>(h, D);
+    if (e == cudaSuccess) e = launch_adjoint_channels<T, S>(h, D);
     if (e == cudaSuccess) {
         prof_begin(h, TT_KSLOT_VECTOR, &ev);
         k_invert<T><<<blocks_for(h->nvox() * h->K), 256, 0, h->stream>>>(D, h->nvox() * h->K, 1e-6 * h->a * kY00);

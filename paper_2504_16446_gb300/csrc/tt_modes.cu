@@ -1,0 +1,294 @@
+// tt_modes.cu -- set-up and launchers of the detector-mode projector
+// (tt_modes.cuh).
+#include <cmath>
+#include <cstring>
+
+#include <cuda.h>
+#include <cudaTypedefs.h>
+
+#include "tt_modes.cuh"
+
+namespace tt {
+
+// The two_theta = 0 circle is a great circle: even functions have even modes
+// only.
+static int mode_step(const tt_handle *h) { return h->two_theta == 0.0 ? 2 : 1; }
+
+// Detector coordinate range of a block of 8 x 4 x 8 voxels relative to its
+// corner: the sum of the slopes' negative, positive parts.
+static void block_range(const double *c, double &lo, double &hi)
+{
+    const double ext[3] = {7.0, 3.0, 7.0};
+    lo = hi = 0.0;
+    for (int t = 0; t < 3; ++t) (c[1 + t] < 0 ? lo : hi) += ext[t] * c[1 + t];
+}
+
+// Tensor map of a plane of row values [S][nj][pitch * w floats], box bj x bk
+// pixels of w floats each.
+static bool encode_rows(const tt_handle *h, const void *base, int w, int pitch, TmaDesc *out)
+{
+    const auto enc = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(driver_tensor_map_encoder());
+    const cuuint64_t dims[3] = {(cuuint64_t)w * h->nk, (cuuint64_t)h->nj, (cuuint64_t)h->S};
+    const cuuint64_t strides[2] = {(cuuint64_t)w * pitch * 4, (cuuint64_t)w * pitch * 4 * h->nj};
+    const cuuint32_t box[3] = {(cuuint32_t)(w * h->box_k), (cuuint32_t)h->box_j, 1}, elem[3] = {1, 1, 1};
+    CUtensorMap m;
+    if (enc(&m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, const_cast<void *>(base), dims, strides, box, elem,
+            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+        return false;
+    std::memcpy(out, &m, sizeof(m));
+    return true;
+}
+
+static size_t modes_smem(const tt_handle *h)
+{
+    const int M = modes_m(h->R), UP = modes_up(M);
+    const uint32_t px = (uint32_t)(h->box_j * h->box_k);
+    const size_t boxes = mode_align(px * 16 * h->R4) + (h->R1 ? mode_align(px * 4) : 0);
+    return kModeStages * (UP * boxes + 2 * (size_t)modes_ku(M) * modes_n(h->K) * 4) + 128;
+}
+
+// The handle works in modes when there are at most kMaxModes of them, the band
+// limit is 2 .. 8, and every projection's box -- the rays of a block lie
+// within (hj, hk) of its voxels' centres, plus the rounding margin and up to
+// three pixels from aligning the box to four -- fits the tensor copies (256
+// floats wide) and, kModeStages deep, the shared memory of two CTAs per SM.
+// (Pixels much finer than voxels put too many rays around a block; the
+// channel kernels take those.)  Coordinates stay below 2^22 in magnitude for
+// volumes and detectors of at most 2^14, which the rounding by kRound needs.
+void plan_modes(tt_handle *h)
+{
+    h->R = 0;
+    if (h->prec == TT_F64 || h->L < 2 || h->L > 8 || !driver_tensor_map_encoder()) return;
+    const int limit = 1 << 14;
+    if (h->N[0] > limit || h->N[1] > limit || h->N[2] > limit || h->nj > limit || h->nk > limit) return;
+    const int R = std::min(h->two_theta == 0.0 ? h->L + 1 : 2 * h->L + 1, h->C);
+    if (R > kMaxModes) return;
+    int bj = 1, bk = 4;
+    for (const ProjGeom &g : h->geo_host) {
+        const AdjConst c = adj_const(g);
+        double jl, jh, kl, kh;
+        block_range(c.jc, jl, jh);
+        block_range(c.kc, kl, kh);
+        const double wj = jh - jl + 2.0 * g.hj + 0.04, wk = kh - kl + 2.0 * g.hk + 0.04;
+        if (!(wj < 200.0) || !(wk < 200.0)) return;
+        // a column whose first ray is in the box is read to its end
+        bj = std::max(bj, (int)std::ceil(wj) + 1 + (c.outer_j ? 0 : c.ni - 1));
+        bk = std::max(bk, ((int)std::ceil(wk) + 1 + (c.outer_j ? c.ni - 1 : 0) + 3 + 3) / 4 * 4);
+    }
+    h->R = R;
+    h->R4 = modes_r4(R);
+    h->R1 = modes_r1(R);
+    h->q_identity = R == h->C;
+    h->nk1 = (h->nk + 3) / 4 * 4;
+    h->box_j = bj;
+    h->box_k = bk;
+    TmaDesc probe;
+    if (bk * 4 * h->R4 > 256 || bj > 256 || (long long)modes_smem(h) > kModeMaxSmem ||
+        !encode_rows(h, (const void *)4096, 4 * h->R4, h->nk, &probe) ||
+        !encode_rows(h, (const void *)4096, 1, h->nk1, &probe)) {
+        h->R = 0;
+        return;
+    }
+    h->mode_params.assign((h->S + ModeParams::kMax - 1) / ModeParams::kMax, ModeParams());
+    for (int s = 0; s < h->S; ++s) {
+        const AdjConst c = adj_const(h->geo_host[s]);
+        ModeProj &p = h->mode_params[s / ModeParams::kMax].p[s % ModeParams::kMax];
+        for (int t = 0; t < 3; ++t) {
+            p.o[t] = (float)c.oc[1 + t];
+            p.i[t] = (float)c.ic[1 + t];
+        }
+        p.uo = (float)c.uo; p.ui = (float)c.ui; p.vo = (float)c.vo; p.vi = (float)c.vi;
+        p.oh = (float)(0.5 - c.ho);
+        p.au = (float)(c.au + 0.5); p.lu = (float)c.lu;
+        p.av = (float)(c.av + 0.5); p.lv = (float)c.lv;
+        p.so = c.outer_j ? bk : 1;
+        p.si = c.outer_j ? 1 : bk;
+        p.k0 = (int)(0u - (unsigned)kRoundBits * (unsigned)(p.so + p.si));
+        p.lim = bj * bk - 1 - (c.ni - 1) * p.si;
+        p.shape = (c.no <= 3 && c.ni <= 3) ? 16 * c.no + c.ni : 0;
+        p.order = c.no | (c.ni << 8);
+    }
+}
+
+// F[s][m][i]: Fourier coefficients of Y_i along the detector circle, mode m
+// (0: constant; 2t - 1, 2t: cos, sin of t * step times phi), by the 32-point
+// rule on the whole circle (exact: two modes of at most 8 each).
+__global__ void __launch_bounds__(32)
+k_mode_matrix(const double *__restrict__ frames, double cth, double sth, int L, int K, int R, int step,
+              double *__restrict__ F)
+{
+    extern __shared__ double ysh[];   // [32][K]
+    const int s = blockIdx.x, t = threadIdx.x;
+    const double *fr = frames + 9 * s;
+    double sp, cp;
+    sincospi(t / 16.0, &sp, &cp);
+    double q[3];
+    for (int r = 0; r < 3; ++r) q[r] = cth * (cp * fr[3 + r] + sp * fr[6 + r]) - sth * fr[r];
+    sh_even<double>(L, q[0], q[1], q[2], ysh + t * K, 1);
+    __syncthreads();
+    for (int e = t; e < R * K; e += 32) {
+        const int m = e / K, i = e - m * K, f = (m + 1) / 2 * step;
+        double acc = 0.0;
+        for (int n = 0; n < 32; ++n) {
+            double sn, cn;
+            sincospi(((n * f) & 31) / 16.0, &sn, &cn);
+            acc += ysh[n * K + i] * (m == 0 ? 1.0 : ((m & 1) ? cn : sn));
+        }
+        F[((size_t)s * R + m) * K + i] = acc * (m == 0 ? 1.0 : 2.0) / 32.0;
+    }
+}
+
+// The adjoint's B operands: per unit of UP projections two KU x N matrices,
+// for D_lo and D_hi, in K-major core-matrix tiles (8 rows x 16 bytes).  Column
+// k of the unit is slot k % (2 M) of projection k / (2 M): the slots hold the
+// M modes' t_hi, then t_lo; D_lo takes F_lo against t_hi and F_hi against
+// t_lo, D_hi F_hi against t_hi.  The projection's step length is folded in.
+__global__ void k_mode_operand(const double *__restrict__ F, const ProjGeom *__restrict__ geo, int S, int R, int K,
+                               int M, int UP, int KU, int N, float *__restrict__ FB, long long n)
+{
+    for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < n;
+         e += (long long)gridDim.x * blockDim.x) {
+        const int k4 = (int)(e & 3), nn = (int)((e >> 2) & 7);
+        long long r = e >> 5;
+        const int nb = (int)(r % (N / 8));
+        r /= N / 8;
+        const int kc = (int)(r % (KU / 4));
+        r /= KU / 4;
+        const bool dhi = r & 1;
+        const int u = (int)(r >> 1), k = 4 * kc + k4, i = 8 * nb + nn, q = k / (2 * M), slot = k - q * 2 * M;
+        const int s = u * UP + q, m = slot % M;
+        const bool tlo = slot >= M;
+        float v = 0.f;
+        if (q < UP && s < S && m < R && i < K && !(dhi && tlo)) {
+            const double f = F[((size_t)s * R + m) * K + i] * geo[s].step;
+            uint32_t hi, lo;
+            tf32_split((float)f, hi, lo);
+            const float rest = (float)(f - (double)__uint_as_float(hi));
+            v = (dhi || tlo) ? __uint_as_float(hi)
+                             : __uint_as_float((__float_as_uint(rest) + 0x1000u) & 0xffffe000u);
+        }
+        FB[e] = v;
+    }
+}
+
+cudaError_t setup_modes(tt_handle *h, const double *frames)
+{
+    if (!h->R) return cudaSuccess;
+    const int CP = h->CP, R = h->R, step = mode_step(h);
+    std::vector<float> Q((size_t)CP * kModeQ, 0.f);
+    for (int c = 0; c < h->C; ++c)
+        for (int m = 0; m < R; ++m) {
+            double v;
+            if (h->q_identity) {
+                v = c == m ? 1.0 : 0.0;
+            } else if (m == 0) {
+                v = 1.0;
+            } else {   // segment mean of cos(f phi) or sin(f phi)
+                const double f = (m + 1) / 2 * step, half = 0.5 * (h->seg1[c] - h->seg0[c]);
+                const double mid = f * 0.5 * (h->seg1[c] + h->seg0[c]), sinc = std::sin(f * half) / (f * half);
+                v = ((m & 1) ? std::cos(mid) : std::sin(mid)) * sinc;
+            }
+            Q[(size_t)c * kModeQ + m] = (float)v;
+        }
+    cudaError_t e = cudaMemcpyAsync(h->Qm, Q.data(), Q.size() * sizeof(float), cudaMemcpyHostToDevice, h->stream);
+    if (e != cudaSuccess) return e;
+    cudaEvent_t ev;
+    prof_begin(h, TT_KSLOT_BASIS, &ev);
+    const double *F = h->B64;
+    if (!h->q_identity) {
+        const double th = 0.5 * h->two_theta;
+        k_mode_matrix<<<h->S, 32, 32 * h->K * sizeof(double), h->stream>>>(frames, std::cos(th), std::sin(th), h->L,
+                                                                         h->K, R, step, h->F64);
+        F = h->F64;
+    }
+    std::vector<ModeOrigin> org(h->S);
+    for (int s = 0; s < h->S; ++s) {
+        const ProjGeom &g = h->geo_host[s];
+        const AdjConst c = adj_const(g);
+        double jl, jh, kl, kh;
+        block_range(c.jc, jl, jh);
+        block_range(c.kc, kl, kh);
+        for (int t = 0; t < 4; ++t) {
+            org[s].j[t] = c.jc[t];
+            org[s].k[t] = c.kc[t];
+        }
+        org[s].jlo = jl - g.hj - 0.02;
+        org[s].klo = kl - g.hk - 0.02;
+        org[s].outer_j = c.outer_j ? 1 : 0;
+    }
+    e = cudaMemcpyAsync(h->mode_org, org.data(), org.size() * sizeof(ModeOrigin), cudaMemcpyHostToDevice, h->stream);
+    if (e != cudaSuccess) return e;
+    const int M = modes_m(R), UP = modes_up(M), N = modes_n(h->K);
+    const long long n = mode_operand_floats(h);
+    k_mode_operand<<<(unsigned)std::min<long long>((n + 255) / 256, 8LL * h->n_sm), 256, 0, h->stream>>>(
+        F, h->geo, h->S, R, h->K, M, UP, modes_ku(M), N, h->FB, n);
+    e = cudaGetLastError();
+    prof_end(h, TT_KSLOT_BASIS, ev);
+    return e == cudaSuccess ? setup_mode_forward(h, F) : e;
+}
+
+template <int N, int R4, int R1>
+static cudaError_t adjoint_modes_run(tt_handle *h, const float *rows, float *g, bool reduce_loss)
+{
+    constexpr int M = 4 * R4 + R1, UP = modes_up(M), KU = modes_ku(M);
+    const int tx = (h->N[0] + 7) / 8, ty = (h->N[1] + 3) / 4, tz = (h->N[2] + 7) / 8;
+    TmaDesc tm4, tm1;
+    if (!encode_rows(h, rows, 4 * R4, h->nk, &tm4)) return cudaErrorInvalidValue;
+    if (!R1) tm1 = tm4;
+    else if (!encode_rows(h, mode_out(h).G1, 1, h->nk1, &tm1)) return cudaErrorInvalidValue;
+    const auto kern = k_adjoint_modes<N, R4, R1>;
+    const size_t smem = modes_smem(h);
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const int nchunk = (int)h->mode_params.size();
+    for (int ci = 0; ci < nchunk && e == cudaSuccess; ++ci) {
+        const int s0 = ci * ModeParams::kMax, ns = std::min(ModeParams::kMax, h->S - s0);
+        const bool last = ci == nchunk - 1;
+        static_assert(ModeParams::kMax % UP == 0, "launches start on a unit");
+        cudaEvent_t ev;
+        prof_begin(h, TT_KSLOT_ADJOINT, &ev);
+        kern<<<(unsigned)(tx * ty * tz), kModeThreads, smem, h->stream>>>(
+            h->mode_params[ci], tm4, tm1, ns, s0, h->mode_org + s0, h->FB + (size_t)(s0 / UP) * 2 * KU * N, h->box_j,
+            h->box_k, h->N[0], h->N[1], h->N[2], ty, tz, (float *)h->gpad, h->KP, ci > 0 ? 1 : 0, last ? g : nullptr,
+            h->K, h->partials, h->n_fwd_ctas, (reduce_loss && ci == 0) ? h->loss_dev : nullptr,
+            (reduce_loss && ci == 0 && h->loss_publish) ? h->loss_slot_dev : nullptr, h->loss_publish);
+        e = cudaGetLastError();
+        prof_end(h, TT_KSLOT_ADJOINT, ev);
+    }
+    return e;
+}
+
+template <int N>
+static cudaError_t adjoint_modes_n(tt_handle *h, const float *rows, float *g, bool rl)
+{
+    if (h->R4 == 1) return h->R1 ? adjoint_modes_run<N, 1, 1>(h, rows, g, rl) : adjoint_modes_run<N, 1, 0>(h, rows, g, rl);
+    return h->R1 ? adjoint_modes_run<N, 2, 1>(h, rows, g, rl) : adjoint_modes_run<N, 2, 0>(h, rows, g, rl);
+}
+
+cudaError_t launch_adjoint_modes(tt_handle *h, const float *rows, float *g, bool reduce_loss)
+{
+    switch (modes_n(h->K)) {
+    case 16: return adjoint_modes_n<16>(h, rows, g, reduce_loss);
+    case 32: return adjoint_modes_n<32>(h, rows, g, reduce_loss);
+    case 48: return adjoint_modes_n<48>(h, rows, g, reduce_loss);
+    default: return cudaErrorInvalidValue;
+    }
+}
+
+cudaError_t launch_backcontract_modes(tt_handle *h, const float *R)
+{
+    const long long npix = h->npix();
+    const unsigned blocks = (unsigned)((npix + kThreads - 1) / kThreads);
+    float *G4 = (float *)h->G, *G1 = mode_out(h).G1;
+    cudaEvent_t ev;
+    prof_begin(h, TT_KSLOT_BACKCONTRACT, &ev);
+    if (h->R4 == 1 && !h->R1) k_backcontract_modes<1, 0><<<blocks, kThreads, 0, h->stream>>>(h->Qm, R, G4, G1, npix, h->nk, h->nk1, h->C);
+    else if (h->R4 == 1) k_backcontract_modes<1, 1><<<blocks, kThreads, 0, h->stream>>>(h->Qm, R, G4, G1, npix, h->nk, h->nk1, h->C);
+    else if (!h->R1) k_backcontract_modes<2, 0><<<blocks, kThreads, 0, h->stream>>>(h->Qm, R, G4, G1, npix, h->nk, h->nk1, h->C);
+    else k_backcontract_modes<2, 1><<<blocks, kThreads, 0, h->stream>>>(h->Qm, R, G4, G1, npix, h->nk, h->nk1, h->C);
+    cudaError_t e = cudaGetLastError();
+    prof_end(h, TT_KSLOT_BACKCONTRACT, ev);
+    return e;
+}
+
+}  // namespace tt
