@@ -37,7 +37,8 @@ __device__ __forceinline__ void fma2(float &a0, float &a1, float w, float x0, fl
     a1 = r.y;
 }
 
-template <typename T, int CPL>
+// acc += w * row; doubles: of the first USED elements (the others are padding).
+template <typename T, int CPL, int USED = CPL>
 __device__ __forceinline__ void fma_row(T (&acc)[CPL], T w, const T *__restrict__ p)
 {
     if constexpr (sizeof(T) == 4 && CPL % 8 == 0) {
@@ -66,7 +67,7 @@ __device__ __forceinline__ void fma_row(T (&acc)[CPL], T w, const T *__restrict_
     } else {
         static_assert(CPL % 2 == 0, "double rows are read as double2");
 #pragma unroll
-        for (int t = 0; t < CPL / 2; ++t) {
+        for (int t = 0; t < USED / 2; ++t) {
             double2 x = __ldg(reinterpret_cast<const double2 *>(p) + t);
             acc[2 * t + 0] = fma(w, x.x, acc[2 * t + 0]);
             acc[2 * t + 1] = fma(w, x.y, acc[2 * t + 1]);
@@ -112,11 +113,11 @@ __device__ __forceinline__ unsigned pack2(float a, float b, __half *)
     return *reinterpret_cast<unsigned *>(&v);
 }
 
-template <typename T, typename S, int CPL>
+template <typename T, typename S, int CPL, int USED = CPL>
 __device__ __forceinline__ void fma_row_s(T (&acc)[CPL], T w, const S *__restrict__ p)
 {
     if constexpr (std::is_same<T, S>::value) {
-        fma_row<T, CPL>(acc, w, p);
+        fma_row<T, CPL, USED>(acc, w, p);
     } else {
         static_assert(sizeof(S) == 2 && CPL % 4 == 0, "2-byte storage rows are read 4 or 8 elements at a time");
         if constexpr (CPL % 8 == 0) {
@@ -987,6 +988,10 @@ __device__ __forceinline__ void adj_geometry(const AdjVoxel<T> &vx, const AdjPro
     }
 }
 
+// Channels of a lane's chunk worth adding: a lone lane's eight at l_max 2 are
+// six and padding, which double precision, bound by its arithmetic, skips.
+__host__ __device__ constexpr int adjoint_used(int KP, int LG) { return LG == 1 && KP == 8 ? 6 : KP / LG; }
+
 // Candidates of a (NO, NI) window, exchanged by shuffles.
 template <typename T, typename S, int CPL, int KP, int LG, int V, int NO, int NI>
 __device__ __forceinline__ void adj_window(T (&acc)[V][CPL], const S *__restrict__ Gq, const AdjVoxel<T> &vx,
@@ -1005,7 +1010,7 @@ __device__ __forceinline__ void adj_window(T (&acc)[V][CPL], const S *__restrict
 #pragma unroll
             for (int src = 0; src < V; ++src) {
                 const T ws = (LG == 1 || V == 1) ? w[a * NI + b] : __shfl_sync(0xffffffffu, w[a * NI + b], src, LG);
-                if (ws != T(0)) fma_row_s<T, S, CPL>(acc[src], ws, Gq + (long long)(rs[src] + b * si) * KP);
+                if (ws != T(0)) fma_row_s<T, S, CPL, adjoint_used(KP, LG)>(acc[src], ws, Gq + (long long)(rs[src] + b * si) * KP);
             }
         }
     }
@@ -1097,7 +1102,7 @@ __device__ __forceinline__ void adj_window_any(T (&acc)[V][CPL], const S *__rest
             for (int src = 0; src < V; ++src) {
                 const T ws = (LG == 1 || V == 1) ? w : __shfl_sync(0xffffffffu, w, src, LG);
                 const int rs = (LG == 1 || V == 1) ? row : __shfl_sync(0xffffffffu, row, src, LG);
-                if (ws != T(0)) fma_row_s<T, S, CPL>(acc[src], ws, Gq + (long long)rs * KP);
+                if (ws != T(0)) fma_row_s<T, S, CPL, adjoint_used(KP, LG)>(acc[src], ws, Gq + (long long)rs * KP);
             }
         }
     }
@@ -1105,8 +1110,14 @@ __device__ __forceinline__ void adj_window_any(T (&acc)[V][CPL], const S *__rest
 
 // Four resident blocks (64 registers) pay off while a lane's accumulators are
 // 16 floats; larger K keeps three.
-template <typename T, typename S, int KP, int LG, int V>
-__global__ void __launch_bounds__(kThreads, (KP <= 16 ? 4 : 3))
+// Double precision on small volumes: gridDim.y CTAs of a cluster split the
+// projections of a block and add their sums through distributed shared memory
+// in a fixed order (16^3 x 30 projections: 32 blocks left most of the chip
+// idle, each a long chain of slow FP64 arithmetic; adjoint 253 -> 72 us, with
+// two resident CTAs instead of four, whose registers spilled, and voxel blocks
+// 8 long in z instead of 32).
+template <typename T, typename S, int KP, int LG, int V, int GZ = adjoint_gz(LG)>
+__global__ void __launch_bounds__(kThreads, (sizeof(T) == 8 ? 2 : (KP <= 16 ? 4 : 3)))
 k_adjoint(const __grid_constant__ AdjParams<T> P, int ns, const S *__restrict__ G, int nj, int nk, int nx,
           int ny, int nz, int ty, int tz, T *__restrict__ gpad, int accumulate, T *__restrict__ gout, int K,
           const double *__restrict__ loss_partials, long long n_partials, double *__restrict__ loss_out,
@@ -1116,7 +1127,7 @@ k_adjoint(const __grid_constant__ AdjParams<T> P, int ns, const S *__restrict__ 
     // launch on this stream, so visible here without fences) and, given a
     // host-mapped slot, publishes the value there: value, system-scope
     // fence, then the sequence number the host waits for.
-    if (loss_out && blockIdx.x == 0) {
+    if (loss_out && blockIdx.x == 0 && blockIdx.y == 0) {
         __shared__ double lred[32];
         const double v = sum_fixed_order(loss_partials, n_partials, lred);
         if (threadIdx.x == 0) {
@@ -1138,7 +1149,7 @@ k_adjoint(const __grid_constant__ AdjParams<T> P, int ns, const S *__restrict__ 
     // lanes repeat a voxel's geometry so that the accumulators, V * CPL per
     // lane, stay in registers for large K).
     constexpr int GPW = 32 / LG;                   // lane groups per warp
-    constexpr int GZ = adjoint_gz(LG), GX = GPW / GZ, BY = 4, BX = (kThreads / 32) / BY;
+    constexpr int GX = GPW / GZ, BY = 4, BX = (kThreads / 32) / BY;
 
     const int b = blockIdx.x;
     const int bz = b % tz, by = (b / tz) % ty, bx = b / (tz * ty);
@@ -1167,7 +1178,8 @@ k_adjoint(const __grid_constant__ AdjParams<T> P, int ns, const S *__restrict__ 
     // Warps whose voxels all lie outside the volume skip the loop as a whole.
     const bool group_live = (xw < nx) && (y < ny) && (bz * GZ < nz);
     if (group_live) {
-        for (int si = 0; si < ns; ++si) {
+        const int s_end = ns * ((int)blockIdx.y + 1) / (int)gridDim.y;
+        for (int si = ns * (int)blockIdx.y / (int)gridDim.y; si < s_end; ++si) {
             const AdjProj<T> &c = P.p[si];
             AdjVoxel<T> vx;
             vx.oc = c.oc[0] + c.oc[1] * fx + c.oc[2] * fy + c.oc[3] * fz;
@@ -1195,6 +1207,21 @@ k_adjoint(const __grid_constant__ AdjParams<T> P, int ns, const S *__restrict__ 
                 break;
             }
 #undef TT_ADJ_CASE
+        }
+    }
+    if constexpr (std::is_same<T, double>::value) {
+        if (gridDim.y > 1) {
+            extern __shared__ double adj_sums[];           // [V * CPL][kThreads]
+#pragma unroll
+            for (int i = 0; i < V * CPL; ++i) adj_sums[i * kThreads + threadIdx.x] = acc[i / CPL][i % CPL];
+            umma::cluster_sync();
+            if (blockIdx.y == 0)
+                for (int k = 1; k < (int)gridDim.y; ++k)
+#pragma unroll
+                    for (int i = 0; i < V * CPL; ++i)
+                        acc[i / CPL][i % CPL] += umma::cluster_load_f64(umma::smem_u32(adj_sums + i * kThreads + threadIdx.x), k);
+            umma::cluster_sync();                          // no CTA leaves while its sums are read
+            if (blockIdx.y != 0) return;
         }
     }
     // lane q writes channel chunk q of the group's V voxels
@@ -1308,16 +1335,10 @@ cudaError_t launch_backcontract_L(tt_handle *h, const T *R)
     return e;
 }
 
-template <typename T, typename S, int L>
-cudaError_t launch_adjoint_L(tt_handle *h, T *g, bool reduce_loss)
+template <typename T, typename S, int KP, int LG, int V, int GZ>
+cudaError_t launch_adjoint_gz(tt_handle *h, T *g, bool reduce_loss)
 {
-    // For K <= 8 a single lane owns a voxel and reads its whole (32-byte) G
-    // row: no candidate exchange, measured 7% faster than two-lane groups.
-    // (one lane per voxel for K = 15 as well was measured 0.37 -> 0.50 ms
-    // at 64^3: the lane's 16 channels cost the shared weight exchange's
-    // savings back in wavefronts)
-    constexpr int K = num_coeffs(L), KP = padded_k(K), LG = K <= 8 ? 1 : lane_group(K), V = adjoint_voxels(KP, LG);
-    constexpr int GZ = adjoint_gz(LG), BXT = (kThreads / 32 / 4) * (32 / LG / GZ) * V, BY = 4;
+    constexpr int BXT = (kThreads / 32 / 4) * (32 / LG / GZ) * V, BY = 4;
     const int tx = (h->N[0] + BXT - 1) / BXT, ty = (h->N[1] + BY - 1) / BY, tz = (h->N[2] + GZ - 1) / GZ;
     const std::vector<AdjParams<T>> &chunks = adj_params<T>(h);
     const T *G = (const T *)h->G;           // G is kept in T for every storage type
@@ -1327,17 +1348,47 @@ cudaError_t launch_adjoint_L(tt_handle *h, T *g, bool reduce_loss)
         const int s0 = ci * AdjParams<T>::kMax;
         const int ns = std::min(AdjParams<T>::kMax, h->S - s0);
         const bool last = ci == nchunk - 1;
+        int split = 1;
+        if (std::is_same<T, double>::value)
+            while (split < 8 && 2LL * split * tx * ty * tz <= 2 * h->n_sm && ns / (2 * split) >= 2) split *= 2;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3((unsigned)(tx * ty * tz), (unsigned)split);
+        cfg.blockDim = dim3(kThreads);
+        cfg.dynamicSmemBytes = split > 1 ? (size_t)V * (KP / LG) * kThreads * sizeof(T) : 0;
+        cfg.stream = h->stream;
+        cudaLaunchAttribute cluster;
+        cluster.id = cudaLaunchAttributeClusterDimension;
+        cluster.val.clusterDim = {1, (unsigned)split, 1};
+        cfg.attrs = &cluster;
+        cfg.numAttrs = split > 1 ? 1 : 0;
+        const auto kern = k_adjoint<T, T, KP, LG, V, GZ>;
+        if (cfg.dynamicSmemBytes > 32 * 1024)
+            cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cfg.dynamicSmemBytes);
         cudaEvent_t ev;
         prof_begin(h, TT_KSLOT_ADJOINT, &ev);
-        k_adjoint<T, T, KP, LG, V><<<(unsigned)(tx * ty * tz), kThreads, 0, h->stream>>>(
-            chunks[ci], ns, G + (size_t)s0 * h->nj * h->nk * KP, h->nj, h->nk, h->N[0], h->N[1], h->N[2], ty, tz,
-            (T *)h->gpad, ci > 0 ? 1 : 0, last ? g : nullptr, h->K, h->partials, h->n_fwd_ctas,
-            (reduce_loss && ci == 0) ? h->loss_dev : nullptr,
-            (reduce_loss && ci == 0 && h->loss_publish) ? h->loss_slot_dev : nullptr, h->loss_publish);
-        e = cudaGetLastError();
+        e = cudaLaunchKernelEx(
+            &cfg, kern, chunks[ci], ns, G + (size_t)s0 * h->nj * h->nk * KP, h->nj, h->nk, h->N[0], h->N[1], h->N[2], ty, tz,
+            (T *)h->gpad, ci > 0 ? 1 : 0, last ? g : (T *)nullptr, h->K, (const double *)h->partials, h->n_fwd_ctas,
+            (reduce_loss && ci == 0) ? h->loss_dev : (double *)nullptr,
+            (reduce_loss && ci == 0 && h->loss_publish) ? h->loss_slot_dev : (LossSlot *)nullptr, h->loss_publish);
+        (void)cudaGetLastError();
         prof_end(h, TT_KSLOT_ADJOINT, ev);
     }
     return e;
+}
+
+template <typename T, typename S, int L>
+cudaError_t launch_adjoint_L(tt_handle *h, T *g, bool reduce_loss)
+{
+    // For K <= 8 a single lane owns a voxel and reads its whole (32-byte) G
+    // row: no candidate exchange, measured 7% faster than two-lane groups.
+    // (one lane per voxel for K = 15 as well was measured 0.37 -> 0.50 ms
+    // at 64^3: the lane's 16 channels cost the shared weight exchange's
+    // savings back in wavefronts)
+    constexpr int K = num_coeffs(L), KP = padded_k(K), LG = K <= 8 ? 1 : lane_group(K), V = adjoint_voxels(KP, LG);
+    // (double is bound by its arithmetic, idle lanes included: short runs)
+    constexpr int GZ = std::is_same<T, double>::value && LG == 1 ? 8 : adjoint_gz(LG);
+    return launch_adjoint_gz<T, S, KP, LG, V, GZ>(h, g, reduce_loss);
 }
 
 template <typename T, typename S>

@@ -45,7 +45,8 @@ static size_t modes_smem(const tt_handle *h)
     const int M = modes_m(h->R), UP = modes_up(M);
     const uint32_t px = (uint32_t)(h->box_j * h->box_k);
     const size_t boxes = mode_align(px * 16 * h->R4) + (h->R1 ? mode_align(px * 4) : 0);
-    return kModeStages * (UP * boxes + 2 * (size_t)modes_ku(M) * modes_n(h->K) * 4) + 128;
+    const size_t ring = kModeStages * (UP * boxes + 2 * (size_t)modes_ku(M) * modes_n(h->K) * 4);
+    return std::max(ring, (size_t)kModeVox * h->K * 4) + 128;   // (the sums at the end)
 }
 
 // The handle works in modes when there are at most kMaxModes of them, the band
@@ -228,6 +229,26 @@ cudaError_t setup_modes(tt_handle *h, const double *frames)
     return e == cudaSuccess ? setup_mode_forward(h, F) : e;
 }
 
+// CTAs that share a block of voxels (1, 2, 4 or 8, three units each at least):
+// the fewest waves of `slots` resident CTAs, a wave of s-fold split blocks
+// lasting 1/s, each doubling counted as 20% for its sums and ramps (measured 7%
+// at l_max 4, 12% at 8 on full chips, more where it starts another wave).  28^3, l_max 2, 60 projections (112 blocks): 46 -> 30
+// us with 4; 20^3, l_max 4: 60 -> 23; 55 x 65 x 55, l_max 4 (833 blocks on 608
+// slots): 482 -> 434 with 2; 64^3 (1024 on 608) stays whole: 280 / 295 / 312.
+static int mode_split(int blocks, int units, int slots)
+{
+    int best = 1;
+    double least = 1e30, cost = 1.0;
+    for (int s = 1; s <= 8 && (s == 1 || units / s >= 3); s *= 2, cost *= 1.2) {
+        const double t = cost * (((long long)blocks * s + slots - 1) / slots) / s;
+        if (t < 0.999 * least) {
+            least = t;
+            best = s;
+        }
+    }
+    return best;
+}
+
 template <int N, int R4, int R1>
 static cudaError_t adjoint_modes_run(tt_handle *h, const float *rows, float *g, bool reduce_loss)
 {
@@ -245,14 +266,26 @@ static cudaError_t adjoint_modes_run(tt_handle *h, const float *rows, float *g, 
         const int s0 = ci * ModeParams::kMax, ns = std::min(ModeParams::kMax, h->S - s0);
         const bool last = ci == nchunk - 1;
         static_assert(ModeParams::kMax % UP == 0, "launches start on a unit");
+        const int blocks = tx * ty * tz, split = mode_split(blocks, (ns + UP - 1) / UP, h->n_sm * mode_ctas(N));
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3((unsigned)blocks, (unsigned)split);
+        cfg.blockDim = dim3(kModeThreads);
+        cfg.dynamicSmemBytes = smem;
+        cfg.stream = h->stream;
+        cudaLaunchAttribute cluster;
+        cluster.id = cudaLaunchAttributeClusterDimension;
+        cluster.val.clusterDim = {1, (unsigned)split, 1};
+        cfg.attrs = &cluster;
+        cfg.numAttrs = split > 1 ? 1 : 0;
         cudaEvent_t ev;
         prof_begin(h, TT_KSLOT_ADJOINT, &ev);
-        kern<<<(unsigned)(tx * ty * tz), kModeThreads, smem, h->stream>>>(
-            h->mode_params[ci], tm4, tm1, ns, s0, h->mode_org + s0, h->FB + (size_t)(s0 / UP) * 2 * KU * N, h->box_j,
-            h->box_k, h->N[0], h->N[1], h->N[2], ty, tz, (float *)h->gpad, h->KP, ci > 0 ? 1 : 0, last ? g : nullptr,
-            h->K, h->partials, h->n_fwd_ctas, (reduce_loss && ci == 0) ? h->loss_dev : nullptr,
-            (reduce_loss && ci == 0 && h->loss_publish) ? h->loss_slot_dev : nullptr, h->loss_publish);
-        e = cudaGetLastError();
+        e = cudaLaunchKernelEx(
+            &cfg, kern, h->mode_params[ci], tm4, tm1, ns, s0, (const ModeOrigin *)h->mode_org + s0, (const float *)h->FB + (size_t)(s0 / UP) * 2 * KU * N, h->box_j,
+            h->box_k, h->N[0], h->N[1], h->N[2], ty, tz, (float *)h->gpad, h->KP, ci > 0 ? 1 : 0,
+            last ? g : (float *)nullptr, h->K, (const double *)h->partials, h->n_fwd_ctas,
+            (reduce_loss && ci == 0) ? h->loss_dev : (double *)nullptr,
+            (reduce_loss && ci == 0 && h->loss_publish) ? h->loss_slot_dev : (LossSlot *)nullptr, h->loss_publish);
+        (void)cudaGetLastError();
         prof_end(h, TT_KSLOT_ADJOINT, ev);
     }
     return e;

@@ -45,6 +45,10 @@ namespace tt {
 // its columns: the boxes may be refilled) and `empty` (its products are
 // done).  One thread of the last warp issues all copies and products.
 //
+// Volumes of too few blocks to fill the chip split the projections between
+// the CTAs of a cluster (gridDim.y of them), which add their sums through
+// distributed shared memory in a fixed order.
+//
 // Why: gathering K-channel rows moved 75% of what the L1 path can deliver
 // (64^3, l_max 4: 0.366 ms; 128^3, l_max 8: 14.4 ms); R = 5 modes are a third
 // of those bytes, 8 a sixth.  What bounds it now is instruction issue (70% of
@@ -225,7 +229,7 @@ k_adjoint_modes(const __grid_constant__ ModeParams P, const __grid_constant__ Tm
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     // CTA 0 first sums the forward's loss partials (see k_adjoint).
-    if (loss_out && blockIdx.x == 0) {
+    if (loss_out && blockIdx.x == 0 && blockIdx.y == 0) {
         __shared__ double lred[32];
         const double v = sum_fixed_order_half(loss_partials, n_partials, lred);
         if (threadIdx.x == 0) {
@@ -251,7 +255,10 @@ k_adjoint_modes(const __grid_constant__ ModeParams P, const __grid_constant__ Tm
     __syncthreads();
     umma::fence_after_sync();
     const uint32_t tbase = tslot;
-    const int nu = (ns + UP - 1) / UP;
+    // this CTA's share of the units, [u_begin, u_end): the cluster's CTAs split them
+    const int units = (ns + UP - 1) / UP, split = gridDim.y;
+    const int u_begin = units * (int)blockIdx.y / split, nu = units * ((int)blockIdx.y + 1) / split - u_begin;
+    ns = min(ns, (u_begin + nu) * UP);
 
     const int b = blockIdx.x;
     const int X = b / (tz * ty) * 8, Y = (b / tz) % ty * 4, Z = b % tz * 8;
@@ -274,11 +281,11 @@ k_adjoint_modes(const __grid_constant__ ModeParams P, const __grid_constant__ Tm
         };
         // boxes, F operand of unit u into its stage
         auto boxes_of = [&](int u) {
-            const int st = u % kModeStages, n = min(UP, ns - u * UP);
+            const int st = u % kModeStages, s0 = (u_begin + u) * UP, n = min(UP, ns - s0);
             umma::mbar_arrive_expect_tx(&stage[st], n * (box4 + box1));
             for (int q = 0; q < n; ++q) {
                 const uint32_t dst = ring + (st * UP + q) * boxes;
-                const int si = u * UP + q, s = s_base + si;
+                const int si = s0 + q, s = s_base + si;
                 const int jb = __float_as_int(hdr[si & 63].z), kb = __float_as_int(hdr[si & 63].w);
                 umma::tma_load_3d_s(dst, &tm4, 4 * R4 * kb, jb, s, &stage[st]);
                 if constexpr (R1) umma::tma_load_3d_s(dst + box4a, &tm1, kb, jb, s, &stage[st]);
@@ -287,9 +294,9 @@ k_adjoint_modes(const __grid_constant__ ModeParams P, const __grid_constant__ Tm
         auto operand_of = [&](int u) {
             const int st = u % kModeStages;
             umma::mbar_arrive_expect_tx(&stage[st], UB);
-            umma::bulk_g2s_s(fring + st * UB, FB + (size_t)u * (UB / 4), UB, &stage[st]);
+            umma::bulk_g2s_s(fring + st * UB, FB + (size_t)(u_begin + u) * (UB / 4), UB, &stage[st]);
         };
-        origins(0);
+        origins(u_begin * UP);
         if (lane == 0)
             for (int u = 0; u < min(kModeStages, nu); ++u) {
                 boxes_of(u);
@@ -299,7 +306,7 @@ k_adjoint_modes(const __grid_constant__ ModeParams P, const __grid_constant__ Tm
         int u = 0;
         for (; u < nu; ++u) {
             const int st = u % kModeStages, un = u + kModeStages;   // un: the unit fetched in this step
-            if (un * UP % 32 == 0) origins(un * UP);
+            if (un * UP % 32 == 0) origins((u_begin + un) * UP);
             if (lane == 0) {
                 const uint32_t f = fring + st * UB;
                 ok = umma::mbar_wait(&stage[st], (u / kModeStages) & 1, kModeWaitTries) &&
@@ -354,7 +361,7 @@ k_adjoint_modes(const __grid_constant__ ModeParams P, const __grid_constant__ Tm
         bool ok = true;                                            // false once a wait gave up: the rest is NaN
         uint32_t stage_phase = 0, empty_phase = 1, box = ring;
         uint64_t *bar = stage;
-        int drain = 0, si = 0;
+        int drain = 0, si = u_begin * UP;
         for (int u = 0; u < nu; ++u) {
             ok = umma::mbar_wait(bar, stage_phase, ok ? kModeWaitTries : 1) && ok;
 #pragma unroll 1
@@ -435,12 +442,11 @@ k_adjoint_modes(const __grid_constant__ ModeParams P, const __grid_constant__ Tm
         ok = __all_sync(0xffffffffu, umma::mbar_wait(&empty, (nu - 1) & 1, ok ? kModeWaitTries : 1) && ok);
         umma::fence_after_sync();
         // Every warp is past its last box (the products of the last unit are
-        // done), so the ring's start now stages each warp's output rows: a run
-        // of eight voxels along z is 8 K consecutive floats of g.
-        float *so = reinterpret_cast<float *>(smem_modes + (ring - umma::smem_u32(smem_modes))) + warp * (8 * K);
-        const int y = Y + warp, nzv = min(8, nz - Z);
+        // done): the ring's start now takes the voxels' sums, K floats each, so
+        // that a run of eight voxels along z is what g holds of them.
+        const uint32_t row = ring + threadIdx.x * (K * 4);
 #pragma unroll
-        for (int v = 0; v < V; ++v) {
+        for (int v = 0; v < V; ++v)
 #pragma unroll
             for (int i = 0; i < N; i += 16) {
                 float d[16], e[16];
@@ -448,32 +454,43 @@ k_adjoint_modes(const __grid_constant__ ModeParams P, const __grid_constant__ Tm
                 umma::tmem_ld16(tw + v * COLS + KU + N + i, e);
 #pragma unroll
                 for (int k = 0; k < 16; ++k)
-                    acc[v][i + k] = ok ? acc[v][i + k] + (d[k] + e[k]) : __int_as_float(0x7fc00000);
+                    if (i + k < K)
+                        asm volatile("st.shared.f32 [%0], %1;" ::"r"(row + (v * 128 * K + i + k) * 4),
+                                     "f"(ok ? acc[v][i + k] + (d[k] + e[k]) : __int_as_float(0x7fc00000))
+                                     : "memory");
             }
-            for (int r = 0; r < 4; ++r) {
-                const int x = X + 4 * v + r;
-                const bool mine = (lane >> 3) == r && (lane & 7) < nzv;
-                if (x >= nx || y >= ny) break;      // uniform across the warp
-                const long long vox = ((long long)x * ny + y) * nz + Z;
-                if (mine) {
-                    const float *prev = gpad + (vox + (lane & 7)) * KP;
-#pragma unroll
-                    for (int i = 0; i < N; ++i)
-                        if (i < K) so[(lane & 7) * K + i] = accumulate ? acc[v][i] + prev[i] : acc[v][i];
-                }
-                __syncwarp();
-                if (gout) {
-                    for (int i = lane; i < nzv * K; i += 32) gout[vox * K + i] = so[i];
-                } else {
-                    for (int i = lane; i < nzv * K; i += 32) gpad[(vox + i / K) * KP + i % K] = so[i];
-                }
-                __syncwarp();
-            }
-        }
     }
     umma::fence_before_sync();
-    __syncthreads();
+    if (split > 1) umma::cluster_sync();
+    else __syncthreads();
     if (warp == NVW) umma::tmem_dealloc(tbase, 2 * COLS);
+    // The cluster's CTAs share out the runs and add the CTAs' sums in their order.
+    const int nz8 = min(8, nz - Z) * K;
+    if (warp < NVW && Y + warp < ny)
+        for (int r = blockIdx.y; r < 8; r += split) {      // tile r / 4, its x row r % 4
+            const int x = X + r;
+            if (x >= nx) break;
+            const long long vox = ((long long)x * ny + Y + warp) * nz + Z;
+            const uint32_t at = ring + ((r >> 2) * 128 + warp * 32 + (r & 3) * 8) * (K * 4);
+            for (int e = lane; e < nz8; e += 32) {
+                float sum;
+                if (split == 1) {
+                    asm volatile("ld.shared.f32 %0, [%1];" : "=f"(sum) : "r"(at + 4 * e) : "memory");
+                } else {
+                    sum = umma::cluster_load(at + 4 * e, 0);
+                    for (int k = 1; k < split; ++k) sum += umma::cluster_load(at + 4 * e, k);
+                }
+                if (gout && !accumulate) {
+                    gout[vox * K + e] = sum;
+                } else {
+                    const long long o = (vox + e / K) * KP + e % K;
+                    if (accumulate) sum += gpad[o];
+                    if (gout) gout[vox * K + e] = sum;
+                    else gpad[o] = sum;
+                }
+            }
+        }
+    if (split > 1) umma::cluster_sync();                   // no CTA leaves while its sums are read
 }
 
 // ------------------------------------------------- back-contraction to modes

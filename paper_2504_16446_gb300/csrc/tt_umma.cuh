@@ -167,6 +167,33 @@ __device__ __forceinline__ void mbar_arrive_expect_tx(uint64_t *mbar, uint32_t b
                  : "memory");
 }
 
+// All CTAs of the cluster (one CTA when the launch has no clusters): shared
+// memory written before is readable by the others after.
+__device__ __forceinline__ void cluster_sync()
+{
+    asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// A float at shared-memory address a of the cluster's CTA `rank`.
+__device__ __forceinline__ float cluster_load(uint32_t a, uint32_t rank)
+{
+    float v;
+    asm volatile("{\n.reg .b32 r;\nmapa.shared::cluster.u32 r, %1, %2;\nld.shared::cluster.f32 %0, [r];\n}"
+                 : "=f"(v)
+                 : "r"(a), "r"(rank)
+                 : "memory");
+    return v;
+}
+
+__device__ __forceinline__ double cluster_load_f64(uint32_t a, uint32_t rank)
+{
+    double v;
+    asm volatile("{\n.reg .b32 r;\nmapa.shared::cluster.u32 r, %1, %2;\nld.shared::cluster.f64 %0, [r];\n}"
+                 : "=d"(v)
+                 : "r"(a), "r"(rank)
+                 : "memory");
+    return v;
+}
+
 // Bulk asynchronous copy of `bytes` (a multiple of 16; both addresses 16-byte
 // aligned) from global to this CTA's shared memory, completing as
 // transaction bytes on the mbarrier.
