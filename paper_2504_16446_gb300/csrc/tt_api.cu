@@ -423,7 +423,7 @@ static void free_handle(tt_handle *h)
 {
     if (!h) return;
     cudaFree(h->geo); cudaFree(h->tmaps); cudaFree(h->B64); cudaFree(h->Bp); cudaFree(h->cpad); cudaFree(h->gpad);
-    cudaFree(h->G); cudaFree(h->Qm); cudaFree(h->F64); cudaFree(h->FB); cudaFree(h->mode_org); cudaFree(h->FM); cudaFree(h->order); cudaFree(h->slots); cudaFree(h->partials); cudaFree(h->loss_dev); cudaFree(h->red);
+    cudaFree(h->G); cudaFree(h->Qm); cudaFree(h->nonfinite); cudaFree(h->F64); cudaFree(h->FB); cudaFree(h->mode_org); cudaFree(h->FM); cudaFree(h->order); cudaFree(h->slots); cudaFree(h->partials); cudaFree(h->loss_dev); cudaFree(h->red);
     cudaFree(h->hc); cudaFree(h->hI); cudaFree(h->hW); cudaFree(h->hg);
     for (cudaEvent_t e : h->chunk_ready) cudaEventDestroy(e);
     if (h->copy_stream) cudaStreamDestroy(h->copy_stream);
@@ -569,6 +569,7 @@ static tt_status adjoint_impl(tt_handle *h, const T *R, T *g)
         // the modes are the segments and R already has their row layout:
         // nothing to contract
         if (h->R && h->q_identity && h->R == 4 * h->R4) {
+            TT_CUDA(launch_check_rows(h, R), "check");
             TT_CUDA(launch_adjoint_modes(h, R, g, false), "adjoint");
             return TT_OK;
         }
@@ -617,6 +618,7 @@ tt_status tt_grad_enqueue(tt_handle *h, const T *c, const T *I, const T *W, T *g
         // evaluation is the back-projection of the data alone
         if (c) TT_CUDA((launch_pack<T, S>(h, c)), "pack");
         const ZeroVolume zero(h, c == nullptr);
+        ++h->rows_id;
         TT_CUDA((launch_forward<T, S>(h, nullptr, I, W, true)), "forward");
         // the adjoint's first CTA reduces the loss partials; without a
         // gradient a one-CTA reduction does
@@ -800,6 +802,7 @@ tt_status tt_create(const tt_problem *P, tt_precision prec, void *stream, tt_han
     plan_modes(h);
     if (h->R) {
         ALLOC(h->Qm, sizeof(float) * h->CP * kModeQ);
+        ALLOC(h->nonfinite, sizeof(unsigned));
         if (!h->q_identity) ALLOC(h->F64, sizeof(double) * h->S * h->R * h->K);
         ALLOC(h->FB, sizeof(float) * mode_operand_floats(h));
         ALLOC(h->mode_org, sizeof(ModeOrigin) * h->S);
@@ -1017,6 +1020,7 @@ tt_status tt_gradient_residual_host(tt_handle *h, const float *c_host, const flo
         TT_CUDA(cudaEventRecord(packed, main_stream), "event");
         for (int t = 0; t < 2; ++t) TT_CUDA(cudaStreamWaitEvent(h->side[t], packed, 0), "stream wait");
         cudaError_t e = cudaSuccess;
+        ++h->rows_id;
         for (int q = 0; q < Q && e == cudaSuccess; ++q) {
             const int s0 = (int)((long long)h->S * q / Q), s1 = (int)((long long)h->S * (q + 1) / Q);
             e = cudaStreamWaitEvent(h->side[h->fwd_modes ? 0 : q & 1], h->chunk_ready[q], 0);

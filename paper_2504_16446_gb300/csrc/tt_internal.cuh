@@ -130,6 +130,8 @@ struct ModeOut {
     const float *Q = nullptr;
     float *G1 = nullptr;
     int row = 0, nk1 = 0;             // nk1: row pitch of G1 (the detector's nk rounded up to 4)
+    unsigned *nonfinite = nullptr;    // set to rows_id when a value written is not finite
+    unsigned rows_id = 0;
 };
 
 // Layout of the R modes of a ray or voxel: rows of 4 * R4 floats and, with R1,
@@ -259,6 +261,8 @@ struct tt_handle {
     int R = 0, R4 = 0, R1 = 0;
     bool q_identity = false;             // the modes are the segments (Q = 1)
     float *Qm = nullptr;                 // device [CP][kModeQ], zero padded
+    unsigned *nonfinite = nullptr;       // device: the last rows_id whose rows were not all finite
+    unsigned rows_id = 0;                // number of the rows in G (a new one for each that are written)
     double *F64 = nullptr;               // device [S][R][K]: F_s
     float *FB = nullptr;                 // device: F_s as the adjoint's tensor-core operand
     tt::ModeOrigin *mode_org = nullptr;  // device [S]
@@ -464,6 +468,8 @@ cudaError_t launch_forward_modes(tt_handle *h, float *Iout, const float *I, cons
 // rows: the mode rows [S][nj][nk][4 R4] (h->G, or a caller's array).
 cudaError_t launch_adjoint_modes(tt_handle *h, const float *rows, float *g, bool reduce_loss);
 cudaError_t launch_backcontract_modes(tt_handle *h, const float *R);
+// Notes whether a caller's rows are all finite, as the kernels that write rows do.
+cudaError_t launch_check_rows(tt_handle *h, const float *rows);
 inline ModeOut mode_out(const tt_handle *h)
 {
     ModeOut m;
@@ -471,6 +477,8 @@ inline ModeOut mode_out(const tt_handle *h)
         m.Q = h->Qm;
         m.row = 4 * h->R4;
         m.nk1 = h->nk1;
+        m.nonfinite = h->nonfinite;
+        m.rows_id = h->rows_id;
         m.G1 = h->R1 ? (float *)h->G + h->npix() * m.row : nullptr;
     }
     return m;

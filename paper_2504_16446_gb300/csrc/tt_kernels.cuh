@@ -346,6 +346,16 @@ __device__ __forceinline__ void stage_modes(float *Qs, const float *Q, int CP)
     }
 }
 
+// Whether all of v is finite (0 * v is 0 for finite v only).
+template <typename T, int N>
+__device__ __forceinline__ bool rows_finite(const T (&v)[N])
+{
+    T s = T(0);
+#pragma unroll
+    for (int i = 0; i < N; ++i) s = fma(v[i], T(0), s);
+    return s == T(0);
+}
+
 // What a forward kernel does with a marched ray: PROJECT writes the segment
 // intensities; GRAD forms the residual, its square and its back-contraction
 // into the K channels, GRAD_MODES into the detector modes (tt_modes.cuh).
@@ -462,7 +472,9 @@ __device__ __forceinline__ T forward_epilogue(const T (&acc)[CPL], int q, int ch
                 const int m = q + i * LG;
                 if (m < mo.row) G[pix * mo.row + m] = T(2) * gm[i];
                 else if (m == mo.row && mo.G1) mo.G1[pix1] = 2.f * (float)gm[i];
+                gm[i] *= T(2);
             }
+            if (!rows_finite(gm)) *mo.nonfinite = mo.rows_id;
         }
     }
     return lossr;

@@ -192,7 +192,9 @@ cudaError_t setup_modes(tt_handle *h, const double *frames)
             }
             Q[(size_t)c * kModeQ + m] = (float)v;
         }
-    cudaError_t e = cudaMemcpyAsync(h->Qm, Q.data(), Q.size() * sizeof(float), cudaMemcpyHostToDevice, h->stream);
+    cudaError_t e = cudaMemsetAsync(h->nonfinite, 0, sizeof(unsigned), h->stream);   // (rows_id starts at 1)
+    if (e != cudaSuccess) return e;
+    e = cudaMemcpyAsync(h->Qm, Q.data(), Q.size() * sizeof(float), cudaMemcpyHostToDevice, h->stream);
     if (e != cudaSuccess) return e;
     cudaEvent_t ev;
     prof_begin(h, TT_KSLOT_BASIS, &ev);
@@ -284,7 +286,8 @@ static cudaError_t adjoint_modes_run(tt_handle *h, const float *rows, float *g, 
             h->box_k, h->N[0], h->N[1], h->N[2], ty, tz, (float *)h->gpad, h->KP, ci > 0 ? 1 : 0,
             last ? g : (float *)nullptr, h->K, (const double *)h->partials, h->n_fwd_ctas,
             (reduce_loss && ci == 0) ? h->loss_dev : (double *)nullptr,
-            (reduce_loss && ci == 0 && h->loss_publish) ? h->loss_slot_dev : (LossSlot *)nullptr, h->loss_publish);
+            (reduce_loss && ci == 0 && h->loss_publish) ? h->loss_slot_dev : (LossSlot *)nullptr, h->loss_publish,
+            (const unsigned *)h->nonfinite, h->rows_id);
         (void)cudaGetLastError();
         prof_end(h, TT_KSLOT_ADJOINT, ev);
     }
@@ -308,17 +311,49 @@ cudaError_t launch_adjoint_modes(tt_handle *h, const float *rows, float *g, bool
     }
 }
 
+// Rows that are their caller's own (the modes are the segments): are they finite?
+__global__ void __launch_bounds__(kThreads)
+k_check_rows(const float4 *__restrict__ rows, long long n, unsigned *__restrict__ nonfinite, unsigned rows_id)
+{
+    bool ok = true;
+    const long long stride = (long long)gridDim.x * kThreads;
+    for (long long i = (long long)blockIdx.x * kThreads + threadIdx.x; i < n; i += 4 * stride) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            if (i + k * stride >= n) break;
+            const float4 v = __ldg(rows + i + k * stride);
+            const float w[4] = {v.x, v.y, v.z, v.w};
+            ok = ok && rows_finite(w);
+        }
+    }
+    if (!ok) *nonfinite = rows_id;
+}
+
+cudaError_t launch_check_rows(tt_handle *h, const float *rows)
+{
+    const long long n = h->npix() * h->R4;
+    ++h->rows_id;
+    cudaEvent_t ev;
+    prof_begin(h, TT_KSLOT_BACKCONTRACT, &ev);
+    k_check_rows<<<(unsigned)std::min<long long>((n + 4 * kThreads - 1) / (4 * kThreads), 8LL * h->n_sm), kThreads, 0,
+                   h->stream>>>(reinterpret_cast<const float4 *>(rows), n, h->nonfinite, h->rows_id);
+    const cudaError_t e = cudaGetLastError();
+    prof_end(h, TT_KSLOT_BACKCONTRACT, ev);
+    return e;
+}
+
 cudaError_t launch_backcontract_modes(tt_handle *h, const float *R)
 {
     const long long npix = h->npix();
     const unsigned blocks = (unsigned)((npix + kThreads - 1) / kThreads);
     float *G4 = (float *)h->G, *G1 = mode_out(h).G1;
+    ++h->rows_id;
     cudaEvent_t ev;
     prof_begin(h, TT_KSLOT_BACKCONTRACT, &ev);
-    if (h->R4 == 1 && !h->R1) k_backcontract_modes<1, 0><<<blocks, kThreads, 0, h->stream>>>(h->Qm, R, G4, G1, npix, h->nk, h->nk1, h->C);
-    else if (h->R4 == 1) k_backcontract_modes<1, 1><<<blocks, kThreads, 0, h->stream>>>(h->Qm, R, G4, G1, npix, h->nk, h->nk1, h->C);
-    else if (!h->R1) k_backcontract_modes<2, 0><<<blocks, kThreads, 0, h->stream>>>(h->Qm, R, G4, G1, npix, h->nk, h->nk1, h->C);
-    else k_backcontract_modes<2, 1><<<blocks, kThreads, 0, h->stream>>>(h->Qm, R, G4, G1, npix, h->nk, h->nk1, h->C);
+    if (h->R4 == 1 && !h->R1) k_backcontract_modes<1, 0><<<blocks, kThreads, 0, h->stream>>>(h->Qm, R, G4, G1, npix, h->nk, h->nk1, h->C, h->nonfinite, h->rows_id);
+    else if (h->R4 == 1) k_backcontract_modes<1, 1><<<blocks, kThreads, 0, h->stream>>>(h->Qm, R, G4, G1, npix, h->nk, h->nk1, h->C, h->nonfinite, h->rows_id);
+    else if (!h->R1) k_backcontract_modes<2, 0><<<blocks, kThreads, 0, h->stream>>>(h->Qm, R, G4, G1, npix, h->nk, h->nk1, h->C, h->nonfinite, h->rows_id);
+    else k_backcontract_modes<2, 1><<<blocks, kThreads, 0, h->stream>>>(h->Qm, R, G4, G1, npix, h->nk, h->nk1, h->C, h->nonfinite, h->rows_id);
     cudaError_t e = cudaGetLastError();
     prof_end(h, TT_KSLOT_BACKCONTRACT, ev);
     return e;

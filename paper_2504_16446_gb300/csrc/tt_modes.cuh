@@ -40,6 +40,11 @@ namespace tt {
 // their FP32 rounding is that of numbers below 32 instead of the detector's
 // size.
 //
+// The kernel that wrote the rows says whether all of them are finite (it
+// leaves its number in *nonfinite otherwise); if not, rays of zero weight are
+// skipped by a branch, else they are added like the others (0.278 -> 0.257 ms
+// at 64^3 against predicated sums).
+//
 // Units of UP projections pass through three barriers: `stage` (boxes and F
 // operand arrived), `full` (a tile's warps have gathered the unit and stored
 // its columns: the boxes may be refilled) and `empty` (its products are
@@ -73,29 +78,15 @@ __device__ __forceinline__ void mode_load(ModeRow<R4, R1> &x, uint32_t a4, uint3
     if constexpr (R1) asm("ld.shared.f32 %0, [%1];" : "=f"(x.v[4 * R4]) : "r"(a1));
 }
 
-// t += w * x where w > 0: a ray of zero weight must not be touched, it may
-// hold an infinity.
-template <int R4, int R1>
+// t += w * x, as paired FMAs.  GUARD: only where w > 0 -- a ray of zero weight
+// must not be touched when it may hold an infinity or NaN.
+template <int R4, int R1, bool GUARD>
 __device__ __forceinline__ void mode_fma(ModeRow<R4, R1> &t, float w, const ModeRow<R4, R1> &x)
 {
-    if constexpr (R4 == 1 && R1)
-        asm("{\n.reg .pred p;\nsetp.gt.f32 p, %5, 0f00000000;\n@p fma.rn.f32 %0, %5, %6, %0;\n"
-            "@p fma.rn.f32 %1, %5, %7, %1;\n@p fma.rn.f32 %2, %5, %8, %2;\n@p fma.rn.f32 %3, %5, %9, %3;\n"
-            "@p fma.rn.f32 %4, %5, %10, %4;\n}"
-            : "+f"(t.v[0]), "+f"(t.v[1]), "+f"(t.v[2]), "+f"(t.v[3]), "+f"(t.v[4])
-            : "f"(w), "f"(x.v[0]), "f"(x.v[1]), "f"(x.v[2]), "f"(x.v[3]), "f"(x.v[4]));
-    else {
+    if (GUARD && !(w > 0.f)) return;
 #pragma unroll
-        for (int i = 0; i < R4; ++i)
-            asm("{\n.reg .pred p;\nsetp.gt.f32 p, %4, 0f00000000;\n@p fma.rn.f32 %0, %4, %5, %0;\n"
-                "@p fma.rn.f32 %1, %4, %6, %1;\n@p fma.rn.f32 %2, %4, %7, %2;\n@p fma.rn.f32 %3, %4, %8, %3;\n}"
-                : "+f"(t.v[4 * i]), "+f"(t.v[4 * i + 1]), "+f"(t.v[4 * i + 2]), "+f"(t.v[4 * i + 3])
-                : "f"(w), "f"(x.v[4 * i]), "f"(x.v[4 * i + 1]), "f"(x.v[4 * i + 2]), "f"(x.v[4 * i + 3]));
-        if constexpr (R1)
-            asm("{\n.reg .pred p;\nsetp.gt.f32 p, %1, 0f00000000;\n@p fma.rn.f32 %0, %1, %2, %0;\n}"
-                : "+f"(t.v[4 * R4])
-                : "f"(w), "f"(x.v[4 * R4]));
-    }
+    for (int i = 0; i < 4 * R4; i += 2) fma2(t.v[i], t.v[i + 1], w, x.v[i], x.v[i + 1]);
+    if constexpr (R1) t.v[4 * R4] = fmaf(w, x.v[4 * R4], t.v[4 * R4]);
 }
 
 // Integers as floats: for |x| < 2^22, x + kRound has round(x) in its low bits.
@@ -143,12 +134,12 @@ __device__ __forceinline__ void mode_gather(ModeRow<R4, R1> &t, const float4 &cu
 #pragma unroll
         for (int b = 0; b < NI; ++b) mode_load<R4, R1>(x[b], k.a4 + b * ci.y * (16 * R4), k.a1 + b * ci.y * 4);
 #pragma unroll
-        for (int b = 0; b < NI; ++b) mode_fma<R4, R1>(t, mode_weight(cu, k, b), x[b]);
+        for (int b = 0; b < NI; ++b) mode_fma<R4, R1, false>(t, mode_weight(cu, k, b), x[b]);
     }
 }
 
-// Windows of any size (unequal voxel and pixel sizes).
-template <int R4, int R1>
+// Windows of any size (unequal voxel and pixel sizes), and guarded.
+template <int R4, int R1, bool GUARD>
 __device__ __forceinline__ void mode_gather_any(ModeRow<R4, R1> &t, const float4 &cu, const float4 &ce, const int4 &ci,
                                                 float d0, float ic, int orow0, uint32_t b4, uint32_t b1, int order)
 {
@@ -158,7 +149,7 @@ __device__ __forceinline__ void mode_gather_any(ModeRow<R4, R1> &t, const float4
         for (int b = 0; b < NI; ++b) {
             ModeRow<R4, R1> x;
             mode_load<R4, R1>(x, k.a4 + b * ci.y * (16 * R4), k.a1 + b * ci.y * 4);
-            mode_fma<R4, R1>(t, mode_weight(cu, k, b), x);
+            mode_fma<R4, R1, GUARD>(t, mode_weight(cu, k, b), x);
         }
     }
 }
@@ -212,7 +203,7 @@ k_adjoint_modes(const __grid_constant__ ModeParams P, const __grid_constant__ Tm
                 const float *__restrict__ FB, int bj, int bk, int nx, int ny, int nz, int ty, int tz,
                 float *__restrict__ gpad, int KP, int accumulate, float *__restrict__ gout, int K,
                 const double *__restrict__ loss_partials, long long n_partials, double *__restrict__ loss_out,
-                LossSlot *loss_slot, unsigned long long loss_seq)
+                LossSlot *loss_slot, unsigned long long loss_seq, const unsigned *__restrict__ nonfinite, unsigned rows_id)
 {
     constexpr int M = 4 * R4 + R1, SW = 2 * M, UP = modes_up(M), KU = modes_ku(M), V = 2, NVW = kModeVox / V / 32;
     constexpr int kDrain = (N == 16 ? 4 : 8) / UP;                // units per D_hi chain
@@ -359,6 +350,7 @@ k_adjoint_modes(const __grid_constant__ ModeParams P, const __grid_constant__ Tm
             umma::tmem_wait_st();
         }
         bool ok = true;                                            // false once a wait gave up: the rest is NaN
+        const bool guard = *nonfinite == rows_id;                  // some row is not finite
         uint32_t stage_phase = 0, empty_phase = 1, box = ring;
         uint64_t *bar = stage;
         int drain = 0, si = u_begin * UP;
@@ -395,14 +387,19 @@ k_adjoint_modes(const __grid_constant__ ModeParams P, const __grid_constant__ Tm
         _Pragma("unroll") for (int v = 0; v < V; ++v)                                                       \
             mode_gather<R4, R1, NO_, NI_>(t[v], cu, ce, ci, d0[v], ic[v], orow[v], b4, b1);                 \
         break;
-                    switch (c.shape) {
+                    switch (guard ? -1 : c.shape) {
                     TT_MODE_CASE(1, 1) TT_MODE_CASE(1, 2) TT_MODE_CASE(1, 3)
                     TT_MODE_CASE(2, 1) TT_MODE_CASE(2, 2) TT_MODE_CASE(2, 3)
                     TT_MODE_CASE(3, 1) TT_MODE_CASE(3, 2) TT_MODE_CASE(3, 3)
+                    case 0:
+#pragma unroll
+                        for (int v = 0; v < V; ++v)
+                            mode_gather_any<R4, R1, false>(t[v], cu, ce, ci, d0[v], ic[v], orow[v], b4, b1, c.order);
+                        break;
                     default:
 #pragma unroll
                         for (int v = 0; v < V; ++v)
-                            mode_gather_any<R4, R1>(t[v], cu, ce, ci, d0[v], ic[v], orow[v], b4, b1, c.order);
+                            mode_gather_any<R4, R1, true>(t[v], cu, ce, ci, d0[v], ic[v], orow[v], b4, b1, c.order);
                         break;
                     }
 #undef TT_MODE_CASE
@@ -498,7 +495,8 @@ k_adjoint_modes(const __grid_constant__ ModeParams P, const __grid_constant__ Tm
 template <int R4, int R1>
 __global__ void __launch_bounds__(kThreads)
 k_backcontract_modes(const float *__restrict__ Q /*[C][kModeQ]*/, const float *__restrict__ R, float *__restrict__ G4,
-                     float *__restrict__ G1, long long npix, int nk, int nk1, int C)
+                     float *__restrict__ G1, long long npix, int nk, int nk1, int C, unsigned *__restrict__ nonfinite,
+                     unsigned rows_id)
 {
     const long long pix = (long long)blockIdx.x * kThreads + threadIdx.x;
     if (pix >= npix) return;
@@ -526,6 +524,7 @@ k_backcontract_modes(const float *__restrict__ Q /*[C][kModeQ]*/, const float *_
     for (int i = 0; i < R4; ++i)
         reinterpret_cast<float4 *>(G4 + pix * (4 * R4))[i] = make_float4(t[4 * i], t[4 * i + 1], t[4 * i + 2], t[4 * i + 3]);
     if constexpr (R1) G1[pix / nk * nk1 + pix % nk] = t[4 * R4];
+    if (!rows_finite(t)) *nonfinite = rows_id;
 }
 
 }  // namespace tt

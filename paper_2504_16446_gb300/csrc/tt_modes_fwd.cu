@@ -153,7 +153,7 @@ k_march_modes(const ProjGeom *__restrict__ geo, const int *__restrict__ order, c
               long long slot_floats, long long slot_vox, int nx, int ny, int nz, int nj, int nk, int C, int CP,
               int tiles_k, const float *__restrict__ Q, float *__restrict__ Iout, const float *__restrict__ Id,
               const float *__restrict__ Wd, float *__restrict__ G, float *__restrict__ G1, int nk1,
-              double *__restrict__ partials)
+              double *__restrict__ partials, unsigned *__restrict__ nonfinite, unsigned rows_id)
 {
     constexpr int R4 = M / 4, R1 = M & 1;
     constexpr bool GRAD = MODE != kProject;
@@ -321,6 +321,7 @@ k_march_modes(const ProjGeom *__restrict__ geo, const int *__restrict__ order, c
             if constexpr (R1)
                 if (h == 1) G1[((long long)s * nj + j) * nk1 + k] = gm[M - 1];
         }
+        if (valid && !rows_finite(gm)) *nonfinite = rows_id;
         const double tot = dot2_block_sum(Dot2{h == 0 && valid ? loss : 0.f, 0.f}, red);
         if (threadIdx.x == 0) partials[(long long)s * gridDim.x + blockIdx.x] = tot;
     }
@@ -363,7 +364,7 @@ static cudaError_t run_march(tt_handle *h, const int *order, int n, const float 
     prof_begin(h, TT_KSLOT_FORWARD, &ev);
     k_march_modes<M, MODE><<<dim3(tiles_k * tiles_j, n), kMarchThreads, h->CP * kModeQ * 4, h->stream>>>(
         h->geo, order, slots, h->slot_floats, h->slot_vox, h->N[0], h->N[1], h->N[2], h->nj, h->nk, h->C, h->CP, tiles_k,
-        mo.Q, Iout, I, W, (float *)h->G, mo.G1, mo.nk1, h->partials);
+        mo.Q, Iout, I, W, (float *)h->G, mo.G1, mo.nk1, h->partials, mo.nonfinite, mo.rows_id);
     const cudaError_t e = cudaGetLastError();
     prof_end(h, TT_KSLOT_FORWARD, ev);
     return e;

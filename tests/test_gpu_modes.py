@@ -108,3 +108,10 @@ def test_a_nonfinite_ray_reaches_only_its_voxels(ell, seg):
     bad, bad64 = ~torch.isfinite(h.adjoint(R)), ~torch.isfinite(ref.adjoint(R.double()))
     assert bad.any() and not bad.all()
     assert torch.equal(bad.any(-1), bad64.any(-1))
+    # the residual of such data, and finite data right after it on the same handle
+    c = torch.randn(st.volume_shape, device="cuda")
+    _, g = h.gradient_residual(c, R, check=False)
+    _, g64 = ref.gradient_residual(c.double(), R.double(), check=False)
+    assert torch.equal((~torch.isfinite(g)).any(-1), (~torch.isfinite(g64)).any(-1))
+    R = torch.nan_to_num(R, nan=0.0, posinf=0.0)
+    assert rel(h.gradient_residual(c, R)[1], ref.gradient_residual(c.double(), R.double())[1]) <= TOL
