@@ -7,22 +7,78 @@
 
 namespace tt {
 
-// value = sum c^2, grad = 2 c.  Grid-stride; per-block FP64 partials.
+// Four elements as 16-byte accesses (two for double), and their number.
+__device__ __forceinline__ void reg_load(const float *p, float (&v)[4])
+{
+    const float4 a = __ldg(reinterpret_cast<const float4 *>(p));
+    v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
+}
+__device__ __forceinline__ void reg_load(const double *p, double (&v)[4])
+{
+    const double2 a = __ldg(reinterpret_cast<const double2 *>(p)), b = __ldg(reinterpret_cast<const double2 *>(p) + 1);
+    v[0] = a.x; v[1] = a.y; v[2] = b.x; v[3] = b.y;
+}
+__device__ __forceinline__ void reg_store(float *p, const float (&v)[4])
+{
+    *reinterpret_cast<float4 *>(p) = make_float4(v[0], v[1], v[2], v[3]);
+}
+__device__ __forceinline__ void reg_store(double *p, const double (&v)[4])
+{
+    reinterpret_cast<double2 *>(p)[0] = make_double2(v[0], v[1]);
+    reinterpret_cast<double2 *>(p)[1] = make_double2(v[2], v[3]);
+}
+
+// Sum of a value per element: compensated FP32 per thread and across the CTA
+// for float, FP64 for double.
+template <typename T>
+struct RegSum {
+    Dot2 a = {0.f, 0.f};
+    double v = 0.0;
+    __device__ __forceinline__ void add(T x)
+    {
+        if constexpr (std::is_same<T, float>::value) dot2_add1(a, x);
+        else v += x;
+    }
+    __device__ __forceinline__ void square(T x)
+    {
+        if constexpr (std::is_same<T, float>::value) dot2_add(a, x, x);
+        else v = fma(x, x, v);
+    }
+    __device__ __forceinline__ double total(double *red) const
+    {
+        if constexpr (std::is_same<T, float>::value) return dot2_block_sum(a, reinterpret_cast<Dot2 *>(red));
+        else return block_sum(v, red);
+    }
+};
+
+// value = sum c^2, grad = 2 c.  Grid-stride over quads (the entry points take
+// 16-byte aligned c and grad only), the last n % 4 elements by themselves;
+// per-block FP64 partials.  Bound by its reads and writes (100^3, 28 channels:
+// 86 -> 80 us in the whole call).
 template <typename T>
 __global__ void k_l2(const T *__restrict__ c, long long n, T *__restrict__ grad, double *__restrict__ partials)
 {
     __shared__ double red[32];
-    double v = 0.0;
-    Dot2 a = {0.f, 0.f};           // float: compensated FP32 per thread and across the CTA
-    for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < n;
-         t += (long long)gridDim.x * blockDim.x) {
-        const T x = c[t];
-        if constexpr (std::is_same<T, float>::value) dot2_add(a, x, x);
-        else v = fma(x, x, v);
-        if (grad) grad[t] = T(2) * x;
+    RegSum<T> sum;
+    const long long n4 = n / 4, stride = (long long)gridDim.x * blockDim.x;
+    const long long t0 = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+#pragma unroll 4
+    for (long long q = t0; q < n4; q += stride) {
+        T x[4];
+        reg_load(c + 4 * q, x);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            sum.square(x[k]);
+            x[k] *= T(2);
+        }
+        if (grad) reg_store(grad + 4 * q, x);
     }
-    if constexpr (std::is_same<T, float>::value) v = dot2_block_sum(a, reinterpret_cast<Dot2 *>(red));
-    else v = block_sum(v, red);
+    for (long long i = 4 * n4 + t0; i < n; i += stride) {
+        const T x = c[i];
+        sum.square(x);
+        if (grad) grad[i] = T(2) * x;
+    }
+    const double v = sum.total(red);
     if (threadIdx.x == 0) partials[blockIdx.x] = v;
 }
 
@@ -31,18 +87,10 @@ __global__ void k_l2(const T *__restrict__ c, long long n, T *__restrict__ grad,
 //   value = sum H(t), H(t) = t^2/(2 delta) (t <= delta) or t - delta/2,
 //   grad_i(y) = sum_{d: y_d >= 1} w(y - e_d) g_i(y - e_d)_d - w(y) sum_d g_i(y)_d,
 //   w = H'(t)/t = 1/delta (t <= delta) or 1/t.
-// One thread per (voxel, channel); neighbours come through L1.
 template <typename T>
-__device__ __forceinline__ void tv_point(const T *__restrict__ c, int x, int y, int z, int nx, int ny, int nz,
-                                         int K, int i, T inv_delta, T delta, T (&g)[3], T &w, T &H)
+__device__ __forceinline__ void tv_point(T g0, T g1, T g2, T inv_delta, T delta, T &w, T &H)
 {
-    const long long sx = (long long)ny * nz * K, sy = (long long)nz * K, sz = K;
-    const T *p = c + (((long long)x * ny + y) * nz + z) * K + i;
-    const T c0 = __ldg(p);
-    g[0] = (x + 1 < nx) ? __ldg(p + sx) - c0 : T(0);
-    g[1] = (y + 1 < ny) ? __ldg(p + sy) - c0 : T(0);
-    g[2] = (z + 1 < nz) ? __ldg(p + sz) - c0 : T(0);
-    const T t = sqrt(g[0] * g[0] + g[1] * g[1] + g[2] * g[2]);
+    const T t = sqrt(g0 * g0 + g1 * g1 + g2 * g2);
     if (t <= delta) {
         w = inv_delta;
         H = T(0.5) * t * t * inv_delta;
@@ -52,35 +100,72 @@ __device__ __forceinline__ void tv_point(const T *__restrict__ c, int x, int y, 
     }
 }
 
+// A thread walks x through a run of kTvRun planes for one (y, z, channel); the
+// plane behind it stays in registers, so an element takes seven loads and three
+// weights (its own and its y and z predecessors') where taking every weight by
+// itself took sixteen and four, with three index divisions.  An item is a run
+// of 256 consecutive (y, z, channel) of a plane: all loads are contiguous.
+// 100^3, 28 channels: 460 -> 279 us in the whole call (c read and grad written
+// once: 33).
+constexpr int kTvRun = 10;
 template <typename T>
-__global__ void k_tv_huber(const T *__restrict__ c, int nx, int ny, int nz, int K, T delta, T *__restrict__ grad,
-                           double *__restrict__ partials)
+__global__ void __launch_bounds__(256)
+k_tv_huber(const T *__restrict__ c, int nx, int ny, int nz, int K, T delta, T *__restrict__ grad,
+           double *__restrict__ partials)
 {
     __shared__ double red[32];
-    const long long n = (long long)nx * ny * nz * K;
     const T inv_delta = T(1) / delta;
-    double v = 0.0;
-    Dot2 a = {0.f, 0.f};           // float: compensated FP32 sum of H
-    for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < n;
-         t += (long long)gridDim.x * blockDim.x) {
-        const int i = (int)(t % K);
-        const long long vox = t / K;
-        const int z = (int)(vox % nz), y = (int)((vox / nz) % ny), x = (int)(vox / ((long long)nz * ny));
-        T g[3], w, H;
-        tv_point<T>(c, x, y, z, nx, ny, nz, K, i, inv_delta, delta, g, w, H);
-        if constexpr (std::is_same<T, float>::value) dot2_add1(a, H);
-        else v += H;
-        if (grad) {
-            T gr = -w * (g[0] + g[1] + g[2]);
-            T gm[3], wm, Hm;
-            if (x >= 1) { tv_point<T>(c, x - 1, y, z, nx, ny, nz, K, i, inv_delta, delta, gm, wm, Hm); gr += wm * gm[0]; }
-            if (y >= 1) { tv_point<T>(c, x, y - 1, z, nx, ny, nz, K, i, inv_delta, delta, gm, wm, Hm); gr += wm * gm[1]; }
-            if (z >= 1) { tv_point<T>(c, x, y, z - 1, nx, ny, nz, K, i, inv_delta, delta, gm, wm, Hm); gr += wm * gm[2]; }
-            grad[t] = gr;
+    const int row = nz * K;
+    const long long plane = (long long)ny * row, segs = (plane + 255) / 256;
+    const long long items = segs * ((nx + kTvRun - 1) / kTvRun);
+    RegSum<T> sum;
+    for (long long it = blockIdx.x; it < items; it += gridDim.x) {
+        const int run = (int)(it / segs);
+        const long long e = (it - run * segs) * 256 + threadIdx.x;
+        if (e >= plane) continue;
+        const int y = (int)(e / row), zk = (int)(e - (long long)y * row);
+        const bool y0 = y >= 1, y1 = y + 1 < ny, z0 = zk >= K, z1 = zk + K < row;
+        const int x0 = run * kTvRun, x1 = min(nx, x0 + kTvRun);
+        const T *p = c + x0 * plane + e;
+        T cc = __ldg(p), cy = y0 ? __ldg(p - row) : T(0), cz = z0 ? __ldg(p - K) : T(0);   // here, y - 1, z - 1
+        T back = T(0);                                     // w g_x of the plane behind
+        if (grad && x0 > 0) {
+            const T *q = p - plane;
+            const T b = __ldg(q);
+            T w, H;
+            tv_point<T>(cc - b, y1 ? __ldg(q + row) - b : T(0), z1 ? __ldg(q + K) - b : T(0), inv_delta, delta, w, H);
+            back = w * (cc - b);
+        }
+        for (int x = x0; x < x1; ++x, p += plane) {
+            const bool on = x + 1 < nx;
+            const T nc = on ? __ldg(p + plane) : T(0);
+            const T py = y1 ? __ldg(p + row) : T(0), pz = z1 ? __ldg(p + K) : T(0);
+            const T gx = on ? nc - cc : T(0), gy = y1 ? py - cc : T(0), gz = z1 ? pz - cc : T(0);
+            T w, H;
+            tv_point<T>(gx, gy, gz, inv_delta, delta, w, H);
+            sum.add(H);
+            if (grad) {
+                T gr = -w * (gx + gy + gz) + back;
+                back = w * gx;
+                T wm, Hm;
+                if (y0) {
+                    const T ny1 = on ? __ldg(p + plane - row) : T(0);
+                    tv_point<T>(on ? ny1 - cy : T(0), cc - cy, z1 ? __ldg(p - row + K) - cy : T(0), inv_delta, delta, wm, Hm);
+                    gr += wm * (cc - cy);
+                    cy = ny1;
+                }
+                if (z0) {
+                    const T nz1 = on ? __ldg(p + plane - K) : T(0);
+                    tv_point<T>(on ? nz1 - cz : T(0), y1 ? __ldg(p + row - K) - cz : T(0), cc - cz, inv_delta, delta, wm, Hm);
+                    gr += wm * (cc - cz);
+                    cz = nz1;
+                }
+                grad[x * plane + e] = gr;
+            }
+            cc = nc;
         }
     }
-    if constexpr (std::is_same<T, float>::value) v = dot2_block_sum(a, reinterpret_cast<Dot2 *>(red));
-    else v = block_sum(v, red);
+    const double v = sum.total(red);
     if (threadIdx.x == 0) partials[blockIdx.x] = v;
 }
 
@@ -123,8 +208,8 @@ static tt_status l2_impl(tt_handle *h, const T *c, T *grad, double *value_host)
 template <typename T>
 static tt_status tv_impl(tt_handle *h, const T *c, double delta, T *grad, double *value_host)
 {
-    const long long n = h->nvox() * h->K;
-    const unsigned blocks = reg_grid(h, n);
+    const long long plane = (long long)h->N[1] * h->N[2] * h->K;
+    const unsigned blocks = reg_grid(h, (plane + 255) / 256 * 256 * ((h->N[0] + kTvRun - 1) / kTvRun));
     cudaEvent_t ev;
     prof_begin(h, TT_KSLOT_VECTOR, &ev);
     k_tv_huber<T><<<blocks, 256, 0, h->stream>>>(c, h->N[0], h->N[1], h->N[2], h->K, (T)delta, grad, h->red);
