@@ -59,22 +59,26 @@ namespace tt {
 // of those bytes, 8 a sixth.  What bounds it now is instruction issue (70% of
 // the slots at l_max 4; the same gather from global memory, with its bounds
 // tests and 64-bit addresses, took 0.358) and, at l_max 8, the latency that
-// eight resident warps leave: 0.259 and 6.8 ms.
+// eight resident warps leave: 0.263 and 6.1 ms.
 
-// One G' row of the box.
+// One G' row of the box.  Rows of two quads (R4 = 2) are 32 bytes apart, so
+// that lanes four rows apart read the same banks: lanes 4 .. 7 of every eight
+// read (and sum) their second quad first, and mode_store puts the quads back
+// (more than half of the wavefronts were conflicts; 128^3, l_max 8: 6.76 ->
+// 6.14 ms, 100^3, l_max 6: 2.54 -> 2.39).
 template <int R4, int R1>
 struct ModeRow {
     float v[4 * R4 + R1];
 };
 
 template <int R4, int R1>
-__device__ __forceinline__ void mode_load(ModeRow<R4, R1> &x, uint32_t a4, uint32_t a1)
+__device__ __forceinline__ void mode_load(ModeRow<R4, R1> &x, uint32_t a4, uint32_t a4b, uint32_t a1)
 {
 #pragma unroll
     for (int i = 0; i < R4; ++i)
         asm("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];"
             : "=f"(x.v[4 * i]), "=f"(x.v[4 * i + 1]), "=f"(x.v[4 * i + 2]), "=f"(x.v[4 * i + 3])
-            : "r"(a4 + 16 * i));
+            : "r"(i ? a4b : a4));
     if constexpr (R1) asm("ld.shared.f32 %0, [%1];" : "=f"(x.v[4 * R4]) : "r"(a1));
 }
 
@@ -95,15 +99,16 @@ constexpr int kRoundBits = 0x4b400000;
 
 // One column of candidate rays of a voxel (see k_adjoint for the enumeration):
 // outer offset d = o - oc; du, dv the offsets of the column's first ray's taps
-// from the voxel, a4 and a1 the addresses of its row.  A column that the clamp
+// from the voxel, a4 (with a4b, the quad read second) and a1 the addresses of
+// its row.  A column that the clamp
 // moves holds no ray of positive weight (such rays lie in the box).
 struct ModeColumn {
     float du, dv;
-    uint32_t a4, a1;
+    uint32_t a4, a4b, a1;
 };
 template <int R4>
 __device__ __forceinline__ ModeColumn mode_column(const float4 &cu, const float4 &ce, const int4 &ci, float d, float ic,
-                                                  int orow, uint32_t b4, uint32_t b1)
+                                                  int orow, uint32_t b4, uint32_t b4b, uint32_t b1)
 {
     const float xr = (ic + fmaxf(fmaf(ce.z, d, ce.x), fmaf(ce.w, d, ce.y))) + kRound;
     const float di = (xr - kRound) - ic;
@@ -113,6 +118,8 @@ __device__ __forceinline__ ModeColumn mode_column(const float4 &cu, const float4
     const uint32_t idx = min((uint32_t)(__float_as_int(xr) * ci.y + orow), (uint32_t)ci.w);
     // (opaque, so that the candidates' addresses are these plus uniform steps)
     asm("mad.lo.u32 %0, %1, %2, %3;" : "=r"(r.a4) : "r"(idx), "n"(16 * R4), "r"(b4));
+    if constexpr (R4 == 2) asm("mad.lo.u32 %0, %1, %2, %3;" : "=r"(r.a4b) : "r"(idx), "n"(16 * R4), "r"(b4b));
+    else r.a4b = 0;
     asm("mad.lo.u32 %0, %1, 4, %2;" : "=r"(r.a1) : "r"(idx), "r"(b1));
     return r;
 }
@@ -125,14 +132,14 @@ __device__ __forceinline__ float mode_weight(const float4 &cu, const ModeColumn 
 
 template <int R4, int R1, int NO, int NI>
 __device__ __forceinline__ void mode_gather(ModeRow<R4, R1> &t, const float4 &cu, const float4 &ce, const int4 &ci,
-                                            float d0, float ic, int orow0, uint32_t b4, uint32_t b1)
+                                            float d0, float ic, int orow0, uint32_t b4, uint32_t b4b, uint32_t b1)
 {
 #pragma unroll
     for (int a = 0; a < NO; ++a) {
-        const ModeColumn k = mode_column<R4>(cu, ce, ci, d0 + (float)a, ic, orow0 + a * ci.x, b4, b1);
+        const ModeColumn k = mode_column<R4>(cu, ce, ci, d0 + (float)a, ic, orow0 + a * ci.x, b4, b4b, b1);
         ModeRow<R4, R1> x[NI];
 #pragma unroll
-        for (int b = 0; b < NI; ++b) mode_load<R4, R1>(x[b], k.a4 + b * ci.y * (16 * R4), k.a1 + b * ci.y * 4);
+        for (int b = 0; b < NI; ++b) mode_load<R4, R1>(x[b], k.a4 + b * ci.y * (16 * R4), k.a4b + b * ci.y * (16 * R4), k.a1 + b * ci.y * 4);
 #pragma unroll
         for (int b = 0; b < NI; ++b) mode_fma<R4, R1, false>(t, mode_weight(cu, k, b), x[b]);
     }
@@ -141,14 +148,14 @@ __device__ __forceinline__ void mode_gather(ModeRow<R4, R1> &t, const float4 &cu
 // Windows of any size (unequal voxel and pixel sizes), and guarded.
 template <int R4, int R1, bool GUARD>
 __device__ __forceinline__ void mode_gather_any(ModeRow<R4, R1> &t, const float4 &cu, const float4 &ce, const int4 &ci,
-                                                float d0, float ic, int orow0, uint32_t b4, uint32_t b1, int order)
+                                                float d0, float ic, int orow0, uint32_t b4, uint32_t b4b, uint32_t b1, int order)
 {
     const int NO = order & 0xff, NI = (order >> 8) & 0xff;
     for (int a = 0; a < NO; ++a) {
-        const ModeColumn k = mode_column<R4>(cu, ce, ci, d0 + (float)a, ic, orow0 + a * ci.x, b4, b1);
+        const ModeColumn k = mode_column<R4>(cu, ce, ci, d0 + (float)a, ic, orow0 + a * ci.x, b4, b4b, b1);
         for (int b = 0; b < NI; ++b) {
             ModeRow<R4, R1> x;
-            mode_load<R4, R1>(x, k.a4 + b * ci.y * (16 * R4), k.a1 + b * ci.y * 4);
+            mode_load<R4, R1>(x, k.a4 + b * ci.y * (16 * R4), k.a4b + b * ci.y * (16 * R4), k.a1 + b * ci.y * 4);
             mode_fma<R4, R1, GUARD>(t, mode_weight(cu, k, b), x);
         }
     }
@@ -166,10 +173,19 @@ __device__ __forceinline__ void tf32_split(float v, uint32_t &hi, uint32_t &lo)
 // A projection's operand columns of one voxel: R split modes, hi then lo, in
 // consecutive columns.
 template <int R4, int R1>
-__device__ __forceinline__ void mode_store(uint32_t ta, const ModeRow<R4, R1> &t)
+__device__ __forceinline__ void mode_store(uint32_t ta, ModeRow<R4, R1> t)
 {
     constexpr int M = 4 * R4 + R1;
     uint32_t v[2 * M];
+    if constexpr (R4 == 2) {
+        const bool swapped = threadIdx.x & 4;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const float a = t.v[i], b = t.v[4 + i];
+            t.v[i] = swapped ? b : a;
+            t.v[4 + i] = swapped ? a : b;
+        }
+    }
 #pragma unroll
     for (int i = 0; i < M; ++i) tf32_split(t.v[i], v[i], v[M + i]);
     if constexpr (2 * M >= 16) {
@@ -351,6 +367,7 @@ k_adjoint_modes(const __grid_constant__ ModeParams P, const __grid_constant__ Tm
         }
         bool ok = true;                                            // false once a wait gave up: the rest is NaN
         const bool guard = *nonfinite == rows_id;                  // some row is not finite
+        const uint32_t quad0 = R4 == 2 ? (lane & 4) * 4 : 0;       // offset of the quad read first
         uint32_t stage_phase = 0, empty_phase = 1, box = ring;
         uint64_t *bar = stage;
         int drain = 0, si = u_begin * UP;
@@ -369,7 +386,7 @@ k_adjoint_modes(const __grid_constant__ ModeParams P, const __grid_constant__ Tm
                     const float4 cu = *reinterpret_cast<const float4 *>(&c.uo), ce = *reinterpret_cast<const float4 *>(&c.au);
                     const int4 ci = *reinterpret_cast<const int4 *>(&c.so);
                     const float2 hd = *reinterpret_cast<const float2 *>(&hdr[si & 63]);
-                    const uint32_t b4 = box, b1 = box + box4a;
+                    const uint32_t b4 = box + quad0, b4b = box + (quad0 ^ 16), b1 = box + box4a;
                     float oc[V], ic[V], d0[V];
                     int orow[V];
                     oc[0] = fmaf(co.z, lz, fmaf(co.y, ly, fmaf(co.x, lx, hd.x)));
@@ -385,7 +402,7 @@ k_adjoint_modes(const __grid_constant__ ModeParams P, const __grid_constant__ Tm
 #define TT_MODE_CASE(NO_, NI_)                                                                              \
     case 16 * NO_ + NI_:                                                                                    \
         _Pragma("unroll") for (int v = 0; v < V; ++v)                                                       \
-            mode_gather<R4, R1, NO_, NI_>(t[v], cu, ce, ci, d0[v], ic[v], orow[v], b4, b1);                 \
+            mode_gather<R4, R1, NO_, NI_>(t[v], cu, ce, ci, d0[v], ic[v], orow[v], b4, b4b, b1);                 \
         break;
                     switch (guard ? -1 : c.shape) {
                     TT_MODE_CASE(1, 1) TT_MODE_CASE(1, 2) TT_MODE_CASE(1, 3)
@@ -394,12 +411,12 @@ k_adjoint_modes(const __grid_constant__ ModeParams P, const __grid_constant__ Tm
                     case 0:
 #pragma unroll
                         for (int v = 0; v < V; ++v)
-                            mode_gather_any<R4, R1, false>(t[v], cu, ce, ci, d0[v], ic[v], orow[v], b4, b1, c.order);
+                            mode_gather_any<R4, R1, false>(t[v], cu, ce, ci, d0[v], ic[v], orow[v], b4, b4b, b1, c.order);
                         break;
                     default:
 #pragma unroll
                         for (int v = 0; v < V; ++v)
-                            mode_gather_any<R4, R1, true>(t[v], cu, ce, ci, d0[v], ic[v], orow[v], b4, b1, c.order);
+                            mode_gather_any<R4, R1, true>(t[v], cu, ce, ci, d0[v], ic[v], orow[v], b4, b4b, b1, c.order);
                         break;
                     }
 #undef TT_MODE_CASE
