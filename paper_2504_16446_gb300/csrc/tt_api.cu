@@ -810,13 +810,10 @@ tt_status tt_create(const tt_problem *P, tt_precision prec, void *stream, tt_han
         if (h->slot_floats) {
             ALLOC(h->FM, sizeof(float) * 2 * h->S * modes_m(h->R) * h->KP);
             ALLOC(h->order, sizeof(int) * h->S);
-            ALLOC(h->slots, sizeof(float) * (h->chunk * h->slot_floats + h->slots1));
         }
-        h->fwd_modes = h->slots != nullptr;
     }
     plan_forward(h);
     h->fwd_staged = false;   // the tap-pair march is the faster one on every measured workload
-    h->n_fwd_ctas = h->fwd_modes ? mode_forward_ctas(h) : forward_ctas(h, h->fwd_staged);
     h->n_partials = std::max(std::max(forward_ctas(h, false), forward_ctas(h, true)), mode_forward_ctas(h));
     ALLOC(h->partials, sizeof(double) * h->n_partials);
     ALLOC(h->loss_dev, sizeof(double) * 4);
@@ -845,6 +842,14 @@ tt_status tt_create(const tt_problem *P, tt_precision prec, void *stream, tt_han
     double *dstage = nullptr;
     ALLOC(dstage, sizeof(double) * stage.size());
 #undef ALLOC
+    // last, and optional: a handle whose slots find no memory marches the volume
+    if (h->slot_floats &&
+        cudaMalloc((void **)&h->slots, sizeof(float) * (h->chunk * h->slot_floats + h->slots1)) != cudaSuccess) {
+        (void)cudaGetLastError();
+        h->slots = nullptr;
+    }
+    h->fwd_modes = h->slots != nullptr;
+    h->n_fwd_ctas = h->fwd_modes ? mode_forward_ctas(h) : forward_ctas(h, h->fwd_staged);
     cudaError_t e = cudaMemcpyAsync(dstage, stage.data(), sizeof(double) * stage.size(), cudaMemcpyHostToDevice, h->stream);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(h->geo, h->geo_host.data(), sizeof(ProjGeom) * h->S, cudaMemcpyHostToDevice, h->stream);
@@ -979,8 +984,10 @@ tt_status tt_gradient_residual_host(tt_handle *h, const float *c_host, const flo
     // stream, then I and W in Q projection chunks on a copy stream.  The
     // forward launch of chunk q waits only for chunk q and runs on one of two
     // side streams, so that a chunk's last wave overlaps the next chunk's
-    // first; the adjoint joins both.  (Reading mapped inputs in place over
-    // the host link measured slower than these copies.)
+    // first (on one of them where the forward maps the volume to modes: its
+    // chunks share the mapped volumes' slots); the adjoint joins both.
+    // (Reading mapped inputs in place over the host link measured slower than
+    // these copies.)
     // A page-locked, device-mapped g_host is written by the adjoint in place,
     // its stores crossing the host link while the kernel runs; any other
     // g_host gets the gradient with one copy.

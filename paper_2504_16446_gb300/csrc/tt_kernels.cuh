@@ -4,7 +4,9 @@
 // Data layout in HBM (all row-major):
 //   cpad [nx][ny][nz][KP]          coefficient volume, channel innermost, zero padded
 //   Bp   [S][CP][KP]               basis matrix in the element type, zero padded
-//   G    [S][nj][nk][KP]           back-contracted weighted residual, 2 B_s^T (W r)
+//   G    [S][nj][nk][KP]           back-contracted weighted residual, 2 B_s^T (W r); in a
+//                                  handle that works in detector modes (tt_modes.cuh) the
+//                                  rows 2 Q^T (W r) of R values instead
 //   gpad [nx][ny][nz][KP]          gradient / adjoint volume
 // A lane group of LG consecutive lanes owns one ray (forward) or one voxel
 // (adjoint); lane q of the group holds channels [q*CPL, (q+1)*CPL), so that a

@@ -228,7 +228,8 @@ class Handle:
 
     def set_forward_kernel(self, kind: str) -> None:
         """Forward-projection kernel for the calls that follow: "auto", "l1" (taps read
-        from the L1/L2-resident volume) or "staged" (taps staged in shared memory)."""
+        from the L1/L2-resident volume) or "staged" (taps staged in shared memory);
+        see tt_set_forward_kernel in include/tt.h."""
         _check(self.lib.tt_set_forward_kernel(self._h, self.FORWARD_KERNELS[kind]), "tt_set_forward_kernel")
 
     @property
