@@ -185,7 +185,7 @@ def _kernel_source_hash():
     import re
     h = hashlib.sha256()
     csrc = os.path.join(ROOT, "paper_2504_16446_gb300", "csrc")
-    for f in ("tt_internal.cuh", "tt_kernels.cuh", "tt_proj_f32.cu"):
+    for f in ("tt_internal.cuh", "tt_kernels.cuh", "tt_modes.cuh", "tt_proj_f32.cu"):
         with open(os.path.join(csrc, f)) as fh:
             code = re.sub(r"/\*.*?\*/", "", fh.read(), flags=re.S)
         code = re.sub(r"//[^\n]*", "", code)
@@ -500,9 +500,10 @@ def measure_forms(torch, tt, synth, flush, steps: int = 20):
                 ev1.synchronize()
                 tot += ev0.elapsed_time(ev1)
             p = h.profile_read()
-            row[prec] = {"ms_per_eval": tot / steps,
-                         "forward_ms": p["forward"][0] / max(1, p["forward"][1]),
-                         "adjoint_ms": p["adjoint"][0] / max(1, p["adjoint"][1])}
+            # per evaluation: packing (and, at l_max 6 and 8, the maps to detector
+            # modes), the marches, the adjoint
+            row[prec] = {"ms_per_eval": tot / steps, "pack_ms": p["pack"][0] / steps,
+                         "forward_ms": p["forward"][0] / steps, "adjoint_ms": p["adjoint"][0] / steps}
             h.close()
         row["workload"] = f"{st.shape[0]}^3, l_max {st.ell_max}, {st.S} x {st.nj}x{st.nk} x {st.C}"
         res[wl] = row
@@ -843,13 +844,14 @@ def run_ours(args):
                      "step_frac": 2 * sweep_bytes / (ms_per_step * 1e-3) / 1e9 / peak},
         # t_roof = max(compulsory HBM bytes / HBM peak, FP32 flops / FP32 peak) against the step time
         "binding_roof": binding_roof(st, ms_per_step, peak, fp32_peak),
-        # the path the projector kernels saturate: bilinear taps delivered from
-        # L1 / shared memory to registers, 4 taps x K channels x 4 B per
-        # (ray, plane) in either direction, against 128 B per clock per SM
+        # the path the forward march saturates: bilinear taps delivered from
+        # L1 to registers, 4 taps x K channels x 4 B per (ray, plane), against
+        # 128 B per clock per SM (the adjoint gathers detector modes, a third
+        # of those bytes, and is bound by instruction issue)
         "l1_roof": {k: {"achieved_gbs": tap_bytes / (prof[k][0] / prof[k][1] * 1e-3) / 1e9, "peak_gbs": l1_peak,
                         "frac": tap_bytes / (prof[k][0] / prof[k][1] * 1e-3) / 1e9 / l1_peak,
                         "bytes_per_launch": tap_bytes}
-                    for k in ("forward", "adjoint") if prof[k][1]},
+                    for k in ("forward",) if prof[k][1]},
         "fp32_alu": {"kernel": dom, "achieved_tflops": flops / (dom_ms * 1e-3) / 1e12,
                      "peak_tflops": fp32_peak, "frac": flops / (dom_ms * 1e-3) / 1e12 / fp32_peak,
                      "peak_formula": "sm_count x 128 lanes x 2 flops x median SM clock"},
