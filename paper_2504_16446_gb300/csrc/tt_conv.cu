@@ -105,13 +105,21 @@ struct TcConvSmem {
     static constexpr uint32_t tmem_cols = 2 * 3 * COUT <= 128 ? 128 : 256;   // two accumulators of 3 COUT
 };
 
+// What a convolution writes: bfloat16 or float rows of COUT channels, or (the
+// network's last layer) float rows of the k_real <= COUT real channels, scaled.
+enum { kOutBf16, kOutF32, kOutRows };
+
 // Tile epilogue: warp w reads tensor-memory lanes 32 (w % 4) .. (input rows
 // y0 + w % 4, z0 - 1 + lane) and, for its half of the output channels, the
 // three z-tap blocks of accumulator `acc_col`; lanes 1..30 combine rows
-// lane-1, lane, lane+1 and write output z0 - 1 + lane.
-template <int COUT, bool RELU, bool OUT_F32>
+// lane-1, lane, lane+1 and write output z0 - 1 + lane.  kOutRows: warps w and
+// w + 4 hold the channels of one row of voxels, which is contiguous in the
+// output; they gather it in `rows` and share the stores.  (The caller's next
+// __syncthreads lets `rows` be written again.)
+template <int COUT, bool RELU, int OUT>
 __device__ __forceinline__ void tile_epilogue(uint32_t tmem, uint32_t acc_col, bool ok, void *__restrict__ out, int x0,
-                                              int y0, int z0, int ny, int nz, int warp, int lane)
+                                              int y0, int z0, int ny, int nz, int warp, int lane, int k_real,
+                                              float scale, float *__restrict__ rows)
 {
     constexpr int CW = COUT / (kTcThreads / 128);
     static_assert(CW == 8 || CW == 16, "a warp reads 8 or 16 accumulator columns per z tap");
@@ -132,9 +140,24 @@ __device__ __forceinline__ void tile_epilogue(uint32_t tmem, uint32_t acc_col, b
         v[c] = ok ? (below + p[1][c]) + above : __int_as_float(0x7fc00000);
     }
     const int gy = y0 + quad, gz = z0 - 1 + lane;
+    if constexpr (OUT == kOutRows) {
+        const int nzr = gy < ny ? min(kTileZ, nz - z0) : 0;
+        float *r = rows + quad * (kTileZ * COUT);
+        if (lane >= 1 && lane <= nzr)
+#pragma unroll
+            for (int c = 0; c < CW; ++c)
+                if (c_base + c < k_real) r[(lane - 1) * k_real + c_base + c] = scale * v[c];
+        asm volatile("bar.sync %0, 64;" ::"r"(1 + quad) : "memory");
+        float *o = static_cast<float *>(out) + (((size_t)x0 * ny + gy) * nz + z0) * k_real;
+        const int e0 = (warp >> 2) * 32 + lane;
+#pragma unroll
+        for (int k = 0; k < (kTileZ * COUT + 63) / 64; ++k)
+            if (e0 + 64 * k < nzr * k_real) o[e0 + 64 * k] = r[e0 + 64 * k];
+        return;
+    }
     if (lane < 1 || lane > kTileZ || gy >= ny || gz >= nz) return;
     const size_t vox = ((size_t)x0 * ny + gy) * nz + gz;
-    if constexpr (OUT_F32) {
+    if constexpr (OUT == kOutF32) {
         float4 *o = reinterpret_cast<float4 *>(static_cast<float *>(out) + vox * COUT + c_base);
 #pragma unroll
         for (int i = 0; i < CW / 4; ++i) {
@@ -162,11 +185,12 @@ __device__ __forceinline__ void tile_epilogue(uint32_t tmem, uint32_t acc_col, b
 // Two CTAs per SM are all that shared and tensor memory admit; said so, the
 // compiler keeps the epilogue's columns in registers (80) where it spilled some
 // at 40 (128^3: 32 -> 32 channels 150 -> 139 us, 16 -> 32 97 -> 89).
-template <int CIN, int COUT, bool RELU, bool OUT_F32>
+template <int CIN, int COUT, bool RELU, int OUT>
 __global__ void __launch_bounds__(kTcThreads, 2)
 k_conv3d_fwd_tc(const __grid_constant__ CUtensorMap planes, const __nv_bfloat16 *__restrict__ wk,
-                void *__restrict__ out, int nx, int ny, int nz, int tiles_y, int tiles_z)
+                void *__restrict__ out, int nx, int ny, int nz, int tiles_y, int tiles_z, int k_real, float scale)
 {
+    __shared__ float rows[OUT == kOutRows ? 4 * kTileZ * COUT : 1];
     using L = TcConvSmem<CIN, COUT>;
     constexpr int KC = CIN / 8, NB = 3 * COUT;
     constexpr uint32_t kLboA = 6 * 512, kLboB = NB * 16;
@@ -258,8 +282,8 @@ k_conv3d_fwd_tc(const __grid_constant__ CUtensorMap planes, const __nv_bfloat16 
                 // buffer takes plane x-2+NBUF now, before the tile is written out
                 if (tid == 0 && x - 2 + NBUF <= xb) copy_plane(x - 2 + NBUF);
                 umma::fence_after_sync();
-                tile_epilogue<COUT, RELU, OUT_F32>(tmem, (uint32_t)(NB * p), ok, out, x - 1, y0, z0, ny, nz, warp,
-                                                   lane);
+                tile_epilogue<COUT, RELU, OUT>(tmem, (uint32_t)(NB * p), ok, out, x - 1, y0, z0, ny, nz, warp, lane,
+                                               k_real, scale, rows);
             }
         }
         umma::fence_before_sync();
@@ -409,34 +433,6 @@ __global__ void k_pack_bf16(const float *__restrict__ x, int k_real, long long n
     }
 }
 
-// y [nvox][16] float -> out [nvox][k_real], scaled: 256 voxels at a time, read
-// as quads and written contiguously through shared memory (bound by the two
-// volumes' bytes; an index division per element took 74 us at 128^3, 15
-// channels, this 39).
-__global__ void __launch_bounds__(256)
-k_unpack_f32(const float *__restrict__ y, int k_real, long long nvox, float scale, float *__restrict__ out)
-{
-    __shared__ float rows[256 * 16];
-    const float4 *y4 = reinterpret_cast<const float4 *>(y);
-    for (long long v0 = (long long)blockIdx.x * 256; v0 < nvox; v0 += (long long)gridDim.x * 256) {
-        const int nv = (int)(nvox - v0 < 256 ? nvox - v0 : 256);
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const int i = q * 256 + threadIdx.x, c = 4 * (i & 3);
-            if ((i >> 2) < nv) {
-                const float4 f = __ldg(y4 + v0 * 4 + i);
-                const float w[4] = {f.x, f.y, f.z, f.w};
-#pragma unroll
-                for (int k = 0; k < 4; ++k)
-                    if (c + k < k_real) rows[(i >> 2) * k_real + c + k] = scale * w[k];
-            }
-        }
-        __syncthreads();
-        for (int i = threadIdx.x; i < nv * k_real; i += 256) out[v0 * k_real + i] = rows[i];
-        __syncthreads();
-    }
-}
-
 // Master weights w [27][R][Cc] (float, padded) -> wk bfloat16, either the same
 // layout (flip = 0) or that of the transposed convolution (flip = 1):
 // wk[t][c][r] = w[26 - t][r][c].
@@ -483,9 +479,12 @@ static unsigned grid_n(long long n)
 // contiguous share of the nx * tiles_y * tiles_z tiles (x fastest) as runs
 // of consecutive x planes (measured at 128^3, 32 -> 32 channels: runs of 16
 // planes dealt round robin left a 19% tail; equal shares cut it and the
-// pipeline fills to about 1.5 runs per CTA).
+// pipeline fills to about 1.5 runs per CTA).  k_real > 0 (32 -> 16 channels,
+// float, no ReLU): `out` takes rows of that many channels, scaled.  At 128^3,
+// 15 channels, that layer and a kernel that took its padded rows to `out` were
+// 108 + 39 us; this layer alone 113.
 cudaError_t conv3d_forward(const __nv_bfloat16 *in, const __nv_bfloat16 *wk, void *out, int nx, int ny, int nz, int cin,
-                           int cout, bool relu, bool out_f32, cudaStream_t st)
+                           int cout, bool relu, bool out_f32, cudaStream_t st, int k_real = 0, float scale = 1.f)
 {
     const int tiles_y = (ny + 3) / 4, tiles_z = (nz + kTileZ - 1) / kTileZ;
     if (nx < 1 || ny < 1 || nz < 1) return cudaSuccess;
@@ -514,18 +513,22 @@ cudaError_t conv3d_forward(const __nv_bfloat16 *in, const __nv_bfloat16 *wk, voi
         const long long slots = (long long)sm_count() * (sm <= 110u * 1024u ? 2 : 1);                  \
         const long long n_tiles = (long long)nx * tiles_y * tiles_z;                                   \
         const int grid = (int)(n_tiles < slots ? n_tiles : slots);                                     \
-        kern<<<grid, kTcThreads, sm, st>>>(planes, wk, out, nx, ny, nz, tiles_y, tiles_z);            \
+        kern<<<grid, kTcThreads, sm, st>>>(planes, wk, out, nx, ny, nz, tiles_y, tiles_z, k_real, scale); \
         return cudaGetLastError();                                                                    \
     } while (0)
-    if (cin == 16 && cout == 32 && relu && !out_f32) TT_CONV_LAUNCH(16, 32, true, false);
-    if (cin == 32 && cout == 32 && relu && !out_f32) TT_CONV_LAUNCH(32, 32, true, false);
-    if (cin == 32 && cout == 16 && !relu && out_f32) TT_CONV_LAUNCH(32, 16, false, true);
-    if (cin == 32 && cout == 32 && !relu && !out_f32) TT_CONV_LAUNCH(32, 32, false, false);
-    if (cin == 16 && cout == 32 && !relu && !out_f32) TT_CONV_LAUNCH(16, 32, false, false);
-    if (cin == 32 && cout == 16 && !relu && !out_f32) TT_CONV_LAUNCH(32, 16, false, false);
-    if (cin == 16 && cout == 16 && !relu && out_f32) TT_CONV_LAUNCH(16, 16, false, true);
-    if (cin == 16 && cout == 32 && !relu && out_f32) TT_CONV_LAUNCH(16, 32, false, true);
-    if (cin == 32 && cout == 32 && !relu && out_f32) TT_CONV_LAUNCH(32, 32, false, true);
+    if (k_real > 0) {
+        if (cin == 32 && cout == 16 && !relu && out_f32) TT_CONV_LAUNCH(32, 16, false, kOutRows);
+        return cudaErrorInvalidValue;
+    }
+    if (cin == 16 && cout == 32 && relu && !out_f32) TT_CONV_LAUNCH(16, 32, true, kOutBf16);
+    if (cin == 32 && cout == 32 && relu && !out_f32) TT_CONV_LAUNCH(32, 32, true, kOutBf16);
+    if (cin == 32 && cout == 16 && !relu && out_f32) TT_CONV_LAUNCH(32, 16, false, kOutF32);
+    if (cin == 32 && cout == 32 && !relu && !out_f32) TT_CONV_LAUNCH(32, 32, false, kOutBf16);
+    if (cin == 16 && cout == 32 && !relu && !out_f32) TT_CONV_LAUNCH(16, 32, false, kOutBf16);
+    if (cin == 32 && cout == 16 && !relu && !out_f32) TT_CONV_LAUNCH(32, 16, false, kOutBf16);
+    if (cin == 16 && cout == 16 && !relu && out_f32) TT_CONV_LAUNCH(16, 16, false, kOutF32);
+    if (cin == 16 && cout == 32 && !relu && out_f32) TT_CONV_LAUNCH(16, 32, false, kOutF32);
+    if (cin == 32 && cout == 32 && !relu && out_f32) TT_CONV_LAUNCH(32, 32, false, kOutF32);
 #undef TT_CONV_LAUNCH
     return cudaErrorInvalidValue;
 }
@@ -633,8 +636,10 @@ static tt_status cast_weights(tt_wsnet *n)
     return TT_OK;
 }
 
-// net(x * in_scale) into n->out [nvox][16] (float).
-static tt_status net_forward(tt_wsnet *n, int nx, int ny, int nz, const float *x, double in_scale)
+// net(x * in_scale) into n->out [nvox][16] (float), or, times out_scale, into
+// y [nvox][kout].
+static tt_status net_forward(tt_wsnet *n, int nx, int ny, int nz, const float *x, double in_scale,
+                             float *y = nullptr, double out_scale = 1.0)
 {
     const long long nvox = (long long)nx * ny * nz;
     tt_status st = ensure_buffers(n, nvox);
@@ -643,8 +648,9 @@ static tt_status net_forward(tt_wsnet *n, int nx, int ny, int nz, const float *x
     TT_NET_CUDA(cudaGetLastError(), "wsnet pack");
     for (int l = 0; l < kNetLayers; ++l) {
         const bool last = l == kNetLayers - 1;
-        TT_NET_CUDA(conv3d_forward(n->a[l], n->wk[l], last ? (void *)n->out : (void *)n->a[l + 1], nx, ny, nz,
-                                   layer_cin(l), layer_cout(l), !last, last, n->stream),
+        TT_NET_CUDA(conv3d_forward(n->a[l], n->wk[l], last ? (void *)(y ? y : n->out) : (void *)n->a[l + 1], nx, ny, nz,
+                                   layer_cin(l), layer_cout(l), !last, last, n->stream, last && y ? n->kout : 0,
+                                   (float)out_scale),
                     "wsnet conv forward");
     }
     return TT_OK;
@@ -767,12 +773,7 @@ tt_status tt_wsnet_forward(tt_wsnet *n, int nx, int ny, int nz, const float *x, 
         set_error("tt_wsnet_forward: bad arguments");
         return TT_INVALID_ARG;
     }
-    tt_status st = net_forward(n, nx, ny, nz, x, 1.0 / in_scale);
-    if (st != TT_OK) return st;
-    const long long nvox = (long long)nx * ny * nz;
-    k_unpack_f32<<<grid_n(nvox), 256, 0, n->stream>>>(n->out, n->kout, nvox, (float)out_scale, y);
-    TT_NET_CUDA(cudaGetLastError(), "wsnet unpack");
-    return TT_OK;
+    return net_forward(n, nx, ny, nz, x, 1.0 / in_scale, y, out_scale);
 }
 
 tt_status tt_wsnet_gradient(tt_wsnet *n, int nx, int ny, int nz, const float *x, const float *target,
