@@ -84,6 +84,13 @@ void plan_modes(tt_handle *h)
     h->nk1 = (h->nk + 3) / 4 * 4;
     h->box_j = bj;
     h->box_k = bk;
+    // Rows of one quad: a pitch of 4 mod 8 pixels puts neighbouring rows of the
+    // box half the banks apart (where the wider box fits).
+    if (h->R4 == 1 && bk % 8 == 0) {
+        h->box_k = bk + 4;
+        if ((bk + 4) * 4 <= 256 && (long long)modes_smem(h) <= kModeMaxSmem) bk += 4;
+        h->box_k = bk;
+    }
     TmaDesc probe;
     if (bk * 4 * h->R4 > 256 || bj > 256 || (long long)modes_smem(h) > kModeMaxSmem ||
         !encode_rows(h, (const void *)4096, 4 * h->R4, h->nk, &probe) ||
