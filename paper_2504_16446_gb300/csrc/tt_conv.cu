@@ -64,9 +64,9 @@ __device__ __forceinline__ void mma_bf16(float (&d)[4], const unsigned (&a)[4], 
 //   y(z) = P_0(z - 1) + P_1(z) + P_2(z + 1).
 // That is 9 * CIN / 16 MMAs of M 128, N 3 COUT, K 16 per tile, a third of
 // the count with the z taps as separate MMAs of N COUT; the MMA chain, not
-// the N width, sets the time at these sizes.  Plane buffers are [CIN/8][y 6]
-// [z 32] 16-byte (8-channel) chunks, zeros outside the volume: SBO = 128 B
-// (next 8 rows), LBO = 6 * 512 B (next 8 channels).  Weights are staged once
+// the N width, sets the time at these sizes.  Plane buffers are [y 6][z 32]
+// rows of CIN channels, swizzled over their 64 (32) bytes, zeros outside the
+// volume: SBO = 8 rows; 16 channels further is 32 bytes on.  Weights are staged once
 // per CTA as [dx,dy][CIN/8][dz * COUT + co][8] (SBO = 128 B, LBO = 3 COUT
 // 16 B).
 //
@@ -74,10 +74,11 @@ __device__ __forceinline__ void mma_bf16(float (&d)[4], const unsigned (&a)[4], 
 // tile column.  Tile x needs planes x-1, x, x+1 from a ring of NBUF plane
 // buffers (4 for 32 -> 32 channels, more where the weights are smaller), so
 // each step stages one new plane, NBUF - 3 steps ahead.  A plane is one tiled tensor
-// copy: the input viewed as a 5-D tensor (8 channels, z, y, channel group,
-// x) whose box of 8 x 32 x 6 x CIN/8 x 1 elements lands in exactly the
-// buffer layout above, zeros outside the volume; it completes on the
-// buffer's own mbarrier.  Step for tile x: thread 0 waits for plane x+1's
+// copy, a box of CIN x 32 x 6 x 1 elements of [x][y][z][CIN], zeros outside
+// the volume; it completes on the buffer's own mbarrier.  (Boxes of 16-byte
+// channel groups, which need no swizzle, were slower: 113 against 110 us for
+// 32 -> 16 channels at 128^3, 88 against 86 for 16 -> 32; 32 -> 32, held by its
+// chain of MMAs, takes 140 either way.)  Step for tile x: thread 0 waits for plane x+1's
 // copy, issues the tile's MMAs into tensor-memory accumulator x % 2 and
 // commits them to mbarrier x % 2; meanwhile all eight warps wait for tile
 // x-1's mbarrier, thread 0 starts the copy of plane x-2+NBUF into the buffer
@@ -101,7 +102,7 @@ struct TcConvSmem {
     // [0, 1] MMA commits, [2, 2 + nbuf) plane copies, then the tensor-memory
     // slot and a failure flag
     static constexpr uint32_t mbar = wts + 9 * dxy;
-    static constexpr uint32_t bytes = mbar + 8 * (2 + nbuf) + 8;
+    static constexpr uint32_t bytes = mbar + 8 * (2 + nbuf) + 8 + 1024;   // (the buffers start on 1024 bytes)
     static constexpr uint32_t tmem_cols = 2 * 3 * COUT <= 128 ? 128 : 256;   // two accumulators of 3 COUT
 };
 
@@ -193,8 +194,9 @@ k_conv3d_fwd_tc(const __grid_constant__ CUtensorMap planes, const __nv_bfloat16 
     __shared__ float rows[OUT == kOutRows ? 4 * kTileZ * COUT : 1];
     using L = TcConvSmem<CIN, COUT>;
     constexpr int KC = CIN / 8, NB = 3 * COUT;
-    constexpr uint32_t kLboA = 6 * 512, kLboB = NB * 16;
-    extern __shared__ __align__(1024) uint8_t smem[];
+    constexpr uint32_t kRowA = CIN * 2, kSwizzleA = CIN == 32 ? 4 : 6, kLboB = NB * 16;
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t *smem = smem_raw + ((0u - umma::smem_u32(smem_raw)) & 1023u);
     uint64_t *mbar = reinterpret_cast<uint64_t *>(smem + L::mbar);   // [0, 1] MMA commits
     constexpr int NBUF = L::nbuf;
     uint64_t *pbar = mbar + 2;                                        // [NBUF] plane copies, one per buffer
@@ -242,7 +244,7 @@ k_conv3d_fwd_tc(const __grid_constant__ CUtensorMap planes, const __nv_bfloat16 
         auto copy_plane = [&](int px) {
             const int bf = (px + NBUF) % NBUF;
             umma::mbar_arrive_expect_tx(pbar + bf, L::plane);
-            umma::tma_load_5d(smem + bf * L::plane, pmap, 0, z0 - 1, y0 - 1, 0, px, pbar + bf);
+            umma::tma_load_4d(smem + bf * L::plane, pmap, 0, z0 - 1, y0 - 1, px, pbar + bf);
             copy_par ^= 1u << bf;
             used |= 1u << bf;
         };
@@ -265,11 +267,11 @@ k_conv3d_fwd_tc(const __grid_constant__ CUtensorMap planes, const __nv_bfloat16 
                 const uint32_t acc = tmem + (uint32_t)(NB * (i & 1));
                 for (int dxy = 0; dxy < 9; ++dxy) {
                     const int dx = dxy / 3, dy = dxy % 3;                  // offset + 1
-                    const uint32_t a0 = s_planes + ((x - 1 + dx + NBUF) % NBUF) * L::plane + dy * 512;
+                    const uint32_t a0 = s_planes + ((x - 1 + dx + NBUF) % NBUF) * L::plane + dy * 32 * kRowA;
                     const uint32_t b0 = s_wts + dxy * L::dxy;
 #pragma unroll
                     for (int kk = 0; kk < CIN / 16; ++kk)
-                        umma::mma_bf16(acc, umma::smem_desc(a0 + kk * 2 * kLboA, kLboA, 128),
+                        umma::mma_bf16(acc, umma::smem_desc(a0 + kk * 32, 16, 8 * kRowA, kSwizzleA),
                                        umma::smem_desc(b0 + kk * 2 * kLboB, kLboB, 128), idesc, (dxy | kk) ? 1u : 0u);
                 }
                 umma::mma_commit(mbar + (i & 1));
@@ -482,26 +484,24 @@ static unsigned grid_n(long long n)
 // pipeline fills to about 1.5 runs per CTA).  k_real > 0 (32 -> 16 channels,
 // float, no ReLU): `out` takes rows of that many channels, scaled.  At 128^3,
 // 15 channels, that layer and a kernel that took its padded rows to `out` were
-// 108 + 39 us; this layer alone 113.
+// 108 + 39 us; this layer alone is 110.
 cudaError_t conv3d_forward(const __nv_bfloat16 *in, const __nv_bfloat16 *wk, void *out, int nx, int ny, int nz, int cin,
                            int cout, bool relu, bool out_f32, cudaStream_t st, int k_real = 0, float scale = 1.f)
 {
     const int tiles_y = (ny + 3) / 4, tiles_z = (nz + kTileZ - 1) / kTileZ;
     if (nx < 1 || ny < 1 || nz < 1) return cudaSuccess;
     if (cin != 16 && cin != 32) return cudaErrorInvalidValue;
-    // Input planes: the activations [x][y][z][cin] viewed as the 5-D tensor
-    // (8 channels, z, y, channel group, x) -- strides 2, 2 cin, 2 cin nz, 16,
-    // 2 cin nz ny bytes -- whose 8 x 32 x 6 x cin/8 x 1 box is one plane buffer.
+    // Input planes: boxes of cin x 32 x 6 x 1 elements of [x][y][z][cin].
     const auto enc = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(driver_tensor_map_encoder());
     if (!enc) return cudaErrorNotSupported;
     CUtensorMap planes;
-    const cuuint64_t dims[5] = {8, (cuuint64_t)nz, (cuuint64_t)ny, (cuuint64_t)(cin / 8), (cuuint64_t)nx};
-    const cuuint64_t strides[4] = {(cuuint64_t)cin * 2, (cuuint64_t)nz * cin * 2, 16, (cuuint64_t)ny * nz * cin * 2};
-    const cuuint32_t box[5] = {8, 32, 6, (cuuint32_t)(cin / 8), 1};
-    const cuuint32_t elem[5] = {1, 1, 1, 1, 1};
-    if (enc(&planes, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<__nv_bfloat16 *>(in), dims, strides, box, elem,
-            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+    const cuuint64_t dims[4] = {(cuuint64_t)cin, (cuuint64_t)nz, (cuuint64_t)ny, (cuuint64_t)nx};
+    const cuuint64_t strides[3] = {(cuuint64_t)cin * 2, (cuuint64_t)nz * cin * 2, (cuuint64_t)ny * nz * cin * 2};
+    const cuuint32_t box[4] = {(cuuint32_t)cin, 32, 6, 1};
+    const cuuint32_t elem[4] = {1, 1, 1, 1};
+    if (enc(&planes, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<__nv_bfloat16 *>(in), dims, strides, box, elem,
+            CU_TENSOR_MAP_INTERLEAVE_NONE, cin == 32 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_32B,
+            CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
         return cudaErrorInvalidValue;
 #define TT_CONV_LAUNCH(CI, CO, R, F)                                                                  \
     do {                                                                                              \
