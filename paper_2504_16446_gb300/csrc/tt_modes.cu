@@ -40,6 +40,12 @@ static bool encode_rows(const tt_handle *h, const void *base, int w, int pitch, 
     return true;
 }
 
+// Blocks of 8 x 4 x 8 voxels.
+static long long mode_blocks(const tt_handle *h)
+{
+    return (long long)((h->N[0] + 7) / 8) * ((h->N[1] + 3) / 4) * ((h->N[2] + 7) / 8);
+}
+
 static size_t modes_smem(const tt_handle *h)
 {
     const int M = modes_m(h->R), UP = modes_up(M);
@@ -57,12 +63,18 @@ static size_t modes_smem(const tt_handle *h)
 // (Pixels much finer than voxels put too many rays around a block; the
 // channel kernels take those.)  Coordinates stay below 2^22 in magnitude for
 // volumes and detectors of at most 2^14, which the rounding by kRound needs.
+// At l_max 2 a row is 3 values for 6, and a block's start and end (some 4 us)
+// cost what few projections save: below 32 of them, on volumes of more than a
+// wave of blocks, the channel kernel stays (78 x 66 x 83 voxels, 55 x 70
+// pixels: 104 against 108 us at 28 projections, 384 against 360 at 112; 128^3,
+// 28: 402 against 405; 40^3, less than a wave: 31.6 against 28.2).
 void plan_modes(tt_handle *h)
 {
     h->R = 0;
     if (h->prec == TT_F64 || h->L < 2 || h->L > 8 || !driver_tensor_map_encoder()) return;
     const int limit = 1 << 14;
     if (h->N[0] > limit || h->N[1] > limit || h->N[2] > limit || h->nj > limit || h->nk > limit) return;
+    if (h->L == 2 && h->S < 32 && mode_blocks(h) > (long long)h->n_sm * mode_ctas(16)) return;
     const int R = std::min(h->two_theta == 0.0 ? h->L + 1 : 2 * h->L + 1, h->C);
     if (R > kMaxModes) return;
     int bj = 1, bk = 4;
