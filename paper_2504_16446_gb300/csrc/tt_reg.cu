@@ -100,7 +100,7 @@ __device__ __forceinline__ void tv_point(T g0, T g1, T g2, T inv_delta, T delta,
     }
 }
 
-// A thread walks x through a run of kTvRun planes for one (y, z, channel); the
+// A thread walks x through a run of up to kTvRun planes for one (y, z, channel); the
 // plane behind it stays in registers, so an element takes seven loads and three
 // weights (its own and its y and z predecessors') where taking every weight by
 // itself took sixteen and four, with three index divisions.  An item is a run
@@ -110,14 +110,14 @@ __device__ __forceinline__ void tv_point(T g0, T g1, T g2, T inv_delta, T delta,
 constexpr int kTvRun = 10;
 template <typename T>
 __global__ void __launch_bounds__(256)
-k_tv_huber(const T *__restrict__ c, int nx, int ny, int nz, int K, T delta, T *__restrict__ grad,
+k_tv_huber(const T *__restrict__ c, int nx, int ny, int nz, int K, int run_len, T delta, T *__restrict__ grad,
            double *__restrict__ partials)
 {
     __shared__ double red[32];
     const T inv_delta = T(1) / delta;
     const int row = nz * K;
     const long long plane = (long long)ny * row, segs = (plane + 255) / 256;
-    const long long items = segs * ((nx + kTvRun - 1) / kTvRun);
+    const long long items = segs * ((nx + run_len - 1) / run_len);
     RegSum<T> sum;
     for (long long it = blockIdx.x; it < items; it += gridDim.x) {
         const int run = (int)(it / segs);
@@ -125,7 +125,7 @@ k_tv_huber(const T *__restrict__ c, int nx, int ny, int nz, int K, T delta, T *_
         if (e >= plane) continue;
         const int y = (int)(e / row), zk = (int)(e - (long long)y * row);
         const bool y0 = y >= 1, y1 = y + 1 < ny, z0 = zk >= K, z1 = zk + K < row;
-        const int x0 = run * kTvRun, x1 = min(nx, x0 + kTvRun);
+        const int x0 = run * run_len, x1 = min(nx, x0 + run_len);
         const T *p = c + x0 * plane + e;
         T cc = __ldg(p), cy = y0 ? __ldg(p - row) : T(0), cz = z0 ? __ldg(p - K) : T(0);   // here, y - 1, z - 1
         T back = T(0);                                     // w g_x of the plane behind
@@ -209,10 +209,15 @@ template <typename T>
 static tt_status tv_impl(tt_handle *h, const T *c, double delta, T *grad, double *value_host)
 {
     const long long plane = (long long)h->N[1] * h->N[2] * h->K;
-    const unsigned blocks = reg_grid(h, (plane + 255) / 256 * 256 * ((h->N[0] + kTvRun - 1) / kTvRun));
+    // Shorter runs while the runs do not give every SM two blocks: small volumes
+    // are bound by the planes a thread takes one after the other.
+    const long long segs = (plane + 255) / 256;
+    int run = kTvRun;
+    while (run > 1 && segs * ((h->N[0] + run - 1) / run) < 2 * h->n_sm) run = (run + 1) / 2;
+    const unsigned blocks = reg_grid(h, segs * 256 * ((h->N[0] + run - 1) / run));
     cudaEvent_t ev;
     prof_begin(h, TT_KSLOT_VECTOR, &ev);
-    k_tv_huber<T><<<blocks, 256, 0, h->stream>>>(c, h->N[0], h->N[1], h->N[2], h->K, (T)delta, grad, h->red);
+    k_tv_huber<T><<<blocks, 256, 0, h->stream>>>(c, h->N[0], h->N[1], h->N[2], h->K, run, (T)delta, grad, h->red);
     prof_end(h, TT_KSLOT_VECTOR, ev);
     return reg_finish<T>(h, blocks, value_host);
 }
