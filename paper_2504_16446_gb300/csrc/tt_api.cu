@@ -446,6 +446,25 @@ static long long forward_ctas(const tt_handle *h, bool staged)
     return (long long)((h->nk + TK - 1) / TK) * ((h->nj + TJ - 1) / TJ) * h->S;
 }
 
+ChannelScope::ChannelScope(tt_handle *h_, bool on) : h(on ? h_ : nullptr)
+{
+    if (!h) return;
+    R = h->R;
+    fwd_modes = h->fwd_modes;
+    n_fwd_ctas = h->n_fwd_ctas;
+    h->R = 0;
+    h->fwd_modes = false;
+    h->n_fwd_ctas = forward_ctas(h, h->fwd_staged);
+}
+
+ChannelScope::~ChannelScope()
+{
+    if (!h) return;
+    h->R = R;
+    h->fwd_modes = fwd_modes;
+    h->n_fwd_ctas = n_fwd_ctas;
+}
+
 // Box of the staged forward for projection g: a tile's rays span W = (TJ - 1)
 // |uj| + (TK - 1)|uk| in u at every plane (the rays are parallel), and the
 // rows floor(c) and floor(c) + 1 for c within kStEps of that span number at
@@ -629,6 +648,22 @@ tt_status tt_grad_enqueue(tt_handle *h, const T *c, const T *I, const T *W, T *g
 }
 template tt_status tt_grad_enqueue<float>(tt_handle *, const float *, const float *, const float *, float *);
 template tt_status tt_grad_enqueue<double>(tt_handle *, const double *, const double *, const double *, double *);
+
+// The evaluation as the solvers make it: on 2-byte storage in channels.  Every
+// trial volume is rounded to 11 or 8 bits there, so that a coefficient at a
+// rounding tie turns the last bits of an earlier gradient into a whole unit of
+// the storage: with the sums in another order, single elements of the gradient
+// after three steps moved by up to 4e-3 of its rms (bf16; 1e-3 f16, 3e-5 with
+// FP32 storage).  The channel kernels' order is the one that solves of this form
+// are known by, and keeps every bit of them.
+template <typename T>
+tt_status tt_solver_enqueue(tt_handle *h, const T *c, const T *I, const T *W, T *g)
+{
+    const ChannelScope scope(h, h->ssize() == 2);
+    return tt_grad_enqueue<T>(h, c, I, W, g);
+}
+template tt_status tt_solver_enqueue<float>(tt_handle *, const float *, const float *, const float *, float *);
+template tt_status tt_solver_enqueue<double>(tt_handle *, const double *, const double *, const double *, double *);
 
 static tt_status check_finite_loss(double v)
 {

@@ -483,6 +483,16 @@ inline ModeOut mode_out(const tt_handle *h)
     }
     return m;
 }
+// While in scope with on = true the handle works in channels throughout: the
+// tap-pair march (or the staged one where it was chosen) and k_adjoint.
+struct ChannelScope {
+    tt_handle *h;
+    int R = 0;
+    bool fwd_modes = false;
+    long long n_fwd_ctas = 0;
+    ChannelScope(tt_handle *h, bool on);
+    ~ChannelScope();
+};
 cudaError_t launch_reduce(tt_handle *h, const double *partials, long long n, double *out,
                           const double *add, double mul);
 cudaError_t launch_basis(tt_handle *h, const double *nodes, const double *weights);

@@ -25,7 +25,7 @@
 #include "tt_internal.cuh"
 
 template <typename T>
-tt_status tt_grad_enqueue(tt_handle *h, const T *c, const T *I, const T *W, T *g);
+tt_status tt_solver_enqueue(tt_handle *h, const T *c, const T *I, const T *W, T *g);
 tt_status tt_read_loss(tt_handle *h, double *loss_host);
 
 using namespace tt;
@@ -519,7 +519,7 @@ static tt_status lbfgs_step(tt_lbfgs *st, double *loss_out, int *n_evals_out)
             s = enqueue_trial<T>(st, a);
             if (s != TT_OK) return s;
         }
-        s = tt_grad_enqueue<T>(h, (const T *)st->xt, (const T *)st->I, (const T *)st->W, (T *)st->gt);
+        s = tt_solver_enqueue<T>(h, (const T *)st->xt, (const T *)st->I, (const T *)st->W, (T *)st->gt);
         if (s != TT_OK) return s;
         s = enqueue_pair_dots<T>(st, used);
         if (s != TT_OK) return s;
@@ -631,8 +631,8 @@ tt_status tt_lbfgs_create(tt_handle *h, int m, const void *c0, const void *I, co
     if (e != cudaSuccess) { free_state(st); return cuda_fail(e, "tt_lbfgs_create"); }
     const void *xc = c0 ? st->x : nullptr;
     s = (h->prec != TT_F64)
-            ? tt_grad_enqueue<float>(h, (const float *)xc, (const float *)I, (const float *)W, (float *)st->g)
-            : tt_grad_enqueue<double>(h, (const double *)xc, (const double *)I, (const double *)W, (double *)st->g);
+            ? tt_solver_enqueue<float>(h, (const float *)xc, (const float *)I, (const float *)W, (float *)st->g)
+            : tt_solver_enqueue<double>(h, (const double *)xc, (const double *)I, (const double *)W, (double *)st->g);
     if (s == TT_OK) s = tt_read_loss(h, &st->f);
     if (s == TT_OK) s = (h->prec != TT_F64) ? initial_gram<float>(st) : initial_gram<double>(st);
     if (s != TT_OK) { free_state(st); return s; }
@@ -658,7 +658,7 @@ static tt_status create_ray(tt_handle *h, int m, const T *u, const T *g0, double
     T *x = (T *)st->x, *g = (T *)st->g;
     const size_t bytes = h->esize() * st->n;
     double Lu = 0.0;
-    s = tt_grad_enqueue<T>(h, u, (const T *)I, (const T *)W, g);
+    s = tt_solver_enqueue<T>(h, u, (const T *)I, (const T *)W, g);
     cudaError_t e = cudaSuccess;
     if (s == TT_OK) e = vec_dot<T>(h, u, g0, st->n, st->part, st->dots, nullptr, 1.0);
     if (s == TT_OK && e == cudaSuccess)

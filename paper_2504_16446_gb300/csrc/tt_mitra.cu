@@ -20,7 +20,7 @@
 #include "tt_internal.cuh"
 
 template <typename T>
-tt_status tt_grad_enqueue(tt_handle *h, const T *c, const T *I, const T *W, T *g);
+tt_status tt_solver_enqueue(tt_handle *h, const T *c, const T *I, const T *W, T *g);
 tt_status tt_read_loss(tt_handle *h, double *loss_host);
 // Early loss (tt_api.cu): loss_publish_begin makes the next adjoint launched
 // with reduce_loss publish the loss in the handle's mapped slot and returns
@@ -183,6 +183,7 @@ tt_status sirt_weights_impl(tt_handle *h, const T *W, T *R, T *D)
 template <typename T>
 tt_status sirt_weights(tt_handle *h, const T *W, T *R, T *D)
 {
+    const ChannelScope scope(h, h->ssize() == 2);   // (see tt_solver_enqueue)
     if constexpr (std::is_same<T, double>::value) {
         return sirt_weights_impl<double, double>(h, W, R, D);
     } else {
@@ -233,7 +234,7 @@ static tt_status mitra_step(tt_mitra *m, double *loss_host)
     // the loss (at y) is read as soon as the adjoint has published it; the
     // update stays in flight behind it
     const unsigned long long seq = loss_host ? loss_publish_begin(h) : 0;
-    tt_status s = tt_grad_enqueue<T>(h, (const T *)m->y, (const T *)m->I, (const T *)m->R, (T *)m->g);
+    tt_status s = tt_solver_enqueue<T>(h, (const T *)m->y, (const T *)m->I, (const T *)m->R, (T *)m->g);
     h->loss_publish = 0;
     if (s != TT_OK) return s;
     m->t += 1;

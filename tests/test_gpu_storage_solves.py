@@ -1,0 +1,67 @@
+"""Solves on 2-byte storage keep their bits.  Each trial volume is rounded to 11
+or 8 bits, so a sum taken in another order changes a solve by whole units of the
+storage: the solvers evaluate in channels, whatever a single evaluation does.
+
+two_theta = 1e-200 gives the basis matrix of two_theta = 0 bit for bit, but twice
+the detector modes (2 l_max + 1): more than the mode kernels take at l_max 6 and
+8, and other ones at l_max 2 and 4.  Solves on both handles are the same bits only
+when no mode kernel has part in them."""
+import pytest
+import torch
+
+from paper_2504_16446_gb300 import synth, tt
+
+pytestmark = pytest.mark.gpu
+
+
+def handles(ell, prec, n=(22, 19, 24), n_proj=30):
+    return [tt.Handle(synth.small_setup(n=n, nj=21, nk=23, ell_max=ell, n_proj=n_proj, n_seg=16, seed=ell, two_theta=t),
+                      prec) for t in (0.0, 1e-200)]
+
+
+def data(h, seed):
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(seed)
+    return 4e-3 * torch.rand(h.data_shape, device="cuda", generator=gen)
+
+
+@pytest.mark.parametrize("prec", ["bf16", "f16"])
+@pytest.mark.parametrize("ell", [2, 4, 6, 8])
+def test_lbfgs_keeps_its_bits(ell, prec):
+    a, b = handles(ell, prec)
+    assert torch.equal(a.basis_matrix(), b.basis_matrix())
+    I = data(a, 1)
+    out = []
+    for h in (a, b):
+        opt = tt.LBFGS(h, None, I, log=False)
+        for _ in range(3):
+            opt.step()
+        out.append(opt.get())
+    assert torch.equal(out[0][0], out[1][0]) and torch.equal(out[0][1], out[1][1]) and out[0][2] == out[1][2]
+
+
+@pytest.mark.parametrize("prec", ["bf16", "f16"])
+@pytest.mark.parametrize("ell,n,n_proj", [(4, (22, 19, 24), 30), (8, (22, 19, 24), 30), (8, (41, 40, 44), 60)])
+def test_mitra_keeps_its_bits(ell, n, n_proj, prec):
+    """The last size is one whose forward goes through modes outside a solver."""
+    a, b = handles(ell, prec, n, n_proj)
+    I = data(a, 2)
+    out = []
+    for h in (a, b):
+        opt = tt.MITRA(h, torch.zeros(h.volume_shape, device="cuda"), I)
+        for _ in range(4):
+            opt.step()
+        out.append(opt.get())
+    for x, y in zip(out[0], out[1]):
+        assert torch.equal(x, y) if torch.is_tensor(x) else x == y
+
+
+@pytest.mark.parametrize("prec", ["bf16", "f16"])
+def test_ray_start_keeps_its_bits(prec):
+    a, b = handles(6, prec)
+    I = data(a, 3)
+    u = torch.rand(a.volume_shape, device="cuda", generator=torch.Generator(device="cuda").manual_seed(4))
+    loss0, g0 = a.gradient_residual(None, I)
+    got = [tt.LBFGS.from_ray(h, u, g0, loss0, I, log=False) for h in (a, b)]
+    assert got[0].alpha == got[1].alpha and got[0].loss == got[1].loss
+    assert torch.equal(got[0].get()[1], got[1].get()[1])
