@@ -443,10 +443,6 @@ cudaError_t launch_backcontract(tt_handle *h, const T *R);
 // reduction launch.
 template <typename T, typename S>
 cudaError_t launch_adjoint(tt_handle *h, T *g, bool reduce_loss = false);
-// The adjoint of K-channel G rows (h->G as [S][nj][nk][KP], filled by the
-// caller), whatever the handle's own layout.
-template <typename T, typename S>
-cudaError_t launch_adjoint_channels(tt_handle *h, T *g);
 // Detector modes: set-up (F_s, Q and the operand; enqueued on the handle's
 // stream, nodes as for launch_basis), the adjoint and the back-contraction.
 AdjConst adj_const(const ProjGeom &g);

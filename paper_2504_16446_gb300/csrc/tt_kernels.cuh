@@ -1454,8 +1454,6 @@ cudaError_t adjoint_channels(tt_handle *h, T *g, bool rl)
         }                                                                                      \
     }                                                                                          \
     template <>                                                                                \
-    cudaError_t launch_adjoint_channels<T, S>(tt_handle * h, T * g) { return adjoint_channels<T, S>(h, g, false); } \
-    template <>                                                                                \
     cudaError_t launch_adjoint<T, S>(tt_handle * h, T * g, bool rl)                            \
     {                                                                                          \
         if constexpr (std::is_same<T, float>::value)                                           \

@@ -20,7 +20,7 @@
 #include "tt_internal.cuh"
 
 template <typename T>
-tt_status tt_solver_enqueue(tt_handle *h, const T *c, const T *I, const T *W, T *g);
+tt_status tt_grad_enqueue(tt_handle *h, const T *c, const T *I, const T *W, T *g);
 tt_status tt_read_loss(tt_handle *h, double *loss_host);
 // Early loss (tt_api.cu): loss_publish_begin makes the next adjoint launched
 // with reduce_loss publish the loss in the handle's mapped slot and returns
@@ -167,7 +167,7 @@ tt_status sirt_weights_impl(tt_handle *h, const T *W, T *R, T *D)
         e = cudaGetLastError();
         prof_end(h, TT_KSLOT_VECTOR, ev);
     }
-    if (e == cudaSuccess) e = launch_adjoint_channels<T, S>(h, D);
+    if (e == cudaSuccess) e = launch_adjoint<T, S>(h, D);
     if (e == cudaSuccess) {
         prof_begin(h, TT_KSLOT_VECTOR, &ev);
         k_invert<T><<<blocks_for(h->nvox() * h->K), 256, 0, h->stream>>>(D, h->nvox() * h->K, 1e-6 * h->a * kY00);
@@ -183,7 +183,7 @@ tt_status sirt_weights_impl(tt_handle *h, const T *W, T *R, T *D)
 template <typename T>
 tt_status sirt_weights(tt_handle *h, const T *W, T *R, T *D)
 {
-    const ChannelScope scope(h, h->ssize() == 2);   // (see tt_solver_enqueue)
+    const ChannelScope scope(h, true);   // (see mitra_step)
     if constexpr (std::is_same<T, double>::value) {
         return sirt_weights_impl<double, double>(h, W, R, D);
     } else {
@@ -234,7 +234,14 @@ static tt_status mitra_step(tt_mitra *m, double *loss_host)
     // the loss (at y) is read as soon as the adjoint has published it; the
     // update stays in flight behind it
     const unsigned long long seq = loss_host ? loss_publish_begin(h) : 0;
-    tt_status s = tt_solver_enqueue<T>(h, (const T *)m->y, (const T *)m->I, (const T *)m->R, (T *)m->g);
+    // In channels on every handle: a voxel that few rays graze has a column
+    // sum of a few 1e-3, whose inverse in D multiplies the rounding of the
+    // gradient's tap weights, and only the kernel that took the column sums
+    // rounds them alike.  (With the gradient in modes, x after five steps was
+    // up to twice as far from an FP64 solve: 3.3e-3 against 1.6e-3 relative
+    // at 30 x 28 x 33, l_max 4, 40 projections.)
+    const ChannelScope scope(h, true);
+    tt_status s = tt_grad_enqueue<T>(h, (const T *)m->y, (const T *)m->I, (const T *)m->R, (T *)m->g);
     h->loss_publish = 0;
     if (s != TT_OK) return s;
     m->t += 1;

@@ -65,3 +65,18 @@ def test_ray_start_keeps_its_bits(prec):
     got = [tt.LBFGS.from_ray(h, u, g0, loss0, I, log=False) for h in (a, b)]
     assert got[0].alpha == got[1].alpha and got[0].loss == got[1].loss
     assert torch.equal(got[0].get()[1], got[1].get()[1])
+
+
+@pytest.mark.parametrize("ell,n,n_proj", [(2, (22, 19, 24), 30), (4, (22, 19, 24), 30), (8, (41, 40, 44), 60)])
+def test_mitra_keeps_its_bits_with_float_storage(ell, n, n_proj):
+    """The preconditioner multiplies the rounding of the gradient's tap weights on voxels that few rays graze, so the
+    gradient comes from the kernel that took the column sums."""
+    a, b = handles(ell, "f32", n, n_proj)
+    I = data(a, 5)
+    out = []
+    for h in (a, b):
+        opt = tt.MITRA(h, torch.zeros(h.volume_shape, device="cuda"), I)
+        for _ in range(4):
+            opt.step()
+        out.append(opt.get())
+    assert all(torch.equal(x, y) for x, y in zip(out[0][:3], out[1][:3]))
