@@ -196,18 +196,26 @@ cudaError_t setup_modes(tt_handle *h, const double *frames)
 {
     if (!h->R) return cudaSuccess;
     const int CP = h->CP, R = h->R, step = mode_step(h);
+    // Segment means of the modes by the nodes that B is formed with: B = Q F
+    // holds for them at any segment width, beyond the few turns the rule is
+    // exact on too.
+    double node[kQuadNodes], weight[kQuadNodes];
+    gauss_legendre(kQuadNodes, node, weight);
     std::vector<float> Q((size_t)CP * kModeQ, 0.f);
     for (int c = 0; c < h->C; ++c)
         for (int m = 0; m < R; ++m) {
-            double v;
+            double v = 0.0;
             if (h->q_identity) {
                 v = c == m ? 1.0 : 0.0;
             } else if (m == 0) {
                 v = 1.0;
-            } else {   // segment mean of cos(f phi) or sin(f phi)
+            } else {
                 const double f = (m + 1) / 2 * step, half = 0.5 * (h->seg1[c] - h->seg0[c]);
-                const double mid = f * 0.5 * (h->seg1[c] + h->seg0[c]), sinc = std::sin(f * half) / (f * half);
-                v = ((m & 1) ? std::cos(mid) : std::sin(mid)) * sinc;
+                const double mid = 0.5 * (h->seg1[c] + h->seg0[c]);
+                for (int n = 0; n < kQuadNodes; ++n) {
+                    const double a = f * (mid + half * node[n]);
+                    v += 0.5 * weight[n] * ((m & 1) ? std::cos(a) : std::sin(a));
+                }
             }
             Q[(size_t)c * kModeQ + m] = (float)v;
         }
