@@ -197,7 +197,6 @@ k_march_modes(const ProjGeom *__restrict__ geo, const int *__restrict__ order, c
     // the rounded coordinates' exponent
     const unsigned base = (unsigned)(B * (e2 + e1) + kSlotLead + h) - (unsigned)kRoundBits * (unsigned)(su + 1);
     const unsigned base1 = (unsigned)(B * (f2 + f1) + kSlotLead + h) - (unsigned)kRoundBits * (unsigned)(su1 + 1);
-    const float urm = ur - 0.5f, vrm = vr - 0.5f;          // floor(x) = round(x - 1/2) up to a tap of weight zero
     // Two batches of NB planes: one's taps travel while the other is summed.
     constexpr int NB = M <= 5 ? 2 : 1;
     struct Batch {
@@ -208,8 +207,12 @@ k_march_modes(const ProjGeom *__restrict__ geo, const int *__restrict__ order, c
         for (int t = 0; t < NB; ++t) {
             const int pt = min(p + t, phi);                // (never past the last plane)
             const float pf = (float)pt;
-            const float ub = fmaf(pf, up, urm) + kRound, vb = fmaf(pf, vp, vrm) + kRound;
-            const float wu = fmaf(pf, up, ur) - (ub - kRound), wv = fmaf(pf, vp, vr) - (vb - kRound);
+            // (rounded down, the sum with kRound holds the floor exactly: the taps
+            // are k_forward's, those of weight zero included, whose voxel may hold
+            // a NaN)
+            const float u = fmaf(pf, up, ur), v = fmaf(pf, vp, vr);
+            const float ub = __fadd_rd(u, kRound), vb = __fadd_rd(v, kRound);
+            const float wu = u - (ub - kRound), wv = v - (vb - kRound);
             const int o = (int)((unsigned)(pt * sm) + __float_as_uint(ub) * (unsigned)su + __float_as_uint(vb) + base);
             const float wvh = p + t > phi ? 0.f : (h ? wv : 1.f - wv);
             q.w0[t] = (1.f - wu) * wvh;
