@@ -589,7 +589,12 @@ static tt_status adjoint_impl(tt_handle *h, const T *R, T *g)
         // nothing to contract
         if (h->R && h->q_identity && h->R == 4 * h->R4) {
             TT_CUDA(launch_check_rows(h, R), "check");
-            TT_CUDA(launch_adjoint_modes(h, R, g, false), "adjoint");
+            TT_CUDA(launch_adjoint_modes(h, R, g, false, R), "adjoint");
+            return TT_OK;
+        }
+        if (h->R) {
+            TT_CUDA(launch_backcontract_modes(h, R), "backcontract");
+            TT_CUDA(launch_adjoint_modes(h, (const float *)h->G, g, false, R), "adjoint");
             return TT_OK;
         }
     }
@@ -729,7 +734,16 @@ static tt_status grad_impl(tt_handle *h, const T *c, const T *I, const T *W, T *
     tt_status st = tt_grad_enqueue<T>(h, c, I, W, g);
     h->loss_publish = 0;
     if (st != TT_OK) return st;
-    return seq ? read_published_loss(h, seq, loss_host) : tt_read_loss(h, loss_host);
+    st = seq ? read_published_loss(h, seq, loss_host) : tt_read_loss(h, loss_host);
+    // The modes give NaN where the channels' sums are infinities: an evaluation
+    // with infinite data or coefficients is taken again in channels.  (A ray's
+    // sums that are not finite make the loss not finite.)
+    if (st == TT_NONFINITE && h->R) {
+        const ChannelScope scope(h, true);
+        st = tt_grad_enqueue<T>(h, c, I, W, g);
+        if (st == TT_OK) st = tt_read_loss(h, loss_host);
+    }
+    return st;
 }
 
 // want = TT_F32 for the float entry points (handles of precision TT_F32,
@@ -1080,7 +1094,15 @@ tt_status tt_gradient_residual_host(tt_handle *h, const float *c_host, const flo
     });
     if (st != TT_OK) return st;
     if (!g_map) TT_CUDA(cudaMemcpyAsync(g_host, h->hg, bc, cudaMemcpyDeviceToHost, h->stream), "D2H g");
-    return tt_read_loss(h, loss_host);
+    st = tt_read_loss(h, loss_host);
+    if (st == TT_NONFINITE && h->R) {   // infinities: again in channels (see grad_impl)
+        const ChannelScope scope(h, true);
+        st = tt_grad_enqueue<float>(h, (const float *)h->hc, I, W, g_map ? g_map : (float *)h->hg);
+        if (st != TT_OK) return st;
+        if (!g_map) TT_CUDA(cudaMemcpyAsync(g_host, h->hg, bc, cudaMemcpyDeviceToHost, h->stream), "D2H g");
+        st = tt_read_loss(h, loss_host);
+    }
+    return st;
 }
 
 tt_status tt_profile_enable(tt_handle *h, int enable)

@@ -126,6 +126,7 @@ struct AdjParams {
 // zero padded.
 constexpr int kModeQ = 12;          // padded mode count of Q (at most 9 modes)
 constexpr int kMaxModes = 9;
+constexpr int kModeKMax = 45;       // coefficients of the largest band limit that works in modes (8)
 struct ModeOut {
     const float *Q = nullptr;
     float *G1 = nullptr;
@@ -191,6 +192,20 @@ struct ModeParams {
 struct ModeOrigin {
     double j[4], k[4], jlo, klo;
     int outer_j;
+};
+// What tt_adjoint was given, for voxels that infinite data reach (R NULL: the
+// rows come from a residual).
+struct ModeData {
+    const float *R;
+    const ProjGeom *geo;
+    const float *Bp;
+    int S, nj, nk, C, CP;
+};
+// The packed volume, for rays through infinite coefficients.
+struct ModeVolume {
+    const void *cpad, *cpadx;            // interior origins of the copies
+    const float *Bp;
+    int prec, K, KP;
 };
 // The adjoint's enumeration constants of a projection in FP64 (see AdjProj).
 struct AdjConst {
@@ -461,8 +476,9 @@ long long mode_forward_ctas(const tt_handle *h);
 cudaError_t setup_mode_forward(tt_handle *h, const double *F);
 template <typename S>
 cudaError_t launch_forward_modes(tt_handle *h, float *Iout, const float *I, const float *W, bool grad, int s0, int s1);
-// rows: the mode rows [S][nj][nk][4 R4] (h->G, or a caller's array).
-cudaError_t launch_adjoint_modes(tt_handle *h, const float *rows, float *g, bool reduce_loss);
+// rows: the mode rows [S][nj][nk][4 R4] (h->G, or a caller's array); data: the
+// caller's data that they come from (tt_adjoint), or NULL.
+cudaError_t launch_adjoint_modes(tt_handle *h, const float *rows, float *g, bool reduce_loss, const float *data = nullptr);
 cudaError_t launch_backcontract_modes(tt_handle *h, const float *R);
 // Notes whether a caller's rows are all finite, as the kernels that write rows do.
 cudaError_t launch_check_rows(tt_handle *h, const float *rows);

@@ -1440,8 +1440,6 @@ cudaError_t adjoint_channels(tt_handle *h, T *g, bool rl)
     template <>                                                                                \
     cudaError_t launch_backcontract<T, S>(tt_handle * h, const T *R)                           \
     {                                                                                          \
-        if constexpr (std::is_same<T, float>::value)                                           \
-            if (h->R) return launch_backcontract_modes(h, (const float *)R);                     \
         switch (h->L) {                                                                        \
         case 0: return launch_backcontract_L<T, S, 0>(h, R);                                   \
         case 2: return launch_backcontract_L<T, S, 2>(h, R);                                   \

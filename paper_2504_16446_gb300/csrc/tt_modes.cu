@@ -279,7 +279,7 @@ static int mode_split(int blocks, int units, int slots)
 }
 
 template <int N, int R4, int R1>
-static cudaError_t adjoint_modes_run(tt_handle *h, const float *rows, float *g, bool reduce_loss)
+static cudaError_t adjoint_modes_run(tt_handle *h, const float *rows, float *g, bool reduce_loss, const float *data)
 {
     constexpr int M = 4 * R4 + R1, UP = modes_up(M), KU = modes_ku(M);
     const int tx = (h->N[0] + 7) / 8, ty = (h->N[1] + 3) / 4, tz = (h->N[2] + 7) / 8;
@@ -314,7 +314,8 @@ static cudaError_t adjoint_modes_run(tt_handle *h, const float *rows, float *g, 
             last ? g : (float *)nullptr, h->K, (const double *)h->partials, h->n_fwd_ctas,
             (reduce_loss && ci == 0) ? h->loss_dev : (double *)nullptr,
             (reduce_loss && ci == 0 && h->loss_publish) ? h->loss_slot_dev : (LossSlot *)nullptr, h->loss_publish,
-            (const unsigned *)h->nonfinite, h->rows_id);
+            (const unsigned *)h->nonfinite, h->rows_id,
+            ModeData{last ? data : nullptr, h->geo, (const float *)h->Bp, h->S, h->nj, h->nk, h->C, h->CP});
         (void)cudaGetLastError();
         prof_end(h, TT_KSLOT_ADJOINT, ev);
     }
@@ -322,18 +323,18 @@ static cudaError_t adjoint_modes_run(tt_handle *h, const float *rows, float *g, 
 }
 
 template <int N>
-static cudaError_t adjoint_modes_n(tt_handle *h, const float *rows, float *g, bool rl)
+static cudaError_t adjoint_modes_n(tt_handle *h, const float *rows, float *g, bool rl, const float *data)
 {
-    if (h->R4 == 1) return h->R1 ? adjoint_modes_run<N, 1, 1>(h, rows, g, rl) : adjoint_modes_run<N, 1, 0>(h, rows, g, rl);
-    return h->R1 ? adjoint_modes_run<N, 2, 1>(h, rows, g, rl) : adjoint_modes_run<N, 2, 0>(h, rows, g, rl);
+    if (h->R4 == 1) return h->R1 ? adjoint_modes_run<N, 1, 1>(h, rows, g, rl, data) : adjoint_modes_run<N, 1, 0>(h, rows, g, rl, data);
+    return h->R1 ? adjoint_modes_run<N, 2, 1>(h, rows, g, rl, data) : adjoint_modes_run<N, 2, 0>(h, rows, g, rl, data);
 }
 
-cudaError_t launch_adjoint_modes(tt_handle *h, const float *rows, float *g, bool reduce_loss)
+cudaError_t launch_adjoint_modes(tt_handle *h, const float *rows, float *g, bool reduce_loss, const float *data)
 {
     switch (modes_n(h->K)) {
-    case 16: return adjoint_modes_n<16>(h, rows, g, reduce_loss);
-    case 32: return adjoint_modes_n<32>(h, rows, g, reduce_loss);
-    case 48: return adjoint_modes_n<48>(h, rows, g, reduce_loss);
+    case 16: return adjoint_modes_n<16>(h, rows, g, reduce_loss, data);
+    case 32: return adjoint_modes_n<32>(h, rows, g, reduce_loss, data);
+    case 48: return adjoint_modes_n<48>(h, rows, g, reduce_loss, data);
     default: return cudaErrorInvalidValue;
     }
 }

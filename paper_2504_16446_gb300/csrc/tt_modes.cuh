@@ -212,6 +212,58 @@ __device__ __forceinline__ double sum_fixed_order_half(const double *__restrict_
     return w == 0 ? warp_sum(l < kThreads / 32 ? red[l] : 0.0) : 0.0;
 }
 
+// Infinities.  A voxel that an infinite ray reaches gets NaN from the modes
+// (inf - inf, in the split and in the sum over modes) where the sum over the
+// K channels is an infinity of one sign, or a NaN.  Behind a tt_adjoint whose
+// data are not all finite, this puts the channels' values there, from the
+// caller's data R.  (A kernel of its own behind the adjoint took 4 us of every
+// call.)
+__device__ static void adjoint_infinite_at(const ModeData &d, float *gx, int K, int KP, int x, int y, int z)
+{
+    bool nan = false;
+    for (int i = 0; i < K; ++i) nan = nan || isnan(gx[i]);
+    if (!nan) return;
+    const double at[3] = {(double)x, (double)y, (double)z};
+    float acc[kModeKMax];
+    for (int i = 0; i < K; ++i) acc[i] = 0.f;
+    for (int s = 0; s < d.S; ++s) {
+        const ProjGeom &P = d.geo[s];
+        const double jc = P.jc0 + P.jU * at[P.u] + P.jV * at[P.v] + P.jP * at[P.m];
+        const double kc = P.kc0 + P.kU * at[P.u] + P.kV * at[P.v] + P.kP * at[P.m];
+        const int j1 = (int)fmin(floor(jc + P.hj), d.nj - 1.0), k1 = (int)fmin(floor(kc + P.hk), d.nk - 1.0);
+        for (int j = (int)fmax(ceil(jc - P.hj), 0.0); j <= j1; ++j)
+            for (int k = (int)fmax(ceil(kc - P.hk), 0.0); k <= k1; ++k) {
+                const double du = P.u0 + j * P.uj + k * P.uk + at[P.m] * P.up - at[P.u];
+                const double dv = P.v0 + j * P.vj + k * P.vk + at[P.m] * P.vp - at[P.v];
+                const float w = (float)(P.step * fmax(0.0, 1.0 - fabs(du)) * fmax(0.0, 1.0 - fabs(dv)));
+                const float *r = d.R + (((long long)s * d.nj + j) * d.nk + k) * d.C;
+                bool finite = true;
+                for (int c = 0; c < d.C; ++c) finite = finite && isfinite(r[c]);
+                if (finite || !(w > 0.f)) continue;
+                for (int i = 0; i < K; ++i) {
+                    float b = 0.f;
+                    for (int c = 0; c < d.C; ++c) b = fmaf(d.Bp[((size_t)s * d.CP + c) * KP + i], r[c], b);
+                    acc[i] = fmaf(w, b, acc[i]);
+                }
+            }
+    }
+    for (int i = 0; i < K; ++i)
+        if (isnan(gx[i]) && !isfinite(acc[i])) gx[i] = acc[i];
+}
+// The voxels that this warp wrote (finds its place again, so that the kernel
+// keeps no register for it).
+__device__ __noinline__ static void adjoint_infinite(const ModeData &d, bool any, float *g, int K, int KP, int nx, int ny,
+                                                     int nz, int ty, int tz)
+{
+    if (!any) return;
+    __syncwarp();
+    const int b = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int X = b / (tz * ty) * 8, y = (b / tz) % ty * 4 + warp, z = b % tz * 8 + lane;
+    if (warp >= 4 || y >= ny || lane >= 8 || z >= nz) return;
+    for (int x = X + blockIdx.y; x < min(X + 8, nx); x += gridDim.y)
+        adjoint_infinite_at(d, g + (((long long)x * ny + y) * nz + z) * K, K, KP, x, y, z);
+}
+
 template <int N, int R4, int R1>
 __global__ void __launch_bounds__(kModeThreads, mode_ctas(N))
 k_adjoint_modes(const __grid_constant__ ModeParams P, const __grid_constant__ TmaDesc tm4,
@@ -219,7 +271,8 @@ k_adjoint_modes(const __grid_constant__ ModeParams P, const __grid_constant__ Tm
                 const float *__restrict__ FB, int bj, int bk, int nx, int ny, int nz, int ty, int tz,
                 float *__restrict__ gpad, int KP, int accumulate, float *__restrict__ gout, int K,
                 const double *__restrict__ loss_partials, long long n_partials, double *__restrict__ loss_out,
-                LossSlot *loss_slot, unsigned long long loss_seq, const unsigned *__restrict__ nonfinite, unsigned rows_id)
+                LossSlot *loss_slot, unsigned long long loss_seq, const unsigned *__restrict__ nonfinite, unsigned rows_id,
+                const __grid_constant__ ModeData data)
 {
     constexpr int M = 4 * R4 + R1, SW = 2 * M, UP = modes_up(M), KU = modes_ku(M), V = 2, NVW = kModeVox / V / 32;
     constexpr int kDrain = (N == 16 ? 4 : 8) / UP;                // units per D_hi chain
@@ -509,6 +562,7 @@ k_adjoint_modes(const __grid_constant__ ModeParams P, const __grid_constant__ Tm
             }
         }
     if (split > 1) umma::cluster_sync();                   // no CTA leaves while its sums are read
+    if (data.R) adjoint_infinite(data, *nonfinite == rows_id, gout, K, KP, nx, ny, nz, ty, tz);
 }
 
 // ------------------------------------------------- back-contraction to modes

@@ -138,6 +138,44 @@ k_map_modes(const S *__restrict__ cpad, const float2 *__restrict__ FM, const int
     if (warp == 0) umma::tmem_dealloc(tb, kMapCols);
 }
 
+// A ray through an infinite coefficient is a NaN in every mode where the sum
+// over channels is an infinity of one sign, or a NaN: the channels' values of
+// such a ray, from the packed volume.
+template <typename S>
+__device__ void project_infinite_as(const ModeVolume &V, const ProjGeom &P, int s, int j, int k, int C, int CP, float *out)
+{
+    float ur, vr, lo = 0.f, hi = (float)(P.Nm - 1);
+    ray_base<float>(P, j, k, ur, vr);
+    const float up = (float)P.up, vp = (float)P.vp;
+    clip_planes<float>(ur, up, P.Nu, lo, hi);
+    clip_planes<float>(vr, vp, P.Nv, lo, hi);
+    const S *vol = (const S *)(P.copy ? V.cpadx : V.cpad);
+    float acc[kModeKMax];
+    for (int i = 0; i < V.K; ++i) acc[i] = 0.f;
+    const int phi = min(P.Nm - 1, (int)ceilf(hi));
+    for (int p = max(0, (int)floorf(lo)); p <= phi; ++p) {
+        const float u = fmaf((float)p, up, ur), v = fmaf((float)p, vp, vr), fu = floorf(u), fv = floorf(v);
+        const int iu = min(max((int)fu, -2), P.Nu), iv = min(max((int)fv, -2), P.Nv);
+        for (int t = 0; t < 4; ++t) {
+            const float w = (t & 1 ? u - fu : 1.f - (u - fu)) * (t & 2 ? v - fv : 1.f - (v - fv));
+            const S *tap = vol + ((long long)p * P.sm + (long long)(iu + (t & 1)) * P.su + iv + (t >> 1)) * V.KP;
+            for (int i = 0; i < V.K; ++i) acc[i] = fmaf(w, float(tap[i]), acc[i]);
+        }
+    }
+    for (int c = 0; c < C; ++c) {
+        float v = 0.f;
+        for (int i = 0; i < V.K; ++i) v = fmaf(V.Bp[((size_t)s * CP + c) * V.KP + i], acc[i], v);
+        if (!isfinite(v)) out[c] = v;
+    }
+}
+__device__ __noinline__ static void project_infinite(const ModeVolume &V, const ProjGeom &P, int s, int j, int k, int C,
+                                                     int CP, float *out)
+{
+    if (V.prec == TT_BF16) project_infinite_as<__nv_bfloat16>(V, P, s, j, k, C, CP, out);
+    else if (V.prec == TT_F16) project_infinite_as<__half>(V, P, s, j, k, C, CP, out);
+    else project_infinite_as<float>(V, P, s, j, k, C, CP, out);
+}
+
 // ------------------------------------------------------------ march kernel
 //
 // Two lanes per ray, lane h taking the tap column iv + h: the pair of taps of
@@ -153,7 +191,8 @@ k_march_modes(const ProjGeom *__restrict__ geo, const int *__restrict__ order, c
               long long slot_floats, long long slot_vox, int nx, int ny, int nz, int nj, int nk, int C, int CP,
               int tiles_k, const float *__restrict__ Q, float *__restrict__ Iout, const float *__restrict__ Id,
               const float *__restrict__ Wd, float *__restrict__ G, float *__restrict__ G1, int nk1,
-              double *__restrict__ partials, unsigned *__restrict__ nonfinite, unsigned rows_id)
+              double *__restrict__ partials, unsigned *__restrict__ nonfinite, unsigned rows_id,
+              const __grid_constant__ ModeVolume V)
 {
     constexpr int R4 = M / 4, R1 = M & 1;
     constexpr bool GRAD = MODE != kProject;
@@ -310,6 +349,11 @@ k_march_modes(const ProjGeom *__restrict__ geo, const int *__restrict__ order, c
             }
         }
     }
+    if constexpr (!GRAD) {
+        const bool again = valid && !rows_finite(acc);
+        __syncwarp();
+        if (again && h == 0) project_infinite(V, P, s, j, k, C, CP, Iout + pix * C);
+    }
     if constexpr (GRAD) {
 #pragma unroll
         for (int i = 0; i < M; ++i) gm[i] = 2.f * (gm[i] + __shfl_xor_sync(0xffffffffu, gm[i], 1));
@@ -367,7 +411,10 @@ static cudaError_t run_march(tt_handle *h, const int *order, int n, const float 
     prof_begin(h, TT_KSLOT_FORWARD, &ev);
     k_march_modes<M, MODE><<<dim3(tiles_k * tiles_j, n), kMarchThreads, h->CP * kModeQ * 4, h->stream>>>(
         h->geo, order, slots, h->slot_floats, h->slot_vox, h->N[0], h->N[1], h->N[2], h->nj, h->nk, h->C, h->CP, tiles_k,
-        mo.Q, Iout, I, W, (float *)h->G, mo.G1, mo.nk1, h->partials, mo.nonfinite, mo.rows_id);
+        mo.Q, Iout, I, W, (float *)h->G, mo.G1, mo.nk1, h->partials, mo.nonfinite, mo.rows_id,
+        ModeVolume{(const char *)h->cpad + h->cpad_origin * h->KP * h->ssize(),
+                   (const char *)h->cpad + (h->pad_vox + h->cpadx_origin) * h->KP * h->ssize(), (const float *)h->Bp,
+                   h->prec, h->K, h->KP});
     const cudaError_t e = cudaGetLastError();
     prof_end(h, TT_KSLOT_FORWARD, ev);
     return e;
