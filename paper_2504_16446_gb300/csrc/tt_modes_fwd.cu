@@ -28,18 +28,25 @@ struct RowRegs {
 // the rows of the A operand in tensor memory; B holds the F rows of a group of
 // projections; the accumulator's row of a voxel is its mode vectors of all
 // those projections, stored as rows of four floats (and single values) that
-// consecutive lanes write contiguously.  The cross products come first, so the
-// sums' truncation at full magnitude happens in the KP / 8 steps of hi * hi
-// only.  Warps w and w + 4 share tensor-memory lanes 32 w .., split the
+// consecutive lanes write contiguously.  The tensor cores truncate each step's
+// sum, a bias that all voxels of a ray add up.  So the order-0 coefficient,
+// which exceeds the others in any object and has the same factor Y_00 in every
+// projection, stays out of the products and is added to the drained rows by one
+// rounded FMA; the cross products come first, then hi * hi from the highest
+// order down, so that what is truncated is small.  (With order 0 among the
+// products and the orders ascending, projections of objects were 4e-7 (l_max 6)
+// and 6e-7 (l_max 8) off, all of one sign; now 1e-7, as the direct march.)
+// Warps w and w + 4 share tensor-memory lanes 32 w .., split the
 // coefficients of their voxels between them and store every other four
 // projections.
 constexpr int kMapThreads = 256;
+constexpr float kY00f = 0.28209479177387814f;             // 1 / (2 sqrt(pi))
 
 template <typename S, int KP, int M>
 __global__ void __launch_bounds__(kMapThreads, 2)
 k_map_modes(const S *__restrict__ cpad, const float2 *__restrict__ FM, const int *__restrict__ order, int nproj,
             int group, int n_in, int ny, int n_out, float *__restrict__ slots, long long slot_floats,
-            long long slot_vox)
+            long long slot_vox, int n0 /* modes that order 0 contributes to */)
 {
     constexpr int R4 = M / 4, R1 = M & 1, NC = KP / 2;
     extern __shared__ __align__(128) unsigned char map_smem[];
@@ -71,19 +78,23 @@ k_map_modes(const S *__restrict__ cpad, const float2 *__restrict__ FM, const int
     const S *src = cpad + half * NC;
     int rowi = 0, in = 0;
     RowRegs<S, NC> c;
+    float next0 = 0.f;                                     // the voxel's order-0 coefficient
     auto fetch = [&](long long t) {
         const int v = (int)min(t * 128 + row, (long long)npos - 1);
         in = v % n8;
         const int r = v / n8, y = r % ny, out = r / ny;
         rowi = (out + kSlotBorder) * (ny + 2 * kSlotBorder) + y + kSlotBorder;
         // (behind a row's end the packed copy has two zeros, then the next row)
-        c.load(src + (((long long)(out + 2) * (ny + 4) + (y + 2)) * (n_in + 4) + min(in, n_in) + 2) * KP);
+        const S *at = src + (((long long)(out + 2) * (ny + 4) + (y + 2)) * (n_in + 4) + min(in, n_in) + 2) * KP;
+        c.load(at);
+        next0 = half ? float(at[-NC]) : c.get(0);
     };
     fetch(blockIdx.x);
     bool ok = true;                                        // false once a wait gave up: the rest is NaN
     uint32_t phase = 0;
     for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x, phase ^= 1) {
         const bool live = tile * 128 + row < npos;
+        const float y0 = next0;
         const int here4 = rowi * slot_pitch4(n_in) + in + kSlotLead, here1 = rowi * slot_pitch1(n_in) + in + kSlotLead;
 #pragma unroll
         for (int i = 0; i < NC; i += 8) {
@@ -106,7 +117,7 @@ k_map_modes(const S *__restrict__ cpad, const float2 *__restrict__ FM, const int
                 umma::mma_tf32_ts(tb + dcol, tb + KP + 8 * ks, bh, idesc, 1);
             }
 #pragma unroll
-            for (int ks = 0; ks < KP / 8; ++ks)
+            for (int ks = KP / 8 - 1; ks >= 0; --ks)
                 umma::mma_tf32_ts(tb + dcol, tb + 8 * ks, umma::smem_desc(sh + ks * N * 32, N * 16, 128), idesc, 1);
             umma::mma_commit(&done);
         }
@@ -116,6 +127,14 @@ k_map_modes(const S *__restrict__ cpad, const float2 *__restrict__ FM, const int
         for (int p = 4 * half; p < P; p += 8) {
             float d[4 * M];
             umma::tmem_ldn<4 * M>(tw + dcol + p * M, d);
+#pragma unroll
+            for (int t = 0; t < 4; ++t) {
+                d[t * M] = fmaf(kY00f, y0, d[t * M]);
+                if (n0 > 1)
+#pragma unroll
+                    for (int i = 1; i < M; ++i)
+                        if (i < n0) d[t * M + i] = fmaf(kY00f, y0, d[t * M + i]);
+            }
             if (!ok)
 #pragma unroll
                 for (int i = 0; i < 4 * M; ++i) d[i] = __int_as_float(0x7fc00000);
@@ -395,7 +414,7 @@ static cudaError_t run_map(tt_handle *h, const int *order, int n, int copy)
     prof_begin(h, TT_KSLOT_PACK, &ev);
     kern<<<dim3((unsigned)gx, groups), kMapThreads, smem, h->stream>>>(
         (const S *)h->cpad + (copy ? h->pad_vox * KP : 0), (const float2 *)h->FM, order, n, group, n_in, h->N[1], n_out,
-        h->slots + (copy ? h->slots1 : 0), h->slot_floats, h->slot_vox);
+        h->slots + (copy ? h->slots1 : 0), h->slot_floats, h->slot_vox, h->q_identity ? h->R : 1);
     const cudaError_t e = cudaGetLastError();
     prof_end(h, TT_KSLOT_PACK, ev);
     return e;
@@ -449,7 +468,7 @@ long long mode_forward_ctas(const tt_handle *h)
     return (long long)((h->nk + kMarchTK - 1) / kMarchTK) * ((h->nj + kMarchTJ - 1) / kMarchTJ) * h->S;
 }
 
-// F rows for the map, [S][M][KP] (hi, lo).
+// F rows for the map, [S][M][KP] (hi, lo), without order 0 (see k_map_modes).
 __global__ void k_map_operand(const double *__restrict__ F, int S, int R, int K, int M, int KP, float2 *__restrict__ FM)
 {
     const long long n = (long long)S * M * KP;
@@ -457,7 +476,7 @@ __global__ void k_map_operand(const double *__restrict__ F, int S, int R, int K,
          e += (long long)gridDim.x * blockDim.x) {
         const int k = (int)(e % KP), m = (int)(e / KP % M), s = (int)(e / ((long long)KP * M));
         float2 v = make_float2(0.f, 0.f);
-        if (m < R && k < K) {
+        if (m < R && k > 0 && k < K) {
             const double f = F[((size_t)s * R + m) * K + k];
             uint32_t hi, lo;
             tf32_split((float)f, hi, lo);
