@@ -531,10 +531,13 @@ k_adjoint_modes(const __grid_constant__ ModeParams P, const __grid_constant__ Tm
                                      : "memory");
             }
     }
+    // The columns go back before the CTA waits for its cluster: a peer may still
+    // be waiting to allocate its own, and no CTA may hold any while it waits.
     umma::fence_before_sync();
-    if (split > 1) umma::cluster_sync();
-    else __syncthreads();
+    __syncthreads();
+    umma::fence_after_sync();
     if (warp == NVW) umma::tmem_dealloc(tbase, 2 * COLS);
+    if (split > 1) umma::cluster_sync();
     // The cluster's CTAs share out the runs and add the CTAs' sums in their order.
     const int nz8 = min(8, nz - Z) * K;
     if (warp < NVW && Y + warp < ny)
