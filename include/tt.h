@@ -127,13 +127,14 @@ tt_status tt_destroy(tt_handle *h);
 tt_status tt_set_stream(tt_handle *h, void *stream);
 /* Chooses the kernel of the forward projection (Eq. forward_model, the
  * Joseph discretisation of Sec. "real_space_geom") for the calls that follow:
- *   0  automatic (the default): for TT_F32 and 2-byte handles with ell_max 6
- *      or 8 and at least 3e6 voxels x projections whose rows have at most nine
- *      detector modes, the mode march -- per projection the volume is mapped
- *      to its modes (tensor cores, into slots of at most 4 GB per orientation,
- *      or one volume, that tt_create allocates when there is memory for
- *      them) and the rays march the mapped volume; the tap-pair march (1)
- *      otherwise: the faster ones on every workload measured;
+ *   0  automatic (the default): for TT_F32 handles with ell_max 6 or 8 and
+ *      2-byte handles with ell_max 8, at least 3e6 voxels x projections and at
+ *      most nine detector modes, where the rays' steps through the volume are
+ *      enough to pay for mapping it, the mode march -- per projection the
+ *      volume is mapped to its modes (tensor cores, into slots of at most 4 GB
+ *      per orientation, or one volume, that tt_create allocates when there is
+ *      memory for them) and the rays march the mapped volume; the tap-pair
+ *      march (1) otherwise: the faster ones on every workload measured;
  *   1  the tap-pair march: bilinear taps read from the L1/L2-resident volume;
  *   2  the staged march: for each plane a copy warp moves the box of a ray
  *      tile's taps into shared memory with one tensor copy, and the rays read

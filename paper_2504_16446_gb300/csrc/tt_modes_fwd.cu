@@ -499,17 +499,48 @@ static std::vector<int> projection_order(tt_handle *h)
     return order;
 }
 
-// Sizes of the mode forward.  It pays for l_max 6 and 8 once there is enough
-// work for its launches and its extra pass over the mapped volumes; measured,
-// whole projection in us, modes / direct march: l_max 6, 28^3 x 60 projections
-// (1.3e6 voxels x projections) 65 / 61, x 150 (3.3e6) 110 / 122, 100^3 x 180
-// 2912 / 4516; l_max 8, 28^3 x 60 69 / 67, 56^3 x 24 (4.2e6) 148 / 163, 128^3
-// x 240 7712 / 18390.  At l_max 4 the mapped volume (five values for
-// fifteen) saves too little: 64^3 x 120 about 360 / 310.
+// Steps of rays through the volume: planes times the detector pixels that the
+// volume's shadow covers (its bounding box), over all projections.
+static double ray_steps(const tt_handle *h)
+{
+    double steps = 0.0;
+    for (const ProjGeom &g : h->geo_host) {
+        auto covered = [&](double at0, double u, double v, double p, int n) {
+            double lo = at0, hi = at0;
+            for (const double d : {u * (g.Nu - 1), v * (g.Nv - 1), p * (g.Nm - 1)}) (d < 0 ? lo : hi) += d;
+            return std::max(0.0, std::min(n - 1.0, hi) - std::max(0.0, lo) + 1.0);
+        };
+        steps += covered(g.jc0, g.jU, g.jV, g.jP, h->nj) * covered(g.kc0, g.kU, g.kV, g.kP, h->nk) * g.Nm;
+    }
+    return steps;
+}
+
+// Sizes of the mode forward, and when it pays (l_max 6 and 8; at 4 the mapped
+// volume, five values for fifteen, saves too little: 64^3 x 120 about 360 / 310
+// us).  The map costs by voxels times projections (8.4e-6 to 1.1e-5 us each,
+// whatever the detector), what the march of the mapped volume saves goes by the
+// steps of rays (FP32: 1.9e-5 us each at l_max 6, 2.3e-5 at 8; 2-byte storage,
+// whose direct march reads half the bytes: 0.7e-5 and 1.35e-5), and there are
+// some 15 us of further launches; hence a floor and a share of the voxels for
+// the steps.  Measured, whole projection in us, modes / direct march, 120
+// projections unless said:
+//   l_max 6  28^3 x 140 98 / 115; 64^3 on 64^2 pixels 558 / 840, on 44^2 451 / 481,
+//            on 38^2 440 / 373, on 32^2 370 / 286, on 8^2 342 / 45; 128^3 on
+//            128^2 3721 / 6183, on 89^2 3043 / 3711, on 76^2 2763 / 2715, on 16^2
+//            2120 / 286; 32^3 on 96^2 172 / 271
+//   l_max 8  28^3 x 140 108 / 127; 64^3 on 64^2 576 / 960, on 38^2 456 / 419; 128^3
+//            on 128^2 3790 / 7400, on 76^2 2827 / 3360, on 64^2 2580 / 2334, on
+//            16^2 2177 / 402
+//   2 bytes  l_max 6: 64^3 549 / 402, 128^3 3655 / 2958: never; l_max 8: 28^3 x 160
+//            125 / 110, 40^3 201 / 185, 64^3 568 / 649, 128^3 3777 / 5130, on 64^2
+//            2522 / 1662; 32^3 on 96^2 179 / 241
 void plan_mode_forward(tt_handle *h)
 {
     h->slot_floats = 0;
-    if (!h->R || h->KP < 32 || h->nvox() * h->S < 3000000) return;
+    const bool half = h->ssize() == 2;
+    const double work = (double)h->nvox() * h->S;
+    if (!h->R || h->KP < 32 || work < 3e6 || (half && h->KP < 48)) return;
+    if (ray_steps(h) < (half ? 2e6 + 0.85 * work : 1e6 + (h->KP < 48 ? 0.43 : 0.33) * work)) return;
     h->order_host = projection_order(h);
     long long single = 0;
     for (int c = 0; c < 2; ++c) {

@@ -15,7 +15,7 @@ pytestmark = pytest.mark.gpu
 @pytest.mark.parametrize("prec", ["f32", "bf16", "f16"])
 @pytest.mark.parametrize("ell,n_seg", [(6, 8), (6, 5), (8, 8), (8, 12), (8, 4)])
 def test_objects_project_without_bias(ell, n_seg, prec):
-    st = synth.small_setup(n=(64, 57, 64), nj=57, nk=64, ell_max=ell, n_proj=80, n_seg=n_seg, seed=ell)
+    st = synth.small_setup(n=(64, 57, 64), nj=57, nk=64, ell_max=ell, n_proj=120, n_seg=n_seg, seed=ell)
     h, ref = tt.Handle(st, prec), tt.Handle(st, "f64")
     gen = torch.Generator(device="cuda")
     gen.manual_seed(5)
