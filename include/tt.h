@@ -131,10 +131,11 @@ tt_status tt_set_stream(tt_handle *h, void *stream);
  *      2-byte handles with ell_max 8, at least 3e6 voxels x projections and at
  *      most nine detector modes, where the rays' steps through the volume are
  *      enough to pay for mapping it, the mode march -- per projection the
- *      volume is mapped to its modes (tensor cores, into slots of at most 4 GB
- *      per orientation, or one volume, that tt_create allocates when there is
- *      memory for them) and the rays march the mapped volume; the tap-pair
- *      march (1) otherwise: the faster ones on every workload measured;
+ *      volume is mapped to its modes (tensor cores, into slots that tt_create
+ *      allocates: 2 to 4 GB per orientation at most, and a sixteenth of the
+ *      free memory; the handle gives them up when another allocation of its
+ *      own or of its solvers fails) and the rays march the mapped volume; the
+ *      tap-pair march (1) otherwise: the faster ones on every workload measured;
  *   1  the tap-pair march: bilinear taps read from the L1/L2-resident volume;
  *   2  the staged march: for each plane a copy warp moves the box of a ray
  *      tile's taps into shared memory with one tensor copy, and the rays read

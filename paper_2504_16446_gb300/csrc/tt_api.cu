@@ -465,6 +465,22 @@ ChannelScope::~ChannelScope()
     h->n_fwd_ctas = n_fwd_ctas;
 }
 
+cudaError_t handle_malloc(tt_handle *h, void **p, size_t bytes)
+{
+    cudaError_t e = cudaMalloc(p, bytes);
+    if (e == cudaErrorMemoryAllocation && h->slots) {
+        (void)cudaGetLastError();
+        cudaFree(h->slots);                              // (waits for the work that uses them)
+        h->slots = nullptr;
+        if (h->fwd_modes) {
+            h->fwd_modes = false;
+            h->n_fwd_ctas = forward_ctas(h, h->fwd_staged);
+        }
+        e = cudaMalloc(p, bytes);
+    }
+    return e;
+}
+
 // Box of the staged forward for projection g: a tile's rays span W = (TJ - 1)
 // |uj| + (TK - 1)|uk| in u at every plane (the rays are parallel), and the
 // rows floor(c) and floor(c) + 1 for c within kStEps of that span number at
@@ -1042,10 +1058,10 @@ tt_status tt_gradient_residual_host(tt_handle *h, const float *c_host, const flo
     // g_host gets the gradient with one copy.
     float *g_map = (float *)mapped_device_pointer(g_host);
     const int Q = std::min(8, h->S);
-    if (!h->hc) TT_CUDA(cudaMalloc(&h->hc, bc), "host-path cudaMalloc");
-    if (!g_map && !h->hg) TT_CUDA(cudaMalloc(&h->hg, bc), "host-path cudaMalloc");
-    if (!h->hI) TT_CUDA(cudaMalloc(&h->hI, bd), "host-path cudaMalloc");
-    if (W_host && !h->hW) TT_CUDA(cudaMalloc(&h->hW, bd), "host-path cudaMalloc");
+    if (!h->hc) TT_CUDA(handle_malloc(h, &h->hc, bc), "host-path cudaMalloc");
+    if (!g_map && !h->hg) TT_CUDA(handle_malloc(h, &h->hg, bc), "host-path cudaMalloc");
+    if (!h->hI) TT_CUDA(handle_malloc(h, &h->hI, bd), "host-path cudaMalloc");
+    if (W_host && !h->hW) TT_CUDA(handle_malloc(h, &h->hW, bd), "host-path cudaMalloc");
     if (!h->copy_stream) TT_CUDA(cudaStreamCreateWithFlags(&h->copy_stream, cudaStreamNonBlocking), "copy stream");
     for (cudaStream_t &t : h->side)
         if (!t) TT_CUDA(cudaStreamCreateWithFlags(&t, cudaStreamNonBlocking), "side stream");

@@ -159,7 +159,6 @@ constexpr int kModeVox = 256;                  // voxels of a CTA: 8 (x) x 4 (y)
 constexpr int kSlotBorder = 3, kSlotLead = 8;
 __host__ __device__ constexpr int slot_pitch4(int n) { return (n + kSlotLead + 7) / 8 * 8 + 2; }
 __host__ __device__ constexpr int slot_pitch1(int n) { return (n + kSlotLead + 15) / 32 * 32 + 16; }
-constexpr long long kSlotBytes = 4LL << 30;    // slots of either copy
 constexpr uint32_t kMapCols = 256;             // tensor-memory columns of a map CTA
 constexpr int kModeStages = 3;                 // units in flight
 constexpr uint32_t kModeWaitTries = 1u << 20;
@@ -458,6 +457,9 @@ cudaError_t launch_backcontract(tt_handle *h, const T *R);
 // reduction launch.
 template <typename T, typename S>
 cudaError_t launch_adjoint(tt_handle *h, T *g, bool reduce_loss = false);
+// cudaMalloc for what is allocated later than the handle: a handle whose mode
+// forward holds memory that is wanted gives its slots up and marches the volume.
+cudaError_t handle_malloc(tt_handle *h, void **p, size_t bytes);
 // Detector modes: set-up (F_s, Q and the operand; enqueued on the handle's
 // stream, nodes as for launch_basis), the adjoint and the back-contraction.
 AdjConst adj_const(const ProjGeom &g);

@@ -571,7 +571,7 @@ static tt_status alloc_state(tt_handle *h, int m, const void *I, const void *W, 
     st->W = W;
     const size_t bytes = h->esize() * st->n;
     const size_t pitch = (bytes + 255) / 256 * 256;
-    cudaError_t e = cudaMalloc(&st->slab, pitch * (7 + 2 * (size_t)m));
+    cudaError_t e = handle_malloc(h, &st->slab, pitch * (7 + 2 * (size_t)m));
     if (e != cudaSuccess) { free_state(st); return cuda_fail(e, "L-BFGS state: cudaMalloc"); }
     char *base = (char *)st->slab;
     void **bufs[] = {&st->x, &st->g, &st->d, &st->xt, &st->gt, &st->ss, &st->ys};
@@ -584,8 +584,8 @@ static tt_status alloc_state(tt_handle *h, int m, const void *I, const void *W, 
     }
     const size_t rows = 6 + 6 * (size_t)m;
     st->pair_blocks = 4 * h->n_sm;
-    e = cudaMalloc(&st->part, sizeof(double) * std::max<size_t>(rows * st->pair_blocks, dot_blocks(h)));
-    if (e == cudaSuccess) e = cudaMalloc(&st->dots, sizeof(double) * rows);
+    e = handle_malloc(h, (void **)&st->part, sizeof(double) * std::max<size_t>(rows * st->pair_blocks, dot_blocks(h)));
+    if (e == cudaSuccess) e = handle_malloc(h, (void **)&st->dots, sizeof(double) * rows);
     if (e == cudaSuccess) e = cudaMallocHost(&st->pinned, sizeof(double) * rows);
     if (e != cudaSuccess) { free_state(st); return cuda_fail(e, "L-BFGS state"); }
     *out = st;

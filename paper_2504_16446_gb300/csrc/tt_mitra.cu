@@ -292,11 +292,11 @@ tt_status tt_mitra_create(tt_handle *h, const void *c0, const void *I, const voi
     m->eta = eta;
     m->momentum = momentum;
     const size_t vb = h->esize() * m->n, db = h->esize() * h->ndata();
-    cudaError_t e = cudaMalloc(&m->x, vb);
-    if (e == cudaSuccess) e = cudaMalloc(&m->y, vb);
-    if (e == cudaSuccess) e = cudaMalloc(&m->g, vb);
-    if (e == cudaSuccess) e = cudaMalloc(&m->D, vb);
-    if (e == cudaSuccess) e = cudaMalloc(&m->R, db);
+    cudaError_t e = handle_malloc(h, &m->x, vb);
+    if (e == cudaSuccess) e = handle_malloc(h, &m->y, vb);
+    if (e == cudaSuccess) e = handle_malloc(h, &m->g, vb);
+    if (e == cudaSuccess) e = handle_malloc(h, &m->D, vb);
+    if (e == cudaSuccess) e = handle_malloc(h, &m->R, db);
     if (e == cudaSuccess) e = cudaMemcpyAsync(m->x, c0, vb, cudaMemcpyDeviceToDevice, h->stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(m->y, c0, vb, cudaMemcpyDeviceToDevice, h->stream);
     if (e != cudaSuccess) { free_mitra(m); return cuda_fail(e, "tt_mitra_create"); }

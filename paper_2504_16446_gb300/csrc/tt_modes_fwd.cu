@@ -550,8 +550,25 @@ void plan_mode_forward(tt_handle *h)
         single = std::max(single, rows * slot_pitch1(in) * h->R1);
     }
     h->slot_floats = (h->slot_vox * 4 * h->R4 + single + 63) / 64 * 64;
+    // Slots for either copy's projections: two gigabytes, four where those hold
+    // fewer than 24, and at most a sixteenth of the free memory, so that what
+    // the caller and the solvers allocate later finds room; fewer than five (of
+    // as many projections) are slower than the direct march.  Whole projections
+    // in ms by gigabytes of slots 0.5 / 1 / 2 / 4, direct: 100^3, l_max 6, 180
+    // projections (44 MB a slot) 3.37 / 3.09 / 2.86 / 2.77, 4.47; 128^3, l_max 8,
+    // 240 (79 MB) 12.3 / 8.8 / 7.93 / 7.89, 13.9; 200^3, l_max 6, 60 (297 MB) 28.5 /
+    // 13.4 / 8.9 / 7.4, 11.9; 256^3, l_max 8, 36 (602 MB) 40.8 / 40.8 / 18.3 / 13.2,
+    // 21.6.
+    size_t free_bytes = 0, total = 0;
+    if (cudaMemGetInfo(&free_bytes, &total) != cudaSuccess) (void)cudaGetLastError();
+    const long long slot = 4 * h->slot_floats, gb = 1LL << 30;
+    const long long bytes = std::min(std::min(4 * gb, std::max(2 * gb, 24 * slot)), (long long)(free_bytes / 16));
     const int most = std::max(h->order_begin[1], h->S - h->order_begin[1]);
-    h->chunk = (int)std::max<long long>(1, std::min<long long>(most, kSlotBytes / (4 * h->slot_floats)));
+    h->chunk = (int)std::min<long long>(most, bytes / slot);
+    if (h->chunk < std::min(most, 5)) {
+        h->slot_floats = 0;
+        return;
+    }
     // the copies' borders coincide in cubic volumes: one set of slots serves both
     h->slots1 = h->N[0] == h->N[2] || h->order_begin[1] == 0 || h->order_begin[1] == h->S ? 0 : h->chunk * h->slot_floats;
 }
