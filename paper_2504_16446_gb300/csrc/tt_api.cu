@@ -423,7 +423,7 @@ static void free_handle(tt_handle *h)
 {
     if (!h) return;
     cudaFree(h->geo); cudaFree(h->tmaps); cudaFree(h->B64); cudaFree(h->Bp); cudaFree(h->cpad); cudaFree(h->gpad);
-    cudaFree(h->G); cudaFree(h->Qm); cudaFree(h->nonfinite); cudaFree(h->F64); cudaFree(h->FB); cudaFree(h->mode_org); cudaFree(h->FM); cudaFree(h->order); cudaFree(h->slots); cudaFree(h->partials); cudaFree(h->loss_dev); cudaFree(h->red);
+    cudaFree(h->G); cudaFree(h->mode_mem); cudaFree(h->slots); cudaFree(h->partials); cudaFree(h->loss_dev); cudaFree(h->red);
     cudaFree(h->hc); cudaFree(h->hI); cudaFree(h->hW); cudaFree(h->hg);
     for (cudaEvent_t e : h->chunk_ready) cudaEventDestroy(e);
     if (h->copy_stream) cudaStreamDestroy(h->copy_stream);
@@ -849,7 +849,11 @@ tt_status tt_create(const tt_problem *P, tt_precision prec, void *stream, tt_han
         cudaError_t _e = cudaMalloc((void **)&(ptr), (bytes));                \
         if (_e != cudaSuccess) { free_handle(h); return cuda_fail(_e, "tt_create: cudaMalloc"); } \
     } while (0)
-    ALLOC(h->geo, sizeof(ProjGeom) * h->S);
+    // the projections' constants, and behind them what the basis is formed from:
+    // [nodes][weights][frames 9S][seg0][seg1]
+    const size_t geo_bytes = sizeof(ProjGeom) * h->S, stage_doubles = 2 * kQuadNodes + 9 * (size_t)h->S + 2 * h->C;
+    static_assert(sizeof(ProjGeom) % 8 == 0, "doubles follow");
+    ALLOC(h->geo, geo_bytes + sizeof(double) * stage_doubles);
     ALLOC(h->B64, sizeof(double) * h->S * h->C * h->K);
     ALLOC(h->Bp, es * h->S * h->CP * h->KP);
     {
@@ -866,16 +870,9 @@ tt_status tt_create(const tt_problem *P, tt_precision prec, void *stream, tt_han
     ALLOC(h->G, es * h->npix() * h->KP);
     plan_modes(h);
     if (h->R) {
-        ALLOC(h->Qm, sizeof(float) * h->CP * kModeQ);
-        ALLOC(h->nonfinite, sizeof(unsigned));
-        if (!h->q_identity) ALLOC(h->F64, sizeof(double) * h->S * h->R * h->K);
-        ALLOC(h->FB, sizeof(float) * mode_operand_floats(h));
-        ALLOC(h->mode_org, sizeof(ModeOrigin) * h->S);
         plan_mode_forward(h);
-        if (h->slot_floats) {
-            ALLOC(h->FM, sizeof(float) * 2 * h->S * modes_m(h->R) * h->KP);
-            ALLOC(h->order, sizeof(int) * h->S);
-        }
+        const cudaError_t em = alloc_modes(h);
+        if (em != cudaSuccess) { free_handle(h); return cuda_fail(em, "tt_create: cudaMalloc"); }
     }
     plan_forward(h);
     h->fwd_staged = false;   // the tap-pair march is the faster one on every measured workload
@@ -898,14 +895,14 @@ tt_status tt_create(const tt_problem *P, tt_precision prec, void *stream, tt_han
         }
         (void)cudaGetLastError();
     }
-    // basis matrix: stage [nodes][weights][frames 9S][seg0][seg1] and run the quadrature kernel
-    std::vector<double> stage(2 * kQuadNodes + 9 * h->S + 2 * h->C);
-    gauss_legendre(kQuadNodes, stage.data(), stage.data() + kQuadNodes);
-    for (int s = 0; s < h->S; ++s) basis_frame(h->frame, h->inner[s], h->outer[s], stage.data() + 2 * kQuadNodes + 9 * s);
-    std::memcpy(stage.data() + 2 * kQuadNodes + 9 * h->S, h->seg0.data(), sizeof(double) * h->C);
-    std::memcpy(stage.data() + 2 * kQuadNodes + 9 * h->S + h->C, h->seg1.data(), sizeof(double) * h->C);
-    double *dstage = nullptr;
-    ALLOC(dstage, sizeof(double) * stage.size());
+    std::vector<char> setup(geo_bytes + sizeof(double) * stage_doubles);
+    std::memcpy(setup.data(), h->geo_host.data(), geo_bytes);
+    double *stage = (double *)(setup.data() + geo_bytes);
+    gauss_legendre(kQuadNodes, stage, stage + kQuadNodes);
+    for (int s = 0; s < h->S; ++s) basis_frame(h->frame, h->inner[s], h->outer[s], stage + 2 * kQuadNodes + 9 * s);
+    std::memcpy(stage + 2 * kQuadNodes + 9 * h->S, h->seg0.data(), sizeof(double) * h->C);
+    std::memcpy(stage + 2 * kQuadNodes + 9 * h->S + h->C, h->seg1.data(), sizeof(double) * h->C);
+    const double *dstage = (const double *)(h->geo + h->S);
 #undef ALLOC
     // last, and optional: a handle whose slots find no memory marches the volume
     if (h->slot_floats &&
@@ -915,14 +912,11 @@ tt_status tt_create(const tt_problem *P, tt_precision prec, void *stream, tt_han
     }
     h->fwd_modes = h->slots != nullptr;
     h->n_fwd_ctas = h->fwd_modes ? mode_forward_ctas(h) : forward_ctas(h, h->fwd_staged);
-    cudaError_t e = cudaMemcpyAsync(dstage, stage.data(), sizeof(double) * stage.size(), cudaMemcpyHostToDevice, h->stream);
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(h->geo, h->geo_host.data(), sizeof(ProjGeom) * h->S, cudaMemcpyHostToDevice, h->stream);
+    cudaError_t e = cudaMemcpyAsync(h->geo, setup.data(), setup.size(), cudaMemcpyHostToDevice, h->stream);
     if (e == cudaSuccess) e = launch_basis(h, dstage, dstage + kQuadNodes);
     if (e == cudaSuccess) e = (prec != TT_F64) ? launch_cast_basis<float>(h) : launch_cast_basis<double>(h);
-    if (e == cudaSuccess) e = setup_modes(h, dstage + 2 * kQuadNodes);
+    if (e == cudaSuccess) e = setup_modes(h, dstage + 2 * kQuadNodes, stage, stage + kQuadNodes);
     if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
-    cudaFree(dstage);
     if (e != cudaSuccess) {
         free_handle(h);
         return cuda_fail(e, "tt_create: basis set-up");

@@ -274,6 +274,8 @@ struct tt_handle {
     // rows of 4 * R4 mode values, then (R1) one more per ray.
     int R = 0, R4 = 0, R1 = 0;
     bool q_identity = false;             // the modes are the segments (Q = 1)
+    void *mode_mem = nullptr;            // device: holds what follows, down to `order`
+    size_t mode_host_bytes = 0;          // of it, the part that the host fills
     float *Qm = nullptr;                 // device [CP][kModeQ], zero padded
     unsigned *nonfinite = nullptr;       // device: the last rows_id whose rows were not all finite
     unsigned rows_id = 0;                // number of the rows in G (a new one for each that are written)
@@ -288,6 +290,7 @@ struct tt_handle {
     // mapped volumes: chunk slots for either copy, zero border.
     void *FM = nullptr;
     int *order = nullptr;                // device [S]
+    std::vector<tt::ModeOrigin> org_host;
     std::vector<int> order_host;
     int order_begin[2] = {0, 0};
     float *slots = nullptr;
@@ -461,7 +464,7 @@ cudaError_t launch_adjoint(tt_handle *h, T *g, bool reduce_loss = false);
 // forward holds memory that is wanted gives its slots up and marches the volume.
 cudaError_t handle_malloc(tt_handle *h, void **p, size_t bytes);
 // Detector modes: set-up (F_s, Q and the operand; enqueued on the handle's
-// stream, nodes as for launch_basis), the adjoint and the back-contraction.
+// stream), the adjoint and the back-contraction.
 AdjConst adj_const(const ProjGeom &g);
 inline long long mode_operand_floats(const tt_handle *h)
 {
@@ -470,7 +473,10 @@ inline long long mode_operand_floats(const tt_handle *h)
 }
 // Sets R and the boxes of a handle that can work in detector modes, else R = 0.
 void plan_modes(tt_handle *h);
-cudaError_t setup_modes(tt_handle *h, const double *frames);
+// One allocation for what the modes keep beside the slots.
+cudaError_t alloc_modes(tt_handle *h);
+// frames: device; node, weight: the kQuadNodes of the segments' rule, host.
+cudaError_t setup_modes(tt_handle *h, const double *frames, const double *node, const double *weight);
 // The forward in modes (tt_modes_fwd.cu): ray tiles (loss partials), sizes
 // (slot_floats 0: the handle does not use it), set-up and launch.
 void plan_mode_forward(tt_handle *h);

@@ -78,13 +78,24 @@ void plan_modes(tt_handle *h)
     const int R = std::min(h->two_theta == 0.0 ? h->L + 1 : 2 * h->L + 1, h->C);
     if (R > kMaxModes) return;
     int bj = 1, bk = 4;
-    for (const ProjGeom &g : h->geo_host) {
-        const AdjConst c = adj_const(g);
+    std::vector<AdjConst> adj(h->S);
+    h->org_host.resize(h->S);
+    for (int s = 0; s < h->S; ++s) {
+        const ProjGeom &g = h->geo_host[s];
+        const AdjConst &c = adj[s] = adj_const(g);
         double jl, jh, kl, kh;
         block_range(c.jc, jl, jh);
         block_range(c.kc, kl, kh);
         const double wj = jh - jl + 2.0 * g.hj + 0.04, wk = kh - kl + 2.0 * g.hk + 0.04;
         if (!(wj < 200.0) || !(wk < 200.0)) return;
+        ModeOrigin &o = h->org_host[s];
+        for (int t = 0; t < 4; ++t) {
+            o.j[t] = c.jc[t];
+            o.k[t] = c.kc[t];
+        }
+        o.jlo = jl - g.hj - 0.02;
+        o.klo = kl - g.hk - 0.02;
+        o.outer_j = c.outer_j ? 1 : 0;
         // a column whose first ray is in the box is read to its end
         bj = std::max(bj, (int)std::ceil(wj) + 1 + (c.outer_j ? 0 : c.ni - 1));
         bk = std::max(bk, ((int)std::ceil(wk) + 1 + (c.outer_j ? c.ni - 1 : 0) + 3 + 3) / 4 * 4);
@@ -112,7 +123,7 @@ void plan_modes(tt_handle *h)
     }
     h->mode_params.assign((h->S + ModeParams::kMax - 1) / ModeParams::kMax, ModeParams());
     for (int s = 0; s < h->S; ++s) {
-        const AdjConst c = adj_const(h->geo_host[s]);
+        const AdjConst &c = adj[s];
         ModeProj &p = h->mode_params[s / ModeParams::kMax].p[s % ModeParams::kMax];
         for (int t = 0; t < 3; ++t) {
             p.o[t] = (float)c.oc[1 + t];
@@ -133,28 +144,33 @@ void plan_modes(tt_handle *h)
 
 // F[s][m][i]: Fourier coefficients of Y_i along the detector circle, mode m
 // (0: constant; 2t - 1, 2t: cos, sin of t * step times phi), by the 32-point
-// rule on the whole circle (exact: two modes of at most 8 each).
-__global__ void __launch_bounds__(32)
+// rule on the whole circle (exact: two modes of at most 8 each).  The 32 points'
+// cosines and sines serve every mode (FP64 is slow here: evaluated for each
+// term they were most of a handle's set-up, 160 us at l_max 4).
+constexpr int kMatrixThreads = 128;
+__global__ void __launch_bounds__(kMatrixThreads)
 k_mode_matrix(const double *__restrict__ frames, double cth, double sth, int L, int K, int R, int step,
               double *__restrict__ F)
 {
     extern __shared__ double ysh[];   // [32][K]
+    __shared__ double cs[32], sn[32];
     const int s = blockIdx.x, t = threadIdx.x;
-    const double *fr = frames + 9 * s;
-    double sp, cp;
-    sincospi(t / 16.0, &sp, &cp);
-    double q[3];
-    for (int r = 0; r < 3; ++r) q[r] = cth * (cp * fr[3 + r] + sp * fr[6 + r]) - sth * fr[r];
-    sh_even<double>(L, q[0], q[1], q[2], ysh + t * K, 1);
+    if (t < 32) {
+        const double *fr = frames + 9 * s;
+        double sp, cp;
+        sincospi(t / 16.0, &sp, &cp);
+        cs[t] = cp;
+        sn[t] = sp;
+        double q[3];
+        for (int r = 0; r < 3; ++r) q[r] = cth * (cp * fr[3 + r] + sp * fr[6 + r]) - sth * fr[r];
+        sh_even<double>(L, q[0], q[1], q[2], ysh + t * K, 1);
+    }
     __syncthreads();
-    for (int e = t; e < R * K; e += 32) {
+    for (int e = t; e < R * K; e += kMatrixThreads) {
         const int m = e / K, i = e - m * K, f = (m + 1) / 2 * step;
+        const double *wave = (m & 1) ? cs : sn;
         double acc = 0.0;
-        for (int n = 0; n < 32; ++n) {
-            double sn, cn;
-            sincospi(((n * f) & 31) / 16.0, &sn, &cn);
-            acc += ysh[n * K + i] * (m == 0 ? 1.0 : ((m & 1) ? cn : sn));
-        }
+        for (int n = 0; n < 32; ++n) acc = fma(ysh[n * K + i], m == 0 ? 1.0 : wave[(n * f) & 31], acc);
         F[((size_t)s * R + m) * K + i] = acc * (m == 0 ? 1.0 : 2.0) / 32.0;
     }
 }
@@ -192,16 +208,48 @@ __global__ void k_mode_operand(const double *__restrict__ F, const ProjGeom *__r
     }
 }
 
-cudaError_t setup_modes(tt_handle *h, const double *frames)
+// What the host fills comes first and travels in one copy: mode_org, Qm, order,
+// nonfinite (0: rows_id starts at 1); then FB, F64, FM.
+cudaError_t alloc_modes(tt_handle *h)
+{
+    size_t at = 0;
+    auto place = [&](size_t bytes) {
+        const size_t p = at;
+        at += (bytes + 255) / 256 * 256;
+        return p;
+    };
+    const size_t org = place(sizeof(ModeOrigin) * h->S), q = place(sizeof(float) * h->CP * kModeQ);
+    const size_t ord = place(sizeof(int) * h->S), flag = place(sizeof(unsigned)), host = at;
+    const size_t fb = place(sizeof(float) * mode_operand_floats(h));
+    const size_t f64 = place(h->q_identity ? 0 : sizeof(double) * h->S * h->R * h->K);
+    const size_t fm = place(h->slot_floats ? sizeof(float) * 2 * h->S * modes_m(h->R) * h->KP : 0);
+    const cudaError_t e = cudaMalloc(&h->mode_mem, at);
+    if (e != cudaSuccess) return e;
+    char *base = (char *)h->mode_mem;
+    h->mode_org = (ModeOrigin *)(base + org);
+    h->Qm = (float *)(base + q);
+    h->order = (int *)(base + ord);
+    h->nonfinite = (unsigned *)(base + flag);
+    h->FB = (float *)(base + fb);
+    h->F64 = (double *)(base + f64);
+    h->FM = base + fm;
+    h->mode_host_bytes = host;
+    return cudaSuccess;
+}
+
+cudaError_t setup_modes(tt_handle *h, const double *frames, const double *node, const double *weight)
 {
     if (!h->R) return cudaSuccess;
-    const int CP = h->CP, R = h->R, step = mode_step(h);
+    const int R = h->R, step = mode_step(h);
+    const char *base = (const char *)h->mode_mem;
+    std::vector<char> host(h->mode_host_bytes, 0);
+    std::memcpy(host.data() + ((char *)h->mode_org - base), h->org_host.data(), sizeof(ModeOrigin) * h->S);
+    if (h->slot_floats)
+        std::memcpy(host.data() + ((char *)h->order - base), h->order_host.data(), sizeof(int) * h->S);
     // Segment means of the modes by the nodes that B is formed with: B = Q F
     // holds for them at any segment width, beyond the few turns the rule is
     // exact on too.
-    double node[kQuadNodes], weight[kQuadNodes];
-    gauss_legendre(kQuadNodes, node, weight);
-    std::vector<float> Q((size_t)CP * kModeQ, 0.f);
+    float *Q = (float *)(host.data() + ((char *)h->Qm - base));
     for (int c = 0; c < h->C; ++c)
         for (int m = 0; m < R; ++m) {
             double v = 0.0;
@@ -219,36 +267,17 @@ cudaError_t setup_modes(tt_handle *h, const double *frames)
             }
             Q[(size_t)c * kModeQ + m] = (float)v;
         }
-    cudaError_t e = cudaMemsetAsync(h->nonfinite, 0, sizeof(unsigned), h->stream);   // (rows_id starts at 1)
-    if (e != cudaSuccess) return e;
-    e = cudaMemcpyAsync(h->Qm, Q.data(), Q.size() * sizeof(float), cudaMemcpyHostToDevice, h->stream);
+    cudaError_t e = cudaMemcpyAsync(h->mode_mem, host.data(), host.size(), cudaMemcpyHostToDevice, h->stream);
     if (e != cudaSuccess) return e;
     cudaEvent_t ev;
     prof_begin(h, TT_KSLOT_BASIS, &ev);
     const double *F = h->B64;
     if (!h->q_identity) {
         const double th = 0.5 * h->two_theta;
-        k_mode_matrix<<<h->S, 32, 32 * h->K * sizeof(double), h->stream>>>(frames, std::cos(th), std::sin(th), h->L,
-                                                                         h->K, R, step, h->F64);
+        k_mode_matrix<<<h->S, kMatrixThreads, 32 * h->K * sizeof(double), h->stream>>>(
+            frames, std::cos(th), std::sin(th), h->L, h->K, R, step, h->F64);
         F = h->F64;
     }
-    std::vector<ModeOrigin> org(h->S);
-    for (int s = 0; s < h->S; ++s) {
-        const ProjGeom &g = h->geo_host[s];
-        const AdjConst c = adj_const(g);
-        double jl, jh, kl, kh;
-        block_range(c.jc, jl, jh);
-        block_range(c.kc, kl, kh);
-        for (int t = 0; t < 4; ++t) {
-            org[s].j[t] = c.jc[t];
-            org[s].k[t] = c.kc[t];
-        }
-        org[s].jlo = jl - g.hj - 0.02;
-        org[s].klo = kl - g.hk - 0.02;
-        org[s].outer_j = c.outer_j ? 1 : 0;
-    }
-    e = cudaMemcpyAsync(h->mode_org, org.data(), org.size() * sizeof(ModeOrigin), cudaMemcpyHostToDevice, h->stream);
-    if (e != cudaSuccess) return e;
     const int M = modes_m(R), UP = modes_up(M), N = modes_n(h->K);
     const long long n = mode_operand_floats(h);
     k_mode_operand<<<(unsigned)std::min<long long>((n + 255) / 256, 8LL * h->n_sm), 256, 0, h->stream>>>(
