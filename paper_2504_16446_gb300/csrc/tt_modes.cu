@@ -55,28 +55,54 @@ static size_t modes_smem(const tt_handle *h)
     return std::max(ring, (size_t)kModeVox * h->K * 4) + 128;   // (the sums at the end)
 }
 
+// Whether the adjoint in modes is the faster one.  It has a start and an end (box
+// origins, tensor memory, sums: 4 us a block at l_max 2, more above) that few
+// projections do not pay for, and its blocks come in waves of those resident;
+// the channel kernel's blocks are 32 voxels long in z at l_max 2.  Measured,
+// channels / modes in us, an adjoint by itself:
+//   l_max 8, 4 projections: 64^3 60.0 / 61.9, 100^3 190 / 197; 8: 99 / 81, 334 / 261
+//   l_max 6, 8: 64^3 64.6 / 68.4, 100^3 208 / 220; 12: 84.5 / 78.6, 275 / 257; 1
+//     projection 56.6 / 127 at 100^3
+//   l_max 4, 4: 64^3 25.1 / 27.3, 100^3 64 / 78; 8: 39.9 / 35.5, 118 / 112
+//   fewer blocks than SMs (16^3, 28^3), l_max 4 to 8, 12: 19.0 / 19.1, 26.2 / 27.2,
+//     21.1 / 25.1; 16: 23.0 / 21.1, 31.0 / 31.2, 28.5 / 28.7
+//   l_max 2, less than a wave, 12: 16^3 15.7 / 17.0, 40^3 21.0 / 21.1; 20: 40^3 27.2 /
+//     25.1; more: 56^3 28 projections 56.1 / 60.1, 36 67.9 / 66.3; 78 x 66 x 83 36 129.7
+//     / 131.8, 44 157.9 / 156.6; 128^3 28 406.7 / 408.4, 44 603 / 593; z padded by 28%:
+//     100^3 12 119 / 116, 20 182 / 166 (but 52^3, little more than a wave, 24: 45 / 51)
+//   l_max 2, five modes (two_theta): 64^3 60 121 / 130, 200 378 / 391; 128^3 120 1586 /
+//     1680; 48^3 60 75 / 65; 100^3 40 345 / 328
+//   l_max 4, nine modes: 24^3 60 58 / 31, 40^3 60 72 / 68, 48^3 60 94 / 99, 64^3 24 86 / 93,
+//     100^3 120 1376 / 1384, 128^3 120 2736 / 2628
+static bool modes_pay(const tt_handle *h, int R)
+{
+    const long long blocks = mode_blocks(h), wave = (long long)h->n_sm * mode_ctas(16);
+    const bool z_padded = 5LL * ((h->N[2] + 31) / 32 * 32) > 6LL * h->N[2];
+    if (h->L == 2) {
+        if (blocks <= wave) return h->S >= 18;
+        if (z_padded && blocks > 2 * wave) return h->S >= (R > 4 ? 40 : 16);
+        return R <= 4 && h->S >= 40;
+    }
+    if (h->L == 4 && R > 8 && 2 * blocks > wave) return false;
+    return h->S >= (blocks <= h->n_sm ? 14 : h->L == 4 ? 8 : h->L == 6 ? 9 : 5);
+}
+
 // The handle works in modes when there are at most kMaxModes of them, the band
-// limit is 2 .. 8, and every projection's box -- the rays of a block lie
+// limit is 2 .. 8, they pay, and every projection's box -- the rays of a block lie
 // within (hj, hk) of its voxels' centres, plus the rounding margin and up to
 // three pixels from aligning the box to four -- fits the tensor copies (256
 // floats wide) and, kModeStages deep, the shared memory of two CTAs per SM.
 // (Pixels much finer than voxels put too many rays around a block; the
 // channel kernels take those.)  Coordinates stay below 2^22 in magnitude for
 // volumes and detectors of at most 2^14, which the rounding by kRound needs.
-// At l_max 2 a row is 3 values for 6, and a block's start and end (some 4 us)
-// cost what few projections save: below 32 of them, on volumes of more than a
-// wave of blocks, the channel kernel stays (78 x 66 x 83 voxels, 55 x 70
-// pixels: 104 against 108 us at 28 projections, 384 against 360 at 112; 128^3,
-// 28: 402 against 405; 40^3, less than a wave: 31.6 against 28.2).
 void plan_modes(tt_handle *h)
 {
     h->R = 0;
     if (h->prec == TT_F64 || h->L < 2 || h->L > 8 || !driver_tensor_map_encoder()) return;
     const int limit = 1 << 14;
     if (h->N[0] > limit || h->N[1] > limit || h->N[2] > limit || h->nj > limit || h->nk > limit) return;
-    if (h->L == 2 && h->S < 32 && mode_blocks(h) > (long long)h->n_sm * mode_ctas(16)) return;
     const int R = std::min(h->two_theta == 0.0 ? h->L + 1 : 2 * h->L + 1, h->C);
-    if (R > kMaxModes) return;
+    if (R > kMaxModes || !modes_pay(h, R)) return;
     int bj = 1, bk = 4;
     std::vector<AdjConst> adj(h->S);
     h->org_host.resize(h->S);
