@@ -284,6 +284,7 @@ struct tt_handle {
     tt::ModeOrigin *mode_org = nullptr;  // device [S]
     int box_j = 0, box_k = 0;            // the adjoint's detector box (pixels)
     int nk1 = 0;                         // row pitch of the single values' plane (R1)
+    tt::TmaDesc rows_map, single_map;    // maps of the rows in G, of their single values
     std::vector<tt::ModeParams> mode_params;   // one block per launch
     // Mode forward (tt_modes_fwd.cu): F rows for the map, the projections
     // reading copy 0, then copy 1 of the packed volume, and the slots of

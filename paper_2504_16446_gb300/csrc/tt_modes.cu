@@ -263,9 +263,8 @@ cudaError_t alloc_modes(tt_handle *h)
     return cudaSuccess;
 }
 
-cudaError_t setup_modes(tt_handle *h, const double *frames, const double *node, const double *weight)
+static cudaError_t form_modes(tt_handle *h, const double *frames, const double *node, const double *weight)
 {
-    if (!h->R) return cudaSuccess;
     const int R = h->R, step = mode_step(h);
     const char *base = (const char *)h->mode_mem;
     std::vector<char> host(h->mode_host_bytes, 0);
@@ -338,13 +337,12 @@ static cudaError_t adjoint_modes_run(tt_handle *h, const float *rows, float *g, 
 {
     constexpr int M = 4 * R4 + R1, UP = modes_up(M), KU = modes_ku(M);
     const int tx = (h->N[0] + 7) / 8, ty = (h->N[1] + 3) / 4, tz = (h->N[2] + 7) / 8;
-    TmaDesc tm4, tm1;
-    if (!encode_rows(h, rows, 4 * R4, h->nk, &tm4)) return cudaErrorInvalidValue;
-    if (!R1) tm1 = tm4;
-    else if (!encode_rows(h, mode_out(h).G1, 1, h->nk1, &tm1)) return cudaErrorInvalidValue;
+    TmaDesc tm4 = h->rows_map;
+    const TmaDesc &tm1 = R1 ? h->single_map : h->rows_map;
+    if (rows != (const float *)h->G && !encode_rows(h, rows, 4 * R4, h->nk, &tm4)) return cudaErrorInvalidValue;
     const auto kern = k_adjoint_modes<N, R4, R1>;
     const size_t smem = modes_smem(h);
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = cudaSuccess;
     const int nchunk = (int)h->mode_params.size();
     for (int ci = 0; ci < nchunk && e == cudaSuccess; ++ci) {
         const int s0 = ci * ModeParams::kMax, ns = std::min(ModeParams::kMax, h->S - s0);
@@ -377,21 +375,44 @@ static cudaError_t adjoint_modes_run(tt_handle *h, const float *rows, float *g, 
     return e;
 }
 
-template <int N>
-static cudaError_t adjoint_modes_n(tt_handle *h, const float *rows, float *g, bool rl, const float *data)
+// f<N, R4, R1>() of the handle's layout.
+template <typename F>
+static cudaError_t with_layout(const tt_handle *h, F f)
 {
-    if (h->R4 == 1) return h->R1 ? adjoint_modes_run<N, 1, 1>(h, rows, g, rl, data) : adjoint_modes_run<N, 1, 0>(h, rows, g, rl, data);
-    return h->R1 ? adjoint_modes_run<N, 2, 1>(h, rows, g, rl, data) : adjoint_modes_run<N, 2, 0>(h, rows, g, rl, data);
+    auto rows = [&]<int N>() {
+        if (h->R4 == 1) return h->R1 ? f.template operator()<N, 1, 1>() : f.template operator()<N, 1, 0>();
+        return h->R1 ? f.template operator()<N, 2, 1>() : f.template operator()<N, 2, 0>();
+    };
+    switch (modes_n(h->K)) {
+    case 16: return rows.template operator()<16>();
+    case 32: return rows.template operator()<32>();
+    case 48: return rows.template operator()<48>();
+    default: return cudaErrorInvalidValue;
+    }
 }
 
 cudaError_t launch_adjoint_modes(tt_handle *h, const float *rows, float *g, bool reduce_loss, const float *data)
 {
-    switch (modes_n(h->K)) {
-    case 16: return adjoint_modes_n<16>(h, rows, g, reduce_loss, data);
-    case 32: return adjoint_modes_n<32>(h, rows, g, reduce_loss, data);
-    case 48: return adjoint_modes_n<48>(h, rows, g, reduce_loss, data);
-    default: return cudaErrorInvalidValue;
-    }
+    return with_layout(h, [&]<int N, int R4, int R1>() { return adjoint_modes_run<N, R4, R1>(h, rows, g, reduce_loss, data); });
+}
+
+// What a launch of the adjoint needs of the driver, once per handle: the maps of
+// the handle's own rows, and leave for the kernel's shared memory (the most that
+// any handle takes, so that handles do not narrow it for each other).
+static cudaError_t ready_adjoint(tt_handle *h)
+{
+    if (!encode_rows(h, h->G, 4 * h->R4, h->nk, &h->rows_map)) return cudaErrorInvalidValue;
+    if (h->R1 && !encode_rows(h, mode_out(h).G1, 1, h->nk1, &h->single_map)) return cudaErrorInvalidValue;
+    return with_layout(h, [&]<int N, int R4, int R1>() {
+        return cudaFuncSetAttribute(k_adjoint_modes<N, R4, R1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kModeMaxSmem);
+    });
+}
+
+cudaError_t setup_modes(tt_handle *h, const double *frames, const double *node, const double *weight)
+{
+    if (!h->R) return cudaSuccess;
+    const cudaError_t e = ready_adjoint(h);
+    return e == cudaSuccess ? form_modes(h, frames, node, weight) : e;
 }
 
 // Rows that are their caller's own (the modes are the segments): are they finite?
