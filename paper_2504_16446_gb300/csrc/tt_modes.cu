@@ -64,8 +64,8 @@ static size_t modes_smem(const tt_handle *h)
 //   l_max 6, 8: 64^3 64.6 / 68.4, 100^3 208 / 220; 12: 84.5 / 78.6, 275 / 257; 1
 //     projection 56.6 / 127 at 100^3
 //   l_max 4, 4: 64^3 25.1 / 27.3, 100^3 64 / 78; 8: 39.9 / 35.5, 118 / 112
-//   fewer blocks than SMs (16^3, 28^3), l_max 4 to 8, 12: 19.0 / 19.1, 26.2 / 27.2,
-//     21.1 / 25.1; 16: 23.0 / 21.1, 31.0 / 31.2, 28.5 / 28.7
+//   fewer blocks than SMs, whole evaluations, 18: 16^3 l_max 4 35.0 / 34.3, 6 36.1 /
+//     37.1, 8 41.7 / 43.5; 30: 45.6 / 33.9, 47.4 / 34.0, 53.7 / 39.4
 //   l_max 2, less than a wave, 12: 16^3 15.7 / 17.0, 40^3 21.0 / 21.1; 20: 40^3 27.2 /
 //     25.1; more: 56^3 28 projections 56.1 / 60.1, 36 67.9 / 66.3; 78 x 66 x 83 36 129.7
 //     / 131.8, 44 157.9 / 156.6; 128^3 28 406.7 / 408.4, 44 603 / 593; z padded by 28%:
@@ -84,7 +84,8 @@ static bool modes_pay(const tt_handle *h, int R)
         return R <= 4 && h->S >= 40;
     }
     if (h->L == 4 && R > 8 && 2 * blocks > wave) return false;
-    return h->S >= (blocks <= h->n_sm ? 14 : h->L == 4 ? 8 : h->L == 6 ? 9 : 5);
+    if (blocks <= h->n_sm) return h->S >= (h->L == 4 ? 18 : 20);
+    return h->S >= (h->L == 4 ? 8 : h->L == 6 ? 9 : 5);
 }
 
 // The handle works in modes when there are at most kMaxModes of them, the band

@@ -16,8 +16,8 @@ CASES = [  # volume, l_max, segments, projections, modes?
     ((56, 60, 64), 4, 9, 7, False), ((56, 60, 64), 4, 9, 8, True),
     ((56, 60, 64), 6, 16, 8, False), ((56, 60, 64), 6, 16, 9, True),
     ((56, 60, 64), 8, 16, 4, False), ((56, 60, 64), 8, 16, 5, True), ((56, 60, 64), 8, 16, 1, False),
-    ((20, 22, 21), 6, 16, 13, False), ((20, 22, 21), 6, 16, 14, True),
-    ((9, 8, 10), 8, 16, 1, False), ((9, 8, 10), 8, 16, 14, True),
+    ((20, 22, 21), 6, 16, 19, False), ((20, 22, 21), 6, 16, 20, True),
+    ((9, 8, 10), 8, 16, 1, False), ((9, 8, 10), 8, 16, 20, True),
 ]
 
 

@@ -24,9 +24,9 @@ def same(a, b):
 
 # rays through a few voxels only; more than one launch of the adjoint; the caller's rows read in place (eight
 # segments at l_max 8); the forward in modes (the last two; the first of them with rays through voxel centres)
-CASES = [dict(n=(11, 12, 13), nj=14, nk=13, ell_max=4, n_proj=16, n_seg=8, seed=32),
+CASES = [dict(n=(11, 12, 13), nj=14, nk=13, ell_max=4, n_proj=20, n_seg=8, seed=32),
          dict(n=(6, 5, 7), nj=7, nk=6, ell_max=2, n_proj=300, n_seg=5, seed=33),
-         dict(n=(11, 12, 13), nj=14, nk=13, ell_max=8, n_proj=16, n_seg=8, seed=34),
+         dict(n=(11, 12, 13), nj=14, nk=13, ell_max=8, n_proj=20, n_seg=8, seed=34),
          dict(n=(41, 30, 53), nj=30, nk=41, ell_max=8, n_proj=50, n_seg=16, seed=24, offsets=False),
          dict(n=(41, 30, 53), nj=31, nk=42, ell_max=6, n_proj=50, n_seg=8, seed=25)]
 

@@ -21,7 +21,7 @@ def rel(a, b):
 
 
 # the last size is one whose forward goes through modes
-@pytest.mark.parametrize("ell,n_seg,n,n_proj", [(2, 4, (12, 11, 13), 19), (4, 6, (12, 11, 13), 15), (8, 10, (12, 11, 13), 16),
+@pytest.mark.parametrize("ell,n_seg,n,n_proj", [(2, 4, (12, 11, 13), 19), (4, 6, (12, 11, 13), 19), (8, 10, (12, 11, 13), 21),
                                                 (8, 10, (41, 40, 44), 48)])
 @pytest.mark.parametrize("turns", [0.5, 1.0, 2.0, 3.0, 5.0])
 def test_wide_segments(ell, n_seg, n, n_proj, turns):
