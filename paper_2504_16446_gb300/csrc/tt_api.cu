@@ -840,6 +840,7 @@ tt_status tt_create(const tt_problem *P, tt_precision prec, void *stream, tt_han
         h->geo_host[s] = make_geom(h, s);
         h->xcopy = h->xcopy || h->geo_host[s].copy == 1;
     }
+    h->wide_detector = shadow_share(h) < 0.45;
     if (prec != TT_F64) build_adj_params<float>(h, h->adj_f32);
     else build_adj_params<double>(h, h->adj_f64);
 

@@ -299,6 +299,7 @@ struct tt_handle {
     long long slots1 = 0;                // where copy 1's slots start
     int chunk = 0;                       // slots, the projections of a chunk
     bool fwd_modes = false;              // the forward maps and marches modes
+    bool wide_detector = false;          // the volume's shadow covers less than 45% of the detector
     double *partials = nullptr;          // device, per-CTA loss partials
     long long n_partials = 0;            // allocated entries
     long long n_fwd_ctas = 0;            // entries the forward kernel writes
@@ -481,6 +482,8 @@ cudaError_t setup_modes(tt_handle *h, const double *frames, const double *node, 
 // The forward in modes (tt_modes_fwd.cu): ray tiles (loss partials), sizes
 // (slot_floats 0: the handle does not use it), set-up and launch.
 void plan_mode_forward(tt_handle *h);
+// Share of the detectors' pixels that the volume's shadow covers.
+double shadow_share(const tt_handle *h);
 long long mode_forward_ctas(const tt_handle *h);
 cudaError_t setup_mode_forward(tt_handle *h, const double *F);
 template <typename S>

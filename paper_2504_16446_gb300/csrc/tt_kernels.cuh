@@ -493,26 +493,41 @@ __device__ __forceinline__ T forward_epilogue(const T (&acc)[CPL], int q, int ch
 // the lane's channels, a butterfly across the lane group, then each lane
 // back-contracts into its own channels.
 // Resident CTAs asked of the compiler (0: none).  What it trades is registers,
-// hence planes in flight, against CTAs; measured in whole calls (us), project /
-// evaluation:
-//   FP32, 16 channels: five when the long gradient epilogue follows, four else
-//     (64^3: project 307 / 328 with four / five, evaluation 578 / 575; 128^3,
-//     l_max 4: 4780 / 5206, 8380 / 7896)
-//   2-byte, 16 channels: 64^3 project 286 / 275 with none / four, 128^3
-//     evaluation 7229 / 7258
-//   2-byte, 8 channels (56^3, 240 projections): 200 / 562 with none, 192 / 562
-//     with four; wider rows (28^3, l_max 6): 41.6 / 104.4 none, 37.0 / 101.5 three
-//   FP32, 8 channels (56^3, 240 projections): 281 / 626 with none, 243 / 606 with
-//     one; wider rows (20^3, l_max 8): 46.9 / 112.5, 37.3 / 102.2
-__host__ __device__ constexpr int fwd_ctas(int KP, int bytes, int mode)
+// hence planes in flight, against CTAs.  wide: detectors that the volume's shadow
+// covers less than 45% of, where most tiles march little and more CTAs pay.
+// Measured in us, a projection unless said, `n x d`: n^3 voxels, d^2 pixels:
+//   FP32, 8 channels (56 x 56, 240 projections): 281 with none, 243 with one
+//   FP32, 16: four, five when the long gradient epilogue follows (64 x 64: 307 / 328
+//     with four / five, evaluation 578 / 575; 128 x 128: 4780 / 5206, 8380 / 7896)
+//   FP32, 32, one / three: 64 x 64 306 / 313, 64 x 20 96 / 114, 32 x 48 70 / 71; wide: 32
+//     x 96 105 / 95, loss 151 / 140, 48 x 144 249 / 229
+//   FP32, 48 (90 x 90): 1764 with none, 1394 with one or two, 1356 with three, which
+//     loses at 40 x 40 (138 / 143) and 64 x 20 (116 / 139)
+//   FP32, 80: none / one / two 1466 / 998 / 870 (64 x 64), 646 / 593 / 462 (32 x 96); 96:
+//     347 / 286 / 301 (64 x 20), 703 / 811 / 667 (32 x 96)
+//   2 bytes, 4 and 8: four (64 x 64 86.9 with none, 80.7)
+//   2 bytes, 16: four (128 x 128 649 / 612 with five / four), five if wide (32 x 96
+//     152.6 with none, 156.9, 153.8); the epilogue none
+//   2 bytes, 32: three / four 180 / 167 (32 x 96), 212 / 219 (64 x 64), with the epilogue
+//     792 / 718 (90 x 90); 48: 349 / 356, 53 / 57 (28 x 28)
+//   2 bytes, 80: none / two / three 813 / 669 / 647, with the epilogue 1152 / 766 / 819;
+//     96: 1130 / 704 / 972, 56.1 / 44.3 / 64.1 (20 x 20)
+__host__ __device__ constexpr int fwd_ctas(int KP, int bytes, int mode, bool wide = false)
 {
+    const bool project = mode == kProject;
     if (bytes == 8) return 0;
-    if (bytes == 4) return KP == 16 ? (mode == kProject ? 4 : 5) : 1;
-    return KP == 16 ? (mode == kProject ? 4 : 0) : (KP <= 8 ? 4 : 3);
+    if (bytes == 4) {
+        if (KP == 16) return project ? 4 : 5;
+        if (KP == 32) return wide ? 3 : 1;
+        return KP == 80 || (KP == 96 && project && wide) ? 2 : 1;
+    }
+    if (KP == 16) return project ? (wide ? 5 : 4) : 0;
+    if (KP == 32) return project && !wide ? 3 : 4;
+    return KP <= 8 ? 4 : KP == 48 ? 3 : 2;
 }
 
-template <typename T, typename S, int KP, int LG, int MODE>
-__global__ void __launch_bounds__(kFwdThreads, fwd_ctas(KP, sizeof(S), MODE))
+template <typename T, typename S, int KP, int LG, int MODE, int CTAS = fwd_ctas(KP, sizeof(S), MODE)>
+__global__ void __launch_bounds__(kFwdThreads, CTAS)
 k_forward(const ProjGeom *__restrict__ geo, const S *__restrict__ cpad /* interior origin */,
           const S *__restrict__ cpadx /* interior origin of the x-innermost copy, or NULL */, const T *__restrict__ Bp,
           int nj, int nk, int C, int CP, int tiles_k, int slab_order, int s_base,
@@ -1318,15 +1333,19 @@ cudaError_t launch_forward_L(tt_handle *h, T *Iout, const T *I, const T *W, bool
                                                          slab, s0, Iout, nullptr, nullptr, nullptr, nullptr,
                                                          ModeOut{});
     };
+    auto run_mode = [&]<int MODE>() {
+        if (h->wide_detector) run(k_forward<T, S, KP, LG, MODE, fwd_ctas(KP, sizeof(S), MODE, true)>);
+        else run(k_forward<T, S, KP, LG, MODE>);
+    };
     if (!grad) {
-        run(k_forward<T, S, KP, LG, kProject>);
+        run_mode.template operator()<kProject>();
     } else {
         bool modes = false;
         if constexpr (std::is_same<T, float>::value && L >= 2 && L <= 8) {
             modes = h->R > 0;
-            if (modes) run(k_forward<T, S, KP, LG, kGradModes>);
+            if (modes) run_mode.template operator()<kGradModes>();
         }
-        if (!modes) run(k_forward<T, S, KP, LG, kGrad>);
+        if (!modes) run_mode.template operator()<kGrad>();
     }
     cudaError_t e = cudaGetLastError();
     prof_end(h, TT_KSLOT_FORWARD, ev);

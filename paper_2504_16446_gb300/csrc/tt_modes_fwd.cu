@@ -499,19 +499,30 @@ static std::vector<int> projection_order(tt_handle *h)
     return order;
 }
 
-// Steps of rays through the volume: planes times the detector pixels that the
-// volume's shadow covers (its bounding box), over all projections.
+// Detector pixels that the volume's shadow (its bounding box) covers.
+static double shadow(const tt_handle *h, const ProjGeom &g)
+{
+    auto covered = [&](double at0, double u, double v, double p, int n) {
+        double lo = at0, hi = at0;
+        for (const double d : {u * (g.Nu - 1), v * (g.Nv - 1), p * (g.Nm - 1)}) (d < 0 ? lo : hi) += d;
+        return std::max(0.0, std::min(n - 1.0, hi) - std::max(0.0, lo) + 1.0);
+    };
+    return covered(g.jc0, g.jU, g.jV, g.jP, h->nj) * covered(g.kc0, g.kU, g.kV, g.kP, h->nk);
+}
+
+double shadow_share(const tt_handle *h)
+{
+    double pixels = 0.0;
+    for (const ProjGeom &g : h->geo_host) pixels += shadow(h, g);
+    return pixels / (double)h->npix();
+}
+
+// Steps of rays through the volume: planes times covered pixels, over all
+// projections.
 static double ray_steps(const tt_handle *h)
 {
     double steps = 0.0;
-    for (const ProjGeom &g : h->geo_host) {
-        auto covered = [&](double at0, double u, double v, double p, int n) {
-            double lo = at0, hi = at0;
-            for (const double d : {u * (g.Nu - 1), v * (g.Nv - 1), p * (g.Nm - 1)}) (d < 0 ? lo : hi) += d;
-            return std::max(0.0, std::min(n - 1.0, hi) - std::max(0.0, lo) + 1.0);
-        };
-        steps += covered(g.jc0, g.jU, g.jV, g.jP, h->nj) * covered(g.kc0, g.kU, g.kV, g.kP, h->nk) * g.Nm;
-    }
+    for (const ProjGeom &g : h->geo_host) steps += shadow(h, g) * g.Nm;
     return steps;
 }
 
