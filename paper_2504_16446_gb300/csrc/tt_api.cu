@@ -657,6 +657,11 @@ tt_status tt_grad_enqueue(tt_handle *h, const T *c, const T *I, const T *W, T *g
         // kernel skips its march (every projection is exactly zero), so the
         // evaluation is the back-projection of the data alone
         if (c) TT_CUDA((launch_pack<T, S>(h, c)), "pack");
+        // the loss alone: the channels' epilogue is the shorter one (bf16, 32^3 on 96 x
+        // 96 pixels, l_max 2: 113 us for 124; 128^3, l_max 4: 693 for 719), but for wide
+        // rows on wide detectors (32^3 on 96 x 96, l_max 4: 196 for 187) and where the
+        // forward itself is in modes
+        const ChannelScope loss_only(h, g == nullptr && !h->fwd_modes && (h->L == 2 || !h->wide_detector));
         const ZeroVolume zero(h, c == nullptr);
         ++h->rows_id;
         TT_CUDA((launch_forward<T, S>(h, nullptr, I, W, true)), "forward");
