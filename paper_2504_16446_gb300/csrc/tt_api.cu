@@ -553,7 +553,7 @@ static void plan_forward(tt_handle *h)
         fits = fits && g.st_rv <= kStMaxRv && g.st_ru <= 256;
         cap = std::max(cap, (long long)((g.st_ru * g.st_rv + 1) & ~1));
     }
-    const long long bytes = (long long)kStRing * cap * 16 * 4 + (long long)h->CP * (16 + 16) * 4 + 128;
+    const long long bytes = (long long)kStRing * cap * 16 * 4 + (long long)h->CP * 16 * 4 + 128;
     if (!fits || bytes > kStMaxSmem) return;
     h->tmaps_host.resize(h->S);
     for (int s = 0; s < h->S; ++s)

@@ -539,10 +539,11 @@ int current_sm_count();
 // CTAs of the dot-product and regulariser reductions: four per SM.
 inline int dot_blocks(const tt_handle *h) { return 4 * h->n_sm; }
 // Dynamic shared memory of the staged forward: the stage ring, B_s and 128
-// bytes of slack to align the ring.
-inline size_t staged_forward_smem(const tt_handle *h)
+// bytes of slack to align the ring; the gradient in modes adds Q, 16 floats a
+// segment too (at most 4 KB, which the SM has beyond kStMaxSmem).
+inline size_t staged_forward_smem(const tt_handle *h, bool modes)
 {
-    return (size_t)kStRing * h->stage_cap * 16 * sizeof(float) + (size_t)h->CP * (16 + 16) * sizeof(float) + 128;   // (B_s and Q, 16 floats a segment each)
+    return (size_t)kStRing * h->stage_cap * 16 * sizeof(float) + (size_t)h->CP * (modes ? 32 : 16) * sizeof(float) + 128;
 }
 
 }  // namespace tt

@@ -1298,7 +1298,7 @@ cudaError_t launch_forward_L(tt_handle *h, T *Iout, const T *I, const T *W, bool
         if (h->fwd_staged && !h->zero_volume) {
             const int tiles_k = (h->nk + kStTK - 1) / kStTK, tiles_j = (h->nj + kStTJ - 1) / kStTJ;
             const dim3 grid = slab ? dim3(tiles_k * ns, tiles_j) : dim3(tiles_k * tiles_j, ns);
-            const size_t smem = staged_forward_smem(h);
+            const size_t smem = staged_forward_smem(h, grad && h->R);
             prof_begin(h, TT_KSLOT_FORWARD, &ev);
             if (grad) {
                 auto kern = h->R ? k_forward_staged<kGradModes> : k_forward_staged<kGrad>;
@@ -1321,9 +1321,9 @@ cudaError_t launch_forward_L(tt_handle *h, T *Iout, const T *I, const T *W, bool
     constexpr int TK = fwd_tk(LG), TJ = fwd_tj(LG);
     const int tiles_k = (h->nk + TK - 1) / TK, tiles_j = (h->nj + TJ - 1) / TJ;
     const dim3 grid = slab ? dim3(tiles_k * ns, tiles_j) : dim3(tiles_k * tiles_j, ns);
-    const size_t smem = (size_t)h->CP * (KP * sizeof(T) + LG * mode_lane(LG) * sizeof(float));
     prof_begin(h, TT_KSLOT_FORWARD, &ev);
-    auto run = [&](auto kern) {
+    auto run = [&](auto kern, int mode) {
+        const size_t smem = (size_t)h->CP * (KP * sizeof(T) + (mode == kGradModes ? LG * mode_lane(LG) * sizeof(float) : 0));
         if (smem > 48 * 1024) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (grad)
             kern<<<grid, kFwdThreads, smem, h->stream>>>(h->geo, cpad, cpadx, Bp, h->nj, h->nk, h->C, h->CP, tiles_k,
@@ -1334,8 +1334,8 @@ cudaError_t launch_forward_L(tt_handle *h, T *Iout, const T *I, const T *W, bool
                                                          ModeOut{});
     };
     auto run_mode = [&]<int MODE>() {
-        if (h->wide_detector) run(k_forward<T, S, KP, LG, MODE, fwd_ctas(KP, sizeof(S), MODE, true)>);
-        else run(k_forward<T, S, KP, LG, MODE>);
+        if (h->wide_detector) run(k_forward<T, S, KP, LG, MODE, fwd_ctas(KP, sizeof(S), MODE, true)>, MODE);
+        else run(k_forward<T, S, KP, LG, MODE>, MODE);
     };
     if (!grad) {
         run_mode.template operator()<kProject>();
