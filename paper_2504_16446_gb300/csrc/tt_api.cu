@@ -1057,7 +1057,12 @@ tt_status tt_gradient_residual_host(tt_handle *h, const float *c_host, const flo
     // its stores crossing the host link while the kernel runs; any other
     // g_host gets the gradient with one copy.
     float *g_map = (float *)mapped_device_pointer(g_host);
-    const int Q = std::min(8, h->S);
+    // Chunks: eight; in modes one per 120 projections, as every launch of the map
+    // reads the whole volume for its few.  Page-locked buffers, one / two / eight
+    // chunks, the direct march before in eight: 64^3, l_max 6, 24 projections 553 /
+    // 618 / 940, 759 us; 240 2226 / 2250 / 2578, 3475; 128^3, l_max 8, 60 6.23 / 6.32 /
+    // 7.79, 14.3 ms; 240 16.5 / 16.2 / 16.7, 34.6.
+    const int Q = std::min(h->fwd_modes ? std::max(1, std::min(8, h->S / 120)) : 8, h->S);
     if (!h->hc) TT_CUDA(handle_malloc(h, &h->hc, bc), "host-path cudaMalloc");
     if (!g_map && !h->hg) TT_CUDA(handle_malloc(h, &h->hg, bc), "host-path cudaMalloc");
     if (!h->hI) TT_CUDA(handle_malloc(h, &h->hI, bd), "host-path cudaMalloc");
