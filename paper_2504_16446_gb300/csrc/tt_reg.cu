@@ -54,8 +54,9 @@ struct RegSum {
 // value = sum c^2, grad = 2 c.  Grid-stride over quads (the entry points take
 // 16-byte aligned c and grad only), the last n % 4 elements by themselves;
 // per-block FP64 partials.  Bound by its reads and writes (100^3, 28 channels:
-// 86 -> 80 us in the whole call).
-template <typename T>
+// 86 -> 80 us in the whole call), in FP64 by its arithmetic, so the value alone
+// has a kernel without the gradient's products (100^3, 45 channels: 197 -> 107 us).
+template <typename T, bool GRAD>
 __global__ void k_l2(const T *__restrict__ c, long long n, T *__restrict__ grad, double *__restrict__ partials)
 {
     __shared__ double red[32];
@@ -69,14 +70,14 @@ __global__ void k_l2(const T *__restrict__ c, long long n, T *__restrict__ grad,
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
             sum.square(x[k]);
-            x[k] *= T(2);
+            if (GRAD) x[k] *= T(2);
         }
-        if (grad) reg_store(grad + 4 * q, x);
+        if (GRAD) reg_store(grad + 4 * q, x);
     }
     for (long long i = 4 * n4 + t0; i < n; i += stride) {
         const T x = c[i];
         sum.square(x);
-        if (grad) grad[i] = T(2) * x;
+        if (GRAD) grad[i] = T(2) * x;
     }
     const double v = sum.total(red);
     if (threadIdx.x == 0) partials[blockIdx.x] = v;
@@ -108,7 +109,7 @@ __device__ __forceinline__ void tv_point(T g0, T g1, T g2, T inv_delta, T delta,
 // 100^3, 28 channels: 460 -> 279 us in the whole call (c read and grad written
 // once: 33).
 constexpr int kTvRun = 10;
-template <typename T>
+template <typename T, bool GRAD>
 __global__ void __launch_bounds__(256)
 k_tv_huber(const T *__restrict__ c, int nx, int ny, int nz, int K, int run_len, T delta, T *__restrict__ grad,
            double *__restrict__ partials)
@@ -127,9 +128,9 @@ k_tv_huber(const T *__restrict__ c, int nx, int ny, int nz, int K, int run_len, 
         const bool y0 = y >= 1, y1 = y + 1 < ny, z0 = zk >= K, z1 = zk + K < row;
         const int x0 = run * run_len, x1 = min(nx, x0 + run_len);
         const T *p = c + x0 * plane + e;
-        T cc = __ldg(p), cy = y0 ? __ldg(p - row) : T(0), cz = z0 ? __ldg(p - K) : T(0);   // here, y - 1, z - 1
+        T cc = __ldg(p), cy = GRAD && y0 ? __ldg(p - row) : T(0), cz = GRAD && z0 ? __ldg(p - K) : T(0);   // here, y - 1, z - 1
         T back = T(0);                                     // w g_x of the plane behind
-        if (grad && x0 > 0) {
+        if (GRAD && x0 > 0) {
             const T *q = p - plane;
             const T b = __ldg(q);
             T w, H;
@@ -144,7 +145,7 @@ k_tv_huber(const T *__restrict__ c, int nx, int ny, int nz, int K, int run_len, 
             T w, H;
             tv_point<T>(gx, gy, gz, inv_delta, delta, w, H);
             sum.add(H);
-            if (grad) {
+            if (GRAD) {
                 T gr = -w * (gx + gy + gz) + back;
                 back = w * gx;
                 T wm, Hm;
@@ -200,24 +201,51 @@ static tt_status l2_impl(tt_handle *h, const T *c, T *grad, double *value_host)
     const unsigned blocks = reg_grid(h, n);
     cudaEvent_t ev;
     prof_begin(h, TT_KSLOT_VECTOR, &ev);
-    k_l2<T><<<blocks, 256, 0, h->stream>>>(c, n, grad, h->red);
+    (grad ? k_l2<T, true> : k_l2<T, false>)<<<blocks, 256, 0, h->stream>>>(c, n, grad, h->red);
     prof_end(h, TT_KSLOT_VECTOR, ev);
     return reg_finish<T>(h, blocks, value_host);
+}
+
+// Planes of a run.  Float: ten, fewer while the runs do not give every SM two
+// blocks (small volumes are bound by the planes a thread takes one after the
+// other).
+static int tv_run_f32(const tt_handle *h, long long segs)
+{
+    int run = kTvRun;
+    while (run > 1 && segs * ((h->N[0] + run - 1) / run) < 2 * h->n_sm) run = (run + 1) / 2;
+    return run;
+}
+// Double is bound by its arithmetic, so by the SM with the most of it: a run
+// takes 3 run + 1 weights with the gradient and run without (the same runs for
+// both, so that the value is the same), and the blocks, four per SM at most, go
+// round the SMs in turn.  55 x 65 x 55, 6 channels, the value alone: 105 us in tens,
+// 86 in threes; 27 x 22 x 25, 15 channels, with the gradient 83 in twos, 79 in threes.
+static int tv_run_f64(const tt_handle *h, long long segs)
+{
+    const long long grid = dot_blocks(h), sms = h->n_sm;
+    int best = 1;
+    long long least = -1;
+    for (int run = 1; run <= kTvRun; ++run) {
+        const long long items = segs * ((h->N[0] + run - 1) / run);
+        const long long most = items / grid * (grid / sms) + (items % grid + sms - 1) / sms;
+        if (least < 0 || most * (4 * run + 1) < least) {
+            least = most * (4 * run + 1);
+            best = run;
+        }
+    }
+    return best;
 }
 
 template <typename T>
 static tt_status tv_impl(tt_handle *h, const T *c, double delta, T *grad, double *value_host)
 {
     const long long plane = (long long)h->N[1] * h->N[2] * h->K;
-    // Shorter runs while the runs do not give every SM two blocks: small volumes
-    // are bound by the planes a thread takes one after the other.
     const long long segs = (plane + 255) / 256;
-    int run = kTvRun;
-    while (run > 1 && segs * ((h->N[0] + run - 1) / run) < 2 * h->n_sm) run = (run + 1) / 2;
+    const int run = std::is_same<T, double>::value ? tv_run_f64(h, segs) : tv_run_f32(h, segs);
     const unsigned blocks = reg_grid(h, segs * 256 * ((h->N[0] + run - 1) / run));
     cudaEvent_t ev;
     prof_begin(h, TT_KSLOT_VECTOR, &ev);
-    k_tv_huber<T><<<blocks, 256, 0, h->stream>>>(c, h->N[0], h->N[1], h->N[2], h->K, run, (T)delta, grad, h->red);
+    (grad ? k_tv_huber<T, true> : k_tv_huber<T, false>)<<<blocks, 256, 0, h->stream>>>(c, h->N[0], h->N[1], h->N[2], h->K, run, (T)delta, grad, h->red);
     prof_end(h, TT_KSLOT_VECTOR, ev);
     return reg_finish<T>(h, blocks, value_host);
 }
