@@ -315,15 +315,18 @@ static cudaError_t form_modes(tt_handle *h, const double *frames, const double *
 
 // CTAs that share a block of voxels (1, 2, 4 or 8, three units each at least):
 // the fewest waves of `slots` resident CTAs, a wave of s-fold split blocks
-// lasting 1/s, each doubling counted as 20% for its sums and ramps (measured 7%
-// at l_max 4, 12% at 8 on full chips, more where it starts another wave).  28^3, l_max 2, 60 projections (112 blocks): 46 -> 30
-// us with 4; 20^3, l_max 4: 60 -> 23; 55 x 65 x 55, l_max 4 (833 blocks on 608
-// slots): 482 -> 434 with 2; 64^3 (1024 on 608) stays whole: 280 / 295 / 312.
-static int mode_split(int blocks, int units, int slots)
+// lasting 1/s, each doubling counted as 20% for its sums and ramps; beyond a wave
+// as it is, only while each keeps 20 projections, which their ramps need.  Over
+// 156 sizes (12^3 to 72^3, l_max 2 to 8, 30 to 120 projections) the choice is
+// within 3% of the best of the four: 20^3, l_max 4, 60: 60 -> 23 us with 8; 28^3,
+// l_max 2, 60: 46 -> 30 with 4; 55 x 65 x 55, l_max 4, 247 (833 blocks on 608 slots):
+// 482 -> 434 with 2; 64^3, 120 (1024 on 608) stays whole: 280 / 295 / 312; 48^3, l_max
+// 8, 30 (432 on 304) too: 80 / 98 / 133.
+static int mode_split(int blocks, int units, int projections, int slots)
 {
     int best = 1;
     double least = 1e30, cost = 1.0;
-    for (int s = 1; s <= 8 && (s == 1 || units / s >= 3); s *= 2, cost *= 1.2) {
+    for (int s = 1; s <= 8 && (s == 1 || (units / s >= 3 && (blocks <= slots || projections / s >= 20))); s *= 2, cost *= 1.2) {
         const double t = cost * (((long long)blocks * s + slots - 1) / slots) / s;
         if (t < 0.999 * least) {
             least = t;
@@ -349,7 +352,7 @@ static cudaError_t adjoint_modes_run(tt_handle *h, const float *rows, float *g, 
         const int s0 = ci * ModeParams::kMax, ns = std::min(ModeParams::kMax, h->S - s0);
         const bool last = ci == nchunk - 1;
         static_assert(ModeParams::kMax % UP == 0, "launches start on a unit");
-        const int blocks = tx * ty * tz, split = mode_split(blocks, (ns + UP - 1) / UP, h->n_sm * mode_ctas(N));
+        const int blocks = tx * ty * tz, split = mode_split(blocks, (ns + UP - 1) / UP, ns, h->n_sm * mode_ctas(N));
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3((unsigned)blocks, (unsigned)split);
         cfg.blockDim = dim3(kModeThreads);
