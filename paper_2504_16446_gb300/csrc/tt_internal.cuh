@@ -209,7 +209,7 @@ struct ModeVolume {
 // The adjoint's enumeration constants of a projection in FP64 (see AdjProj).
 struct AdjConst {
     double oc[4], ic[4], bu[4], bv[4], jc[4], kc[4];
-    double uo, ui, vo, vi, ho, hi, au, lu, av, lv;
+    double uo, ui, vo, vi, ho, au, lu, av, lv;
     int no, ni;
     bool outer_j;
 };

@@ -94,17 +94,11 @@ __device__ __forceinline__ void mma_tf32_ts(uint32_t d_tmem, uint32_t a_tmem, ui
         : "memory");
 }
 
-// Stores of 2, 4, 8 or 16 consecutive columns of this warp's 32 lanes (shape
+// Stores of 2, 8 or 16 consecutive columns of this warp's 32 lanes (shape
 // 32x32b), and the wait for this thread's stores.
 __device__ __forceinline__ void tmem_st2(uint32_t taddr, const uint32_t *v)
 {
     asm volatile("tcgen05.st.sync.aligned.32x32b.x2.b32 [%0], {%1, %2};" ::"r"(taddr), "r"(v[0]), "r"(v[1]) : "memory");
-}
-__device__ __forceinline__ void tmem_st4(uint32_t taddr, const uint32_t *v)
-{
-    asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1, %2, %3, %4};" ::"r"(taddr), "r"(v[0]), "r"(v[1]),
-                 "r"(v[2]), "r"(v[3])
-                 : "memory");
 }
 __device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t *v)
 {
