@@ -1139,6 +1139,7 @@ __device__ __forceinline__ void adj_window_any(T (&acc)[V][CPL], const S *__rest
 
 // Four resident blocks (64 registers) pay off while a lane's accumulators are
 // 16 floats; larger K keeps three.
+//
 // Double precision on small volumes: gridDim.y CTAs of a cluster split the
 // projections of a block and add their sums through distributed shared memory
 // in a fixed order (16^3 x 30 projections: 32 blocks left most of the chip
@@ -1207,8 +1208,14 @@ k_adjoint(const __grid_constant__ AdjParams<T> P, int ns, const S *__restrict__ 
     // Warps whose voxels all lie outside the volume skip the loop as a whole.
     const bool group_live = (xw < nx) && (y < ny) && (bz * GZ < nz);
     if (group_live) {
-        const int s_end = ns * ((int)blockIdx.y + 1) / (int)gridDim.y;
-        for (int si = ns * (int)blockIdx.y / (int)gridDim.y; si < s_end; ++si) {
+        int s_begin = 0, s_end = ns;
+        // (float never splits; measured, the loop over all projections gains 1% up
+        // to 48 channels and loses 5% at 80)
+        if constexpr (std::is_same<T, double>::value || KP >= 80) {
+            s_begin = ns * (int)blockIdx.y / (int)gridDim.y;
+            s_end = ns * ((int)blockIdx.y + 1) / (int)gridDim.y;
+        }
+        for (int si = s_begin; si < s_end; ++si) {
             const AdjProj<T> &c = P.p[si];
             AdjVoxel<T> vx;
             vx.oc = c.oc[0] + c.oc[1] * fx + c.oc[2] * fy + c.oc[3] * fz;
@@ -1368,6 +1375,32 @@ cudaError_t launch_backcontract_L(tt_handle *h, const T *R)
     return e;
 }
 
+// CTAs that share a block's projections in double precision (1, 2, 4 or 8, two
+// projections each at least).  The arithmetic binds it, so the SM with the most
+// CTAs does: it has k = ceil(blocks s / SMs) of them, each ns / s projections and a
+// start and sums worth two to four more; while all are resident, the blocks that
+// the volume does not fill (`fill` of them is voxels) share SMs with full ones.
+// Measured (us): 16^3, l_max 2, 30 projections (16 blocks) 217 whole, 72 with 8;
+// 20^3, l_max 4, 30 (45) 181 with 2, 154 with 4; 24^3, 30 (54) 181 with 2, 198 with 4;
+// 28^3, l_max 2, 120 (112) 845 whole, 683 with 4 -- in two they only share SMs, with
+// 10 projections 89 whole, 103; 36^3, l_max 4, 120 (225) 2620 whole, 1997 with 4; 28^3,
+// l_max 4, 30 341 whole, 372 with 4.
+inline int adjoint_split(long long blocks, int ns, int n_sm, int KP, double fill)
+{
+    int split = 1;
+    double least = 1e30;
+    for (int s = 1; s <= 8 && (s == 1 || ns / s >= 2); s *= 2) {
+        const bool resident = blocks * s <= 2 * n_sm;
+        const double k = (double)((blocks * s + n_sm - 1) / n_sm), ends = KP <= 8 || (KP <= 16 && resident) ? 2.0 : 4.0;
+        const double t = (resident ? 1.0 + (k - 1.0) * fill : k) * ((double)ns / s + ends);
+        if (t < 0.95 * least) {
+            least = t;
+            split = s;
+        }
+    }
+    return split;
+}
+
 template <typename T, typename S, int KP, int LG, int V, int GZ>
 cudaError_t launch_adjoint_gz(tt_handle *h, T *g, bool reduce_loss)
 {
@@ -1381,9 +1414,8 @@ cudaError_t launch_adjoint_gz(tt_handle *h, T *g, bool reduce_loss)
         const int s0 = ci * AdjParams<T>::kMax;
         const int ns = std::min(AdjParams<T>::kMax, h->S - s0);
         const bool last = ci == nchunk - 1;
-        int split = 1;
-        if (std::is_same<T, double>::value)
-            while (split < 8 && 2LL * split * tx * ty * tz <= 2 * h->n_sm && ns / (2 * split) >= 2) split *= 2;
+        const int split = std::is_same<T, double>::value ? adjoint_split((long long)tx * ty * tz, ns, h->n_sm, KP,
+                                                                           (double)h->nvox() / ((double)tx * ty * tz * BXT * BY * GZ)) : 1;
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3((unsigned)(tx * ty * tz), (unsigned)split);
         cfg.blockDim = dim3(kThreads);
