@@ -185,7 +185,7 @@ def _kernel_source_hash():
     import re
     h = hashlib.sha256()
     csrc = os.path.join(ROOT, "paper_2504_16446_gb300", "csrc")
-    for f in ("tt_internal.cuh", "tt_kernels.cuh", "tt_modes.cuh", "tt_proj_f32.cu"):
+    for f in ("tt_internal.cuh", "tt_kernels.cuh", "tt_modes.cuh", "tt_modes.cu", "tt_proj_f32.cu"):
         with open(os.path.join(csrc, f)) as fh:
             code = re.sub(r"/\*.*?\*/", "", fh.read(), flags=re.S)
         code = re.sub(r"//[^\n]*", "", code)
