@@ -575,11 +575,13 @@ void plan_mode_forward(tt_handle *h)
     const long long slot = 4 * h->slot_floats, gb = 1LL << 30;
     const long long bytes = std::min(std::min(4 * gb, std::max(2 * gb, 24 * slot)), (long long)(free_bytes / 16));
     const int most = std::max(h->order_begin[1], h->S - h->order_begin[1]);
-    h->chunk = (int)std::min<long long>(most, bytes / slot);
-    if (h->chunk < std::min(most, 5)) {
+    const int fit = (int)std::min<long long>(most, bytes / slot);
+    if (fit < std::min(most, 5)) {
         h->slot_floats = 0;
         return;
     }
+    const int parts = (most + fit - 1) / fit;
+    h->chunk = (most + parts - 1) / parts;                 // (equal chunks need no more)
     // the copies' borders coincide in cubic volumes: one set of slots serves both
     h->slots1 = h->N[0] == h->N[2] || h->order_begin[1] == 0 || h->order_begin[1] == h->S ? 0 : h->chunk * h->slot_floats;
 }
