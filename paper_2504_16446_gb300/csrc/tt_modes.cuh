@@ -59,7 +59,7 @@ namespace tt {
 // of those bytes, 8 a sixth.  What bounds it now is instruction issue (70% of
 // the slots at l_max 4; the same gather from global memory, with its bounds
 // tests and 64-bit addresses, took 0.358) and, at l_max 8, the latency that
-// eight resident warps leave: 0.263 and 6.1 ms.
+// eight resident warps leave: 0.245 and 6.1 ms.
 
 // One G' row of the box.  Rows of two quads (R4 = 2) are 32 bytes apart, so
 // that lanes four rows apart read the same banks: lanes 4 .. 7 of every eight

@@ -80,3 +80,23 @@ def test_mitra_keeps_its_bits_with_float_storage(ell, n, n_proj):
             opt.step()
         out.append(opt.get())
     assert all(torch.equal(x, y) for x, y in zip(out[0][:3], out[1][:3]))
+
+
+@pytest.mark.parametrize("prec,unit", [("bf16", 2.0 ** -9), ("f16", 2.0 ** -12)])
+@pytest.mark.parametrize("ell", [2, 4, 6, 8])
+def test_lbfgs_stays_with_the_solve_in_64_bits(ell, prec, unit):
+    """Rounding the trial volume to `unit` puts at most that of the projections on the residual, so that of the gradient at
+    zero on the gradients (four times, for the line search's and the pairs' share), and as much of the iterate on it."""
+    st = synth.small_setup(n=(22, 19, 24), nj=21, nk=23, ell_max=ell, n_proj=30, n_seg=16, seed=ell)
+    h, ref = tt.Handle(st, prec), tt.Handle(st, "f64")
+    I = data(h, 6)
+    _, g0 = ref.gradient_residual(None, I.double())
+    out = []
+    for handle, d in ((h, I), (ref, I.double())):
+        opt = tt.LBFGS(handle, None, d, log=False)
+        for _ in range(3):
+            opt.step()
+        out.append(opt.get())
+    (x, g, loss), (x64, g64, loss64) = out
+    assert float((x.double() - x64).norm()) <= 4 * unit * float(x64.norm())
+    assert float((g.double() - g64).norm()) <= 4 * unit * float(g0.norm())
