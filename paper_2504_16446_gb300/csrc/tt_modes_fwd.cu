@@ -643,7 +643,10 @@ cudaError_t launch_forward_modes(tt_handle *h, float *Iout, const float *I, cons
         for (int i = 0; i < parts && e == cudaSuccess; ++i) {
             const int a = i0 + (int)((long long)(i1 - i0) * i / parts);
             const int n = i0 + (int)((long long)(i1 - i0) * (i + 1) / parts) - a;
-            e = h->KP == 32 ? run_m<S, 32>(h, a, n, c, Iout, I, W, grad) : run_m<S, 48>(h, a, n, c, Iout, I, W, grad);
+            if constexpr (sizeof(S) == 4)                  // (2-byte storage: l_max 8 only, see plan_mode_forward)
+                e = h->KP == 32 ? run_m<S, 32>(h, a, n, c, Iout, I, W, grad) : run_m<S, 48>(h, a, n, c, Iout, I, W, grad);
+            else
+                e = run_m<S, 48>(h, a, n, c, Iout, I, W, grad);
         }
     }
     return e;
