@@ -93,3 +93,24 @@ def test_a_solver_gets_the_slots_memory():
         del filler
         torch.cuda.empty_cache()
     assert float((got - want).norm()) <= 1e-6 * float(want.norm())
+
+
+def test_no_room_for_the_modes():
+    """60000 projections: the modes keep 0.75 GB, the rest of the handle takes 0.55.  Between the two the handle works in
+    channels, as one with more modes than the mode kernels take does (two_theta = 1e-200: the same basis)."""
+    st = [synth.small_setup(n=(4, 5, 6), nj=1, nk=2, ell_max=8, n_proj=60000, n_seg=16, seed=5, two_theta=t) for t in (0.0, 1e-200)]
+    channels = tt.Handle(st[1], "f32")
+    R = torch.randn(channels.data_shape, device="cuda", generator=torch.Generator(device="cuda").manual_seed(1))
+    want = channels.adjoint(R)
+    channels.close()
+    room = tt.Handle(st[0], "f32")
+    assert not torch.equal(room.adjoint(R), want)           # (in modes)
+    room.close()
+    filler = fill(950 * MB)
+    try:
+        h = tt.Handle(st[0], "f32")
+        assert torch.equal(h.adjoint(R), want)
+        h.close()
+    finally:
+        del filler
+        torch.cuda.empty_cache()
