@@ -422,8 +422,7 @@ tt_status validate(const tt_problem *P)
 static void free_handle(tt_handle *h)
 {
     if (!h) return;
-    cudaFree(h->geo); cudaFree(h->tmaps); cudaFree(h->B64); cudaFree(h->Bp); cudaFree(h->cpad); cudaFree(h->gpad);
-    cudaFree(h->G); cudaFree(h->mode_mem); cudaFree(h->slots); cudaFree(h->partials); cudaFree(h->loss_dev); cudaFree(h->red);
+    cudaFree(h->arena); cudaFree(h->tmaps); cudaFree(h->slots);
     cudaFree(h->hc); cudaFree(h->hI); cudaFree(h->hW); cudaFree(h->hg);
     for (cudaEvent_t e : h->chunk_ready) cudaEventDestroy(e);
     if (h->copy_stream) cudaStreamDestroy(h->copy_stream);
@@ -850,45 +849,50 @@ tt_status tt_create(const tt_problem *P, tt_precision prec, void *stream, tt_han
     else build_adj_params<double>(h, h->adj_f64);
 
     const size_t es = h->esize();
-#define ALLOC(ptr, bytes)                                                     \
-    do {                                                                      \
-        cudaError_t _e = cudaMalloc((void **)&(ptr), (bytes));                \
-        if (_e != cudaSuccess) { free_handle(h); return cuda_fail(_e, "tt_create: cudaMalloc"); } \
-    } while (0)
-    // the projections' constants, and behind them what the basis is formed from:
-    // [nodes][weights][frames 9S][seg0][seg1]
+    // One allocation for what the handle always has (each by itself costs 40 us once
+    // it is beyond the allocator's small pages).  geo: the projections' constants,
+    // and behind them what the basis is formed from: [nodes][weights][frames
+    // 9S][seg0][seg1].
     const size_t geo_bytes = sizeof(ProjGeom) * h->S, stage_doubles = 2 * kQuadNodes + 9 * (size_t)h->S + 2 * h->C;
     static_assert(sizeof(ProjGeom) % 8 == 0, "doubles follow");
-    ALLOC(h->geo, geo_bytes + sizeof(double) * stage_doubles);
-    ALLOC(h->B64, sizeof(double) * h->S * h->C * h->K);
-    ALLOC(h->Bp, es * h->S * h->CP * h->KP);
-    {
-        const long long padded = (long long)(h->N[0] + 4) * (h->N[1] + 4) * (h->N[2] + 4);
-        const long long copies = h->xcopy ? 2 : 1;
-        h->pad_vox = padded;
-        ALLOC(h->cpad, h->ssize() * copies * padded * h->KP);
-        h->cpad_origin = 2LL * (h->N[1] + 4) * (h->N[2] + 4) + 2LL * (h->N[2] + 4) + 2;
-        h->cpadx_origin = 2LL * (h->N[1] + 4) * (h->N[0] + 4) + 2LL * (h->N[0] + 4) + 2;
-        cudaError_t ez = cudaMemsetAsync(h->cpad, 0, h->ssize() * copies * padded * h->KP, h->stream);   // border stays zero
-        if (ez != cudaSuccess) { free_handle(h); return cuda_fail(ez, "tt_create: memset"); }
-    }
-    ALLOC(h->gpad, es * h->nvox() * h->KP);
-    ALLOC(h->G, es * h->npix() * h->KP);
+    h->pad_vox = (long long)(h->N[0] + 4) * (h->N[1] + 4) * (h->N[2] + 4);
+    h->cpad_origin = 2LL * (h->N[1] + 4) * (h->N[2] + 4) + 2LL * (h->N[2] + 4) + 2;
+    h->cpadx_origin = 2LL * (h->N[1] + 4) * (h->N[0] + 4) + 2LL * (h->N[0] + 4) + 2;
+    h->n_partials = std::max(std::max(forward_ctas(h, false), forward_ctas(h, true)), mode_forward_ctas(h));
+    const size_t cpad_bytes = h->ssize() * (h->xcopy ? 2 : 1) * h->pad_vox * h->KP;
+    const struct { void **p; size_t bytes; } parts[] = {
+        {(void **)&h->geo, geo_bytes + sizeof(double) * stage_doubles},
+        {(void **)&h->B64, sizeof(double) * h->S * h->C * h->K},
+        {(void **)&h->Bp, es * h->S * h->CP * h->KP},
+        {(void **)&h->cpad, cpad_bytes},
+        {(void **)&h->gpad, es * h->nvox() * h->KP},
+        {(void **)&h->G, es * h->npix() * h->KP},
+        {(void **)&h->partials, sizeof(double) * h->n_partials},
+        {(void **)&h->loss_dev, sizeof(double) * 4},
+        {(void **)&h->red, sizeof(double) * dot_blocks(h)},
+    };
+    size_t total = 0;
+    for (const auto &q : parts) total += (q.bytes + 1023) / 1024 * 1024;
     plan_modes(h);
-    if (h->R) {
-        plan_mode_forward(h);
-        if (alloc_modes(h) != cudaSuccess) {               // (thousands of projections: hundreds of MB)
-            (void)cudaGetLastError();
-            h->R = 0;                                      // a handle that has no room for them works in channels
-            h->slot_floats = 0;
-        }
+    if (h->R) plan_mode_forward(h, total);
+    cudaError_t ea = cudaMalloc(&h->arena, total + (h->R ? place_modes(h, nullptr) : 0));
+    if (ea != cudaSuccess && h->R) {                       // (thousands of projections: hundreds of MB for the modes)
+        (void)cudaGetLastError();
+        h->R = 0;                                          // a handle that has no room for them works in channels
+        h->slot_floats = 0;
+        ea = cudaMalloc(&h->arena, total);
     }
+    if (ea != cudaSuccess) { free_handle(h); return cuda_fail(ea, "tt_create: cudaMalloc"); }
+    char *at = (char *)h->arena;
+    for (const auto &q : parts) {
+        *q.p = at;
+        at += (q.bytes + 1023) / 1024 * 1024;
+    }
+    if (h->R) place_modes(h, at);
+    ea = cudaMemsetAsync(h->cpad, 0, cpad_bytes, h->stream);   // border stays zero
+    if (ea != cudaSuccess) { free_handle(h); return cuda_fail(ea, "tt_create: memset"); }
     plan_forward(h);
     h->fwd_staged = false;   // the tap-pair march is the faster one on every measured workload
-    h->n_partials = std::max(std::max(forward_ctas(h, false), forward_ctas(h, true)), mode_forward_ctas(h));
-    ALLOC(h->partials, sizeof(double) * h->n_partials);
-    ALLOC(h->loss_dev, sizeof(double) * 4);
-    ALLOC(h->red, sizeof(double) * dot_blocks(h));
     {
         cudaError_t e = cudaMallocHost((void **)&h->loss_pinned, sizeof(double) * 4);
         if (e != cudaSuccess) { free_handle(h); return cuda_fail(e, "tt_create: cudaMallocHost"); }
@@ -912,7 +916,6 @@ tt_status tt_create(const tt_problem *P, tt_precision prec, void *stream, tt_han
     std::memcpy(stage + 2 * kQuadNodes + 9 * h->S, h->seg0.data(), sizeof(double) * h->C);
     std::memcpy(stage + 2 * kQuadNodes + 9 * h->S + h->C, h->seg1.data(), sizeof(double) * h->C);
     const double *dstage = (const double *)(h->geo + h->S);
-#undef ALLOC
     // last, and optional: a handle whose slots find no memory marches the volume
     if (h->slot_floats &&
         cudaMalloc((void **)&h->slots, sizeof(float) * (h->chunk * h->slot_floats + h->slots1)) != cudaSuccess) {

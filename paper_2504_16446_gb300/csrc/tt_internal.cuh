@@ -268,13 +268,14 @@ struct tt_handle {
     bool xcopy = false;                  // the x-innermost copy exists
     long long pad_vox = 0;               // voxels of one padded copy
     long long cpadx_origin = 0;          // voxel offset of (0,0,0) in the x-innermost copy (from its start)
+    void *arena = nullptr;               // device: holds geo, B64, Bp, cpad, gpad, G, partials, loss_dev, red, mode_mem
     void *gpad = nullptr;                // device [nvox][KP]
     void *G = nullptr;                   // device [S][nj][nk][KP]
     // Detector modes (tt_modes.cuh; 0: the handle works in channels): G holds
     // rows of 4 * R4 mode values, then (R1) one more per ray.
     int R = 0, R4 = 0, R1 = 0;
     bool q_identity = false;             // the modes are the segments (Q = 1)
-    void *mode_mem = nullptr;            // device: holds what follows, down to `order`
+    void *mode_mem = nullptr;            // in the arena: holds what follows, down to `order`
     size_t mode_host_bytes = 0;          // of it, the part that the host fills
     float *Qm = nullptr;                 // device [CP][kModeQ], zero padded
     unsigned *nonfinite = nullptr;       // device: the last rows_id whose rows were not all finite
@@ -475,13 +476,14 @@ inline long long mode_operand_floats(const tt_handle *h)
 }
 // Sets R and the boxes of a handle that can work in detector modes, else R = 0.
 void plan_modes(tt_handle *h);
-// One allocation for what the modes keep beside the slots.
-cudaError_t alloc_modes(tt_handle *h);
+// Bytes of what the modes keep beside the slots; with base, where each part lies.
+size_t place_modes(tt_handle *h, char *base);
 // frames: device; node, weight: the kQuadNodes of the segments' rule, host.
 cudaError_t setup_modes(tt_handle *h, const double *frames, const double *node, const double *weight);
 // The forward in modes (tt_modes_fwd.cu): ray tiles (loss partials), sizes
-// (slot_floats 0: the handle does not use it), set-up and launch.
-void plan_mode_forward(tt_handle *h);
+// (slot_floats 0: the handle does not use it; `reserved`: bytes still to be
+// allocated), set-up and launch.
+void plan_mode_forward(tt_handle *h, size_t reserved);
 // Share of the detectors' pixels that the volume's shadow covers.
 double shadow_share(const tt_handle *h);
 long long mode_forward_ctas(const tt_handle *h);

@@ -237,7 +237,7 @@ __global__ void k_mode_operand(const double *__restrict__ F, const ProjGeom *__r
 
 // What the host fills comes first and travels in one copy: mode_org, Qm, order,
 // nonfinite (0: rows_id starts at 1); then FB, F64, FM.
-cudaError_t alloc_modes(tt_handle *h)
+size_t place_modes(tt_handle *h, char *base)
 {
     size_t at = 0;
     auto place = [&](size_t bytes) {
@@ -250,18 +250,18 @@ cudaError_t alloc_modes(tt_handle *h)
     const size_t fb = place(sizeof(float) * mode_operand_floats(h));
     const size_t f64 = place(h->q_identity ? 0 : sizeof(double) * h->S * h->R * h->K);
     const size_t fm = place(h->slot_floats ? sizeof(float) * 2 * h->S * modes_m(h->R) * h->KP : 0);
-    const cudaError_t e = cudaMalloc(&h->mode_mem, at);
-    if (e != cudaSuccess) return e;
-    char *base = (char *)h->mode_mem;
-    h->mode_org = (ModeOrigin *)(base + org);
-    h->Qm = (float *)(base + q);
-    h->order = (int *)(base + ord);
-    h->nonfinite = (unsigned *)(base + flag);
-    h->FB = (float *)(base + fb);
-    h->F64 = (double *)(base + f64);
-    h->FM = base + fm;
-    h->mode_host_bytes = host;
-    return cudaSuccess;
+    if (base) {
+        h->mode_mem = base;
+        h->mode_org = (ModeOrigin *)(base + org);
+        h->Qm = (float *)(base + q);
+        h->order = (int *)(base + ord);
+        h->nonfinite = (unsigned *)(base + flag);
+        h->FB = (float *)(base + fb);
+        h->F64 = (double *)(base + f64);
+        h->FM = base + fm;
+        h->mode_host_bytes = host;
+    }
+    return at;
 }
 
 static cudaError_t form_modes(tt_handle *h, const double *frames, const double *node, const double *weight)

@@ -545,7 +545,7 @@ static double ray_steps(const tt_handle *h)
 //   2 bytes  l_max 6: 64^3 549 / 402, 128^3 3655 / 2958: never; l_max 8: 28^3 x 160
 //            125 / 110, 40^3 201 / 185, 64^3 568 / 649, 128^3 3777 / 5130, on 64^2
 //            2522 / 1662; 32^3 on 96^2 179 / 241
-void plan_mode_forward(tt_handle *h)
+void plan_mode_forward(tt_handle *h, size_t reserved)
 {
     h->slot_floats = 0;
     const bool half = h->ssize() == 2;
@@ -572,6 +572,7 @@ void plan_mode_forward(tt_handle *h)
     // 21.6.
     size_t free_bytes = 0, total = 0;
     if (cudaMemGetInfo(&free_bytes, &total) != cudaSuccess) (void)cudaGetLastError();
+    free_bytes -= std::min(free_bytes, reserved);
     const long long slot = 4 * h->slot_floats, gb = 1LL << 30;
     const long long bytes = std::min(std::min(4 * gb, std::max(2 * gb, 24 * slot)), (long long)(free_bytes / 16));
     const int most = std::max(h->order_begin[1], h->S - h->order_begin[1]);
