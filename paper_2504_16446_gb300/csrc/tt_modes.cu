@@ -67,23 +67,30 @@ static size_t modes_smem(const tt_handle *h)
 //   fewer blocks than SMs, whole evaluations, 18: 16^3 l_max 4 35.0 / 34.3, 6 36.1 /
 //     37.1, 8 41.7 / 43.5; 30: 45.6 / 33.9, 47.4 / 34.0, 53.7 / 39.4
 //   l_max 2, less than a wave, 12: 16^3 15.7 / 17.0, 40^3 21.0 / 21.1; 20: 40^3 27.2 /
-//     25.1; more: 56^3 28 projections 56.1 / 60.1, 36 67.9 / 66.3; 78 x 66 x 83 36 129.7
-//     / 131.8, 44 157.9 / 156.6; 128^3 28 406.7 / 408.4, 44 603 / 593; z padded by 28%:
-//     100^3 12 119 / 116, 20 182 / 166 (but 52^3, little more than a wave, 24: 45 / 51)
+//     25.1, but evaluations, whose forward does more in modes, 48.3 / 49.0, 24 49.0 / 50.3,
+//     28 57.7 / 57.0, FP16 36 x 32 x 33 28 46.2 / 47.4, 32 51.1 / 50.1; more than a wave:
+//     56^3 28 56.1 / 60.1, 36 67.9 / 66.3; 78 x 66 x 83 36 129.7 / 131.8, 44 157.9 /
+//     156.6; 128^3 28 406.7 / 408.4, 44 603 / 593; z padded by 28%: 100^3 12 119 / 116, 20
+//     182 / 166 (but 52^3, little more than a wave, 24: 45 / 51); by 22%: 110 x 100 x 105,
+//     evaluations, 20 375 / 375, page-locked buffers 647 / 708
 //   l_max 2, five modes (two_theta): 64^3 60 121 / 130, 200 378 / 391; 128^3 120 1586 /
 //     1680; 48^3 60 75 / 65; 100^3 40 345 / 328
 //   l_max 4, nine modes: 24^3 60 58 / 31, 40^3 60 72 / 68, 48^3 60 94 / 99, 64^3 24 86 / 93,
 //     100^3 120 1376 / 1384, 128^3 120 2736 / 2628
+//   l_max 4, 2-byte storage, whose forward pays more for the modes' epilogue, whole
+//     evaluations: 30 x 28 x 31 18 44.6 / 46.0, 28 47.7 / 47.6, 35 56.9 / 52.2; 40 x 44 x 40
+//     18 58.1 / 60.2, 24 63.8 / 65.9, 28 69.9 / 67.9; 50 x 52 x 48 20 83.7 / 78.5
 static bool modes_pay(const tt_handle *h, int R)
 {
     const long long blocks = mode_blocks(h), wave = (long long)h->n_sm * mode_ctas(16);
-    const bool z_padded = 5LL * ((h->N[2] + 31) / 32 * 32) > 6LL * h->N[2];
+    const bool z_padded = 4LL * ((h->N[2] + 31) / 32 * 32) > 5LL * h->N[2];
     if (h->L == 2) {
-        if (blocks <= wave) return h->S >= 18;
+        if (blocks <= wave) return h->S >= 30;
         if (z_padded && blocks > 2 * wave) return h->S >= (R > 4 ? 40 : 16);
         return R <= 4 && h->S >= 40;
     }
     if (h->L == 4 && R > 8 && 2 * blocks > wave) return false;
+    if (h->L == 4 && h->ssize() == 2 && blocks <= 2 * h->n_sm) return h->S >= 28;
     if (blocks <= h->n_sm) return h->S >= (h->L == 4 ? 18 : 20);
     return h->S >= (h->L == 4 ? 8 : h->L == 6 ? 9 : 5);
 }
