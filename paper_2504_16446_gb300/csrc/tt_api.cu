@@ -1063,12 +1063,18 @@ tt_status tt_gradient_residual_host(tt_handle *h, const float *c_host, const flo
     // its stores crossing the host link while the kernel runs; any other
     // g_host gets the gradient with one copy.
     float *g_map = (float *)mapped_device_pointer(g_host);
-    // Chunks: eight; in modes one per 120 projections, as every launch of the map
-    // reads the whole volume for its few.  Page-locked buffers, one / two / eight
-    // chunks, the direct march before in eight: 64^3, l_max 6, 24 projections 553 /
-    // 618 / 940, 759 us; 240 2226 / 2250 / 2578, 3475; 128^3, l_max 8, 60 6.23 / 6.32 /
-    // 7.79, 14.3 ms; 240 16.5 / 16.2 / 16.7, 34.6.
-    const int Q = std::min(h->fwd_modes ? std::max(1, std::min(8, h->S / 120)) : 8, h->S);
+    // Chunks: at most eight.  In modes one per 120 projections, as every launch of the
+    // map reads the whole volume for its few: page-locked buffers, one / two / eight
+    // chunks, the direct march before in eight: 64^3, l_max 6, 24 projections 553 / 618 /
+    // 940, 759 us; 240 2226 / 2250 / 2578, 3475; 128^3, l_max 8, 60 6.23 / 6.32 / 7.79,
+    // 14.3 ms; 240 16.5 / 16.2 / 16.7, 34.6.  The direct march one per 20: each chunk is a
+    // copy, two events and a launch of less than a wave at few projections.  Us with
+    // eight / one per 10 / 20 / 40 projections: 30 x 28 x 31, l_max 2, 20: 131 / 80 / 80 /
+    // 80, 60: 141 / 126 / 100 / 96, 160: 166 / 168 / 165 / 147; 90 x 80 x 85, l_max 4, FP16,
+    // 35: 775 / 757 / 750 / 750, 60: 933 / 931 / 929 / 947; l_max 2, 60 586 / 575 / 578 /
+    // 597; 110 x 100 x 105, l_max 4, 20: 1274 / 1171 / 1153 / 1156, pageable 160 3922 /
+    // 3948 / 3919 / 3848.
+    const int Q = std::max(1, std::min(8, h->S / (h->fwd_modes ? 120 : 20)));
     if (!h->hc) TT_CUDA(handle_malloc(h, &h->hc, bc), "host-path cudaMalloc");
     if (!g_map && !h->hg) TT_CUDA(handle_malloc(h, &h->hg, bc), "host-path cudaMalloc");
     if (!h->hI) TT_CUDA(handle_malloc(h, &h->hI, bd), "host-path cudaMalloc");
