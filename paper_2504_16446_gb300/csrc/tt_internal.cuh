@@ -268,7 +268,7 @@ struct tt_handle {
     bool xcopy = false;                  // the x-innermost copy exists
     long long pad_vox = 0;               // voxels of one padded copy
     long long cpadx_origin = 0;          // voxel offset of (0,0,0) in the x-innermost copy (from its start)
-    void *arena = nullptr;               // device: holds geo, B64, Bp, cpad, gpad, G, partials, loss_dev, red, mode_mem
+    void *arena = nullptr;               // device: holds geo, B64, Bp, cpad, gpad, G, partials, red, mode_mem
     void *gpad = nullptr;                // device [nvox][KP]
     void *G = nullptr;                   // device [S][nj][nk][KP]
     // Detector modes (tt_modes.cuh; 0: the handle works in channels): G holds
